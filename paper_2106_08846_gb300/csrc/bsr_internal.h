@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "bsr.h"
+#include "dense.h"
 #include "gk.h"
 #include "tc.h"
 #include "xstage.h"
@@ -63,6 +64,7 @@ struct Schedule {
     XsPlan xs;                          // xstage task footprints
     TcPlan tc;                          // tcgen05 task footprints
     GkPlan gk;                          // gathered-K tensor-core kernel, alongside the variant's own
+    DensePlan dense;                    // dense-tile tensor-core kernel, alongside the tcgen05 variant's own
     int n_slots = 0;
     int64_t empty_rows = 0, max_row = 0;
     int sm_count = 148;
@@ -139,6 +141,7 @@ struct LaunchArgs {
     cudaStream_t stream;
     uint64_t wait_ns;      // bound on every device-side wait
     int stall_chunk;       // test hook, -1 in normal use
+    const void *raw;       // the caller's block values
 };
 cudaError_t launch_generic(const LaunchArgs &a);
 cudaError_t launch_xstage(const LaunchArgs &a, int G);

@@ -1,0 +1,155 @@
+// Plan and dispatch of the dense-tile kernel (dense.h): row groups, the
+// chunks each task size's tasks touch, and the task size of a call.
+#include <algorithm>
+#include <cstdlib>
+
+#include "bsr_internal.h"
+#include "schedule.h"
+
+namespace bsr {
+
+int64_t plan_dense(Schedule &sc, int64_t base) {
+    DensePlan &pl = sc.dense;
+    pl.ok = false;
+    const bool shape_ok = kDnGroup % sc.R == 0 || sc.R % kDnGroup == 0;
+    if (sc.variant != V_TC || sc.dt != BSR_BF16 || sc.M % kDnGroup || sc.K % 8 || !shape_ok) return base;
+    const int64_t n_groups = sc.M / kDnGroup, nch = (sc.K + kDnChunk - 1) / kDnChunk;
+    if (n_groups > INT32_MAX / 32 || nch > 1 << 20) return base;
+    // per row group, the chunks that hold a kept block (a byte each)
+    std::vector<uint8_t> used((size_t)(n_groups * nch), 0);
+    for (int64_t i = 0; i < sc.MB; i++) {
+        const int64_t gl = i * sc.R / kDnGroup, gh = (i * sc.R + sc.R - 1) / kDnGroup;
+        for (int32_t p = sc.indptr[(size_t)i]; p < sc.indptr[(size_t)i + 1]; p++) {
+            const int64_t col = (int64_t)sc.indices[(size_t)p] * sc.C;
+            for (int64_t c = col / kDnChunk; c <= (col + sc.C - 1) / kDnChunk; c++)
+                for (int64_t g = gl; g <= gh; g++) used[(size_t)(g * nch + c)] = 1;
+        }
+    }
+    std::vector<int32_t> count((size_t)n_groups, 0);
+    for (int64_t g = 0; g < n_groups; g++)
+        for (int64_t c = 0; c < nch; c++) count[(size_t)g] += used[(size_t)(g * nch + c)];
+    // groups with blocks first, in row order (a task's outputs are then runs of
+    // Y, which the kernel stores in 64-column boxes); by their chunk counts
+    // where full-width tasks then visit a fifth fewer chunks (long groups share
+    // tasks and short ones leave chunks out)
+    pl.group_row.resize((size_t)n_groups);
+    for (int64_t g = 0; g < n_groups; g++) pl.group_row[(size_t)g] = (int32_t)g;
+    std::vector<int32_t> sorted = pl.group_row;
+    auto more = [&](int32_t x, int32_t y) { return count[(size_t)x] > count[(size_t)y]; };
+    auto some = [&](int32_t x, int32_t y) { return (count[(size_t)x] > 0) > (count[(size_t)y] > 0); };
+    std::stable_sort(pl.group_row.begin(), pl.group_row.end(), some);
+    std::stable_sort(sorted.begin(), sorted.end(), more);
+    std::vector<uint8_t> any((size_t)nch);
+    // the chunks of the task of groups [k0, k1) in an order
+    auto unite = [&](const std::vector<int32_t> &order, int64_t k0, int64_t k1) {
+        std::fill(any.begin(), any.end(), 0);
+        for (int64_t k = k0; k < k1; k++) {
+            const uint8_t *u = &used[(size_t)(order[(size_t)k] * nch)];
+            for (int64_t c = 0; c < nch; c++) any[(size_t)c] |= u[c];
+        }
+        return std::count(any.begin(), any.end(), 1);
+    };
+    int64_t in_rows = 0, in_count = 0;
+    for (int64_t k = 0; k < n_groups; k += kDnMaxGroups) {
+        in_rows += unite(pl.group_row, k, std::min(n_groups, k + kDnMaxGroups));
+        in_count += unite(sorted, k, std::min(n_groups, k + kDnMaxGroups));
+    }
+    if (in_count < in_rows - in_rows / 5) pl.group_row = sorted;
+    pl.group_pos.resize((size_t)n_groups);
+    for (int64_t k = 0; k < n_groups; k++) pl.group_pos[(size_t)pl.group_row[(size_t)k]] = (int32_t)k;
+    pl.n_groups = (int)n_groups;
+    pl.n_full = (int)std::count_if(count.begin(), count.end(), [](int32_t c) { return c > 0; });
+    pl.table.clear();
+    for (int g = 1; g <= kDnMaxGroups; g++) {
+        const int64_t tasks = (n_groups + g - 1) / g;
+        const size_t at = pl.table.size();
+        pl.table_at[g] = (int32_t)at;
+        pl.n_tasks[g] = (int)tasks;
+        pl.chunks[g] = 0;
+        pl.max_chunks[g] = 0;
+        pl.table.resize(at + (size_t)tasks + 1);
+        for (int64_t t = 0; t < tasks; t++) {
+            pl.table[at + (size_t)t] = (int32_t)(pl.table.size() - at);
+            const int32_t n = (int32_t)unite(pl.group_row, t * g, std::min(n_groups, t * g + g));
+            for (int64_t c = 0; c < nch; c++)
+                if (any[(size_t)c]) pl.table.push_back((int32_t)c);
+            pl.chunks[g] += n;
+            pl.max_chunks[g] = std::max(pl.max_chunks[g], n);
+        }
+        pl.table[at + (size_t)tasks] = (int32_t)(pl.table.size() - at);
+        if (pl.table.size() > (size_t)INT32_MAX / 4) return base;
+    }
+    pl.w_off = (base + 1023) & ~int64_t(1023);
+    pl.w_bytes = (int64_t)std::max(pl.n_full, 1) * kDnGroup * sc.K * 2;
+    if (pl.w_bytes > (int64_t)1 << 30 && pl.w_bytes > sc.nnzb * sc.R * sc.C * 128) return base;   // 64 times the blocks
+    pl.ok = true;
+    return pl.w_off + pl.w_bytes;
+}
+
+// The busiest SM's cycles at each task size, and the least of them against the
+// block-by-block kernel's. A chunk costs about 250 + 34 g cycles (one CTA) or
+// 300 + 24 g (a pair: half the weight tile per CTA), and no less than 400 to 430
+// (a producer's wait and issue), the start of a pair about
+// 950 more, 64 columns of epilogue about 500: fitted to 1024 x 1024 weights at
+// 16384 tokens (g = 8 33.9 and 32.9 us, g = 16 29.8 and 26.6 us) and 768 x 768
+// ones at 1024 and 3000 tokens (g = 3 to 8). The block-by-block kernel pays
+// about 300 cycles per unit of its own model (250 to 410 where measured):
+// against it the dense tiles won on every 50 to 95% sparse weight tried and on
+// 16x16 blocks of 1024 x 1024 at 99% (24 against 40 us at 16384 tokens), and
+// lost on 16x16 blocks of 4096 x 4096 at 97% (60 against 40 us at 2048
+// tokens: every chunk has a block of some row, and the dense tiles do 33
+// times the kept multiply-adds).
+int choose_dense(const Schedule &sc, int64_t N) {
+    static const int mode = [] {
+        const char *v = getenv("BSR_DENSE");
+        return v && *v ? atoi(v) : -1;   // 0: never, 1: always, unset: by the model
+    }();
+    static const int forced = [] {
+        const char *v = getenv("BSR_DENSE_G");
+        return v ? atoi(v) : 0;
+    }();
+    const DensePlan &pl = sc.dense;
+    if (!pl.ok || N <= 0 || mode == 0) return 0;
+    const int fg = forced & ~kDnPair;
+    if (fg >= 1 && fg <= kDnMaxGroups && !((forced & kDnPair) && fg % 2)) return forced;
+    // (the choice for the last N asked, which is what a steady stream of calls asks again)
+    const uint64_t memo = pl.last.load(std::memory_order_relaxed);
+    if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return (int)(memo & 0xffff);
+    int best = 1;
+    double best_cost = -1.0;
+    for (int pair = 0; pair <= (N > kDnTokens && sc.sm_count >= 2 ? 1 : 0); pair++) {
+        const int64_t tiles = (N + kDnTokens * (1 + pair) - 1) / (kDnTokens * (1 + pair));
+        const int64_t sms = pair ? sc.sm_count / 2 : sc.sm_count;
+        for (int g = 1 + pair; g <= kDnMaxGroups; g += 1 + pair) {
+            const double chunk = pair ? std::max(430.0, 300.0 + 24.0 * g) : std::max(400.0, 250.0 + 34.0 * g);
+            const double epi = 500.0 * ((g + 3) / 4);
+            const int64_t n_work = (pl.n_full + g - 1) / g, units = tiles * n_work;
+            // the busiest SM takes every sms-th unit, the longest of each round;
+            // task by task in the order of their chunks (about: the mean, past 64 rounds)
+            const int64_t rounds = (units + sms - 1) / sms;
+            double mma = 0.0;
+            if (rounds <= 64) {
+                const int32_t *off = &pl.table[(size_t)pl.table_at[g]];
+                for (int64_t r = 0; r < rounds; r++) {
+                    const int64_t t = r * sms / tiles;
+                    mma += (double)(off[t + 1] - off[t]);
+                }
+            } else {
+                mma = (double)(rounds * pl.chunks[g]) / (double)std::max<int64_t>(n_work, 1);
+            }
+            const double stores = (double)((tiles * pl.n_tasks[g] + sms - 1) / sms) * epi;
+            const double cost = std::max(mma * chunk, stores) + epi + (pair ? 950.0 : 0.0);
+            if (best_cost < 0 || cost < best_cost) {
+                best_cost = cost;
+                best = g | (pair ? kDnPair : 0);
+            }
+        }
+    }
+    double by_blocks = 0.0;
+    choose_tc_tasks(sc, N, &by_blocks);
+    if (mode != 1 && by_blocks > 0 && best_cost > 300.0 * by_blocks) best = 0;
+    if (N < (int64_t)1 << 48) pl.last.store((uint64_t)N << 16 | (uint64_t)best, std::memory_order_relaxed);
+    return best;
+}
+
+}  // namespace bsr

@@ -489,7 +489,7 @@ bsr_status_t build_schedule(Schedule &sc) {
         // block values stream per chunk: only balance decides the splitting
         make_items(sc, split_limit(sc), true);
         plan_tc(sc);
-        plan_tcp(sc);
+        if (tcp_enabled()) plan_tcp(sc);
         if (reblock) {
             sc.indptr.swap(uptr);
             sc.indices.swap(uind);
@@ -515,10 +515,11 @@ bsr_status_t build_schedule(Schedule &sc) {
         plan_xstage(sc);
     }
     if (sc.variant == V_XSTAGE && (int64_t)sc.xs_blob.size() > INT32_MAX) sc.variant = V_GENERIC;   // blob offsets are int32
+    // the dense-tile kernel (bf16 tensor-core schedules) and
     // the gathered-K kernel, after the variant's own packed values (the
     // generic kernel's: a copy of the caller's block values)
     if (sc.variant == V_TC)
-        plan_gk(sc, sc.tc_w_total);
+        plan_gk(sc, plan_dense(sc, sc.tc_w_total));
     else if (sc.variant == V_XSTAGE)
         plan_gk(sc, (int64_t)sc.xs_blob.size() * 4);
     else
@@ -538,7 +539,10 @@ bsr_status_t build_schedule(Schedule &sc) {
         upload(&sc.d_group_begin, sc.group_begin) != cudaSuccess ||
         upload(&sc.d_indptr, sc.indptr) != cudaSuccess || upload(&sc.d_indices, sc.indices) != cudaSuccess ||
         upload(&sc.d_xs_perm, sc.xs_perm) != cudaSuccess || upload(&sc.d_xs_vdst, sc.xs_vdst) != cudaSuccess ||
-        upload(&sc.d_vmap, sc.vmap) != cudaSuccess) {
+        upload(&sc.d_vmap, sc.vmap) != cudaSuccess ||
+        upload(&sc.dense.d_group_row, sc.dense.group_row) != cudaSuccess ||
+        upload(&sc.dense.d_group_pos, sc.dense.group_pos) != cudaSuccess ||
+        upload(&sc.dense.d_table, sc.dense.table) != cudaSuccess) {
         cudaGetLastError();
         return BSR_ERR_ALLOC;
     }
@@ -568,12 +572,13 @@ bsr_status_t build_schedule(Schedule &sc) {
 bsr_status_t pack_data(Handle &h) {
     h.data_packed = nullptr;
     const Schedule &sc = *h.sched;
-    if (sc.variant == V_TC && sc.ex_nnzb == 0 && !sc.gk.ok) return BSR_OK;
+    if (sc.variant == V_TC && sc.ex_nnzb == 0 && !sc.gk.ok && !sc.dense.ok) return BSR_OK;
     if (sc.variant != V_XSTAGE && sc.variant != V_TC && !sc.gk.ok) return BSR_OK;
     const size_t raw_bytes = (size_t)sc.nnzb * sc.R * sc.C * dtype_size(sc.dt);
     // xstage: the task blobs (item tables and records from the schedule's
     // template, then this handle's block values)
     size_t bytes = sc.variant == V_TC ? (size_t)sc.tc_w_total : sc.variant == V_XSTAGE ? sc.xs_blob.size() * 4 : raw_bytes;
+    if (sc.dense.ok) bytes = std::max(bytes, (size_t)(sc.dense.w_off + sc.dense.w_bytes));
     if (sc.gk.ok) bytes = std::max(bytes, (size_t)sc.gk.total_bytes);
     if (bytes == 0) return BSR_OK;
     if (cudaMalloc(&h.data_packed, bytes) != cudaSuccess) {
@@ -617,6 +622,7 @@ bsr_status_t pack_data(Handle &h) {
             e = pack_xstage_data(h.data, sc.dt, sc.d_items, sc.d_xs_perm, sc.d_xs_vdst, (int64_t)sc.items.size(),
                                  sc.R, sc.C, (float *)h.data_packed, 0);
     }
+    if (e == cudaSuccess && sc.dense.ok) e = pack_dense_data(sc, h.data, h.data_packed, 0);
     // the gathered-K kernel's operands: zero padding, then the block values
     int64_t gk_lo = -1;
     for (int gi = 0; gi < kGkTaskSizes; gi++)
@@ -636,6 +642,7 @@ bsr_status_t pack_data(Handle &h) {
 
 int launches_per_call(const Schedule &sc, int64_t N) {
     if (choose_gk(sc, N) >= 0) return 1;   // no split rows, no reduce pass
+    if (choose_tcp(sc, N) < 0 && choose_dense(sc, N) > 0) return 1;
     return 1 + (sc.splits.empty() ? 0 : 1);
 }
 
@@ -684,14 +691,15 @@ int choose_tasks(const Schedule &sc, int64_t N) {
 // in per-CTA phase stamps) is counted as kOverheadMma MMA units, a
 // conservative weight: at 32 the model preferred five waves of two-row tasks
 // to three waves of four-row tasks on Zipf rows, measured 9% slower.
-int choose_tc_tasks(const Schedule &sc, int64_t N) {
+int choose_tc_tasks(const Schedule &sc, int64_t N, double *cost_out) {
     static const int forced = [] {
         const char *v = getenv("BSR_TC_G");
         return v ? atoi(v) : 0;
     }();
     auto fits = [&](int G) { return sc.tc.w_off[tc_g_index(G)] >= 0; };   // planned and packed for G
-    for (int gi = 0; gi < kTcTaskSizes; gi++)
-        if (forced == kTcG[gi] && fits(forced)) return forced;
+    if (!cost_out)
+        for (int gi = 0; gi < kTcTaskSizes; gi++)
+            if (forced == kTcG[gi] && fits(forced)) return forced;
     const double kOverheadMma = 64.0;
     const int64_t tiles = (N + kTcTokens - 1) / kTcTokens;
     int best = 1;
@@ -709,8 +717,13 @@ int choose_tc_tasks(const Schedule &sc, int64_t N) {
             best = G;
         }
     }
+    if (cost_out) *cost_out = best_cost;
     return best;
 }
+
+// Products of the dense-tile kernel share grids whatever their shapes (the
+// other classes are below it).
+constexpr int kDenseClass = 1 << 28;
 
 int fusion_class(const Schedule &sc, int64_t N, int *G) {
     if (choose_gk(sc, N) >= 0) {   // a grid of its own
@@ -726,6 +739,7 @@ int fusion_class(const Schedule &sc, int64_t N, int *G) {
             *G = 0;
             return -1;
         }
+        if ((*G = choose_dense(sc, N)) > 0) return kDenseClass + (*G & kDnPair);
         *G = choose_tc_tasks(sc, N);
         return 2 * tc_fusion_key(sc) + 1;
     }
@@ -762,6 +776,11 @@ cudaError_t launch_spmm_batch(const LaunchArgs *as, int n) {
             done[(size_t)j] = 1;
         }
         const int m = (int)grp.size();
+        if (key >= kDenseClass) {   // no split rows, no reduce pass
+            cudaError_t e = launch_dense(grp.data(), gs.data(), m);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
         cudaError_t e = tc ? (m == 1 ? launch_tc(grp[0], gs[0]) : launch_tc_batch(grp.data(), gs.data(), m))
                            : (m == 1 ? launch_xstage(grp[0], gs[0]) : launch_xstage_batch(grp.data(), gs.data(), m));
         if (e != cudaSuccess) return e;
@@ -778,6 +797,8 @@ cudaError_t launch_spmm(const LaunchArgs &a) {
     const int tG = a.sc->variant == V_TC ? choose_tcp(*a.sc, a.N) : -1;
     if (tG >= 0)
         e = launch_tcp(a, tG);
+    else if (const int g = choose_dense(*a.sc, a.N); g > 0)
+        return launch_dense(&a, &g, 1);   // no split rows, no reduce pass
     else if (a.sc->variant == V_TC)
         e = launch_tc(a, choose_tc_tasks(*a.sc, a.N));
     else if (a.sc->variant == V_XSTAGE)

@@ -21,6 +21,10 @@ cudaError_t launch_spmm(const LaunchArgs &a);
 // runs alone. *G receives the task size chosen for N.
 int fusion_class(const Schedule &sc, int64_t N, int *G);
 
+// Task size of the block-by-block tensor-core kernel for N tokens; *cost: the
+// model's cost of it, in MMA units.
+int choose_tc_tasks(const Schedule &sc, int64_t N, double *cost = nullptr);
+
 // Launches n products that share X, N and the stream: products whose kernels
 // share a template (xstage, or tensor-core of one dtype and R) run as one
 // grid, up to 64 at a time; generic-kernel products one after another.

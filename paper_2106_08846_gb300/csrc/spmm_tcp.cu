@@ -678,17 +678,20 @@ cudaError_t launch_t(const LaunchArgs &la, int G) {
 
 }  // namespace
 
-int choose_tcp(const Schedule &sc, int64_t N) {
-    static const int mode = [] {
+bool tcp_enabled() {
+    static const bool on = [] {
         const char *v = getenv("BSR_TCP");
-        return v && *v ? atoi(v) : -1;   // 0: never, 1: whenever a task size fits, unset: by the model
+        return v && atoi(v) == 1;
     }();
+    return on;
+}
+
+int choose_tcp(const Schedule &sc, int64_t N) {
     static const int forced_g = [] {
         const char *v = getenv("BSR_TCP_G");
         return v ? atoi(v) : 0;
     }();
-    if (sc.variant != V_TC || N <= 0 || mode == 0) return -1;
-    if (mode != 1) return -1;
+    if (sc.variant != V_TC || N <= 0 || !tcp_enabled()) return -1;
     // a task size runs when its A slots fit tensor memory and two X and two W
     // buffers fit shared memory
     const uint32_t xbytes = (uint32_t)tcp_stage_chunks(sc.dt) * kBoxBytes;

@@ -99,6 +99,7 @@ inline int tc_chunk_cols(bsr_dtype_t dt) { return dt == BSR_F32 ? 32 : 64; }
 // descriptor offset / 16 in the stage's X buffer), instruction descriptor. Issuer q owns a contiguous
 // range of the task's items, balanced by block count.
 void plan_tcp(struct Schedule &sc);
+bool tcp_enabled();   // BSR_TCP=1: only then are the programs built and the kernel run
 // The tensor map of X [N, K] both tensor-core kernels load from: boxes of
 // 128 bytes x 128 token rows, 128-byte swizzle.
 cudaError_t tc_encode_x(bsr_dtype_t dt, const void *X, int64_t N, int64_t K, CUtensorMap *map);

@@ -1,0 +1,70 @@
+"""The dense-tile tensor-core kernel for bf16 weights: task sizes at the edges
+of its range, ragged tokens, rows and columns, unequal and empty rows, X with
+infinities and NaN, and a fused batch of different shapes."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.mark.parametrize("g", [None, 1, 3, 7, 16, 34, 38, 48])   # 32 + g: pairs of CTAs
+def test_dense_parity_at_task_size(g):
+    env = dict(os.environ, **({} if g is None else {"BSR_DENSE_G": str(g)}))
+    r = subprocess.run([sys.executable, "-m", "tests.dense_check"], cwd=ROOT, env=env, capture_output=True, text=True,
+                       timeout=600)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("g", [4, 48])
+def test_dense_bounded_wait_times_out_and_reports(g):
+    """A chunk that is never loaded: both CTAs of a pair give up, complete each
+    other's loads and return; a later call computes correctly."""
+    code = """
+import os, numpy as np, oracle, synth, torch
+import paper_2106_08846_gb300 as bsr
+from paper_2106_08846_gb300 import bsrlib as b
+from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
+w = synth.make_weight("ds", 7700, 512, 1536, 16, 16, "bf16", 80)
+gpu = build_on_gpu(w.W, 16, 16)
+os.environ.update(BSR_WAIT_LIMIT_NS="2000000", BSR_TEST_STALL_CHUNK="9")
+h = bsr.bsr_create(*gpu, 16, 16, 512, 1536)
+del os.environ["BSR_WAIT_LIMIT_NS"], os.environ["BSR_TEST_STALL_CHUNK"]
+X = synth.activations(7701, 3000, 1536, "bf16")
+h.spmm(to_dev(X), to_dev(w.bias))
+assert h.check_device_status() == b.BSR_ERR_TIMEOUT
+h2 = bsr.bsr_create(*gpu, 16, 16, 512, 1536)
+Y = to_host(h2.spmm(to_dev(X), to_dev(w.bias)))
+assert h2.check_device_status() == b.BSR_OK
+check_product(Y, oracle.bsr_from_dense(w.W, 16, 16), X, w.bias, 512, rows=np.arange(0, 3000, 37))
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, BSR_DENSE_G=str(g)),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-3000:]
+
+
+def test_dense_batch_of_different_shapes_is_bitwise_the_single_calls():
+    import paper_2106_08846_gb300 as bsr
+    N, K = 333, 384
+    ws = [synth.make_weight("db", 7500 + i, M, K, R, C, "bf16", 0,
+                            mask=synth.uniform_block_mask(7500 + i, M // R, K // C, (M // R) * (K // C) // 3))
+          for i, (R, C, M) in enumerate([(16, 16, 512), (32, 1, 256), (1, 32, 80), (64, 64, 1024)])]
+    hs = [bsr.bsr_create(*build_on_gpu(w.W, w.R, w.C), w.R, w.C, w.M, w.K) for w in ws]
+    X = synth.activations(7600, N, K, "bf16")
+    Xd, bs = to_dev(X), [to_dev(w.bias) for w in ws]
+    Ys = [torch.empty((N, w.M), dtype=torch.bfloat16, device="cuda") for w in ws]
+    bsr.bsr_spmm_batch(hs, Xd, bs, Ys, N)
+    for h, w, b, Y in zip(hs, ws, bs, Ys):
+        single = to_host(h.spmm(Xd, b))
+        assert np.array_equal(to_host(Y), single)
+        check_product(single, oracle.bsr_from_dense(w.W, w.R, w.C), X, w.bias, w.M)
+        assert h.check_device_status() == 0
