@@ -125,7 +125,11 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
     int32_t *I_s = reinterpret_cast<int32_t *>(base + a.trec_smem);   // the task record
     float *B_s = reinterpret_cast<float *>(base + a.bias_off);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (a shuffle, so that the warp index and what follows from it is uniform:
+    // whole warps run the producer and the issuers with one elected lane, whose
+    // operands then sit in uniform registers)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const bool elected = ptx::elect_one();
     const int task = (int)(cta % a.n_tasks);
     const int64_t n0 = (int64_t)(cta / a.n_tasks) * TN;
     const int32_t *trec = a.trec + __ldg(a.trec_off + task);
@@ -163,39 +167,41 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
 
     if (warp == 0) {
         // ---------------- producer
-        if (lane == 0) {
-            ptx::prefetch_tensormap(&xmap);
+        {
             const int n_ent = __ldg(trec + 4 + nch);
             const uint32_t rec_bytes = (uint32_t)(items_at + 4 * g_count + pad4(n_ent)) * 4;
-            ptx::mbar_arrive_expect_tx(rbar, rec_bytes);
-            ptx::bulk_load(I_s, trec, rec_bytes, rbar);
+            if (elected) {
+                ptx::prefetch_tensormap(&xmap);
+                ptx::mbar_arrive_expect_tx(rbar, rec_bytes);
+                ptx::bulk_load(I_s, trec, rec_bytes, rbar);
+            }
             ptx::pdl_wait();   // X may be an earlier kernel's output
             const unsigned char *wsrc = static_cast<const unsigned char *>(a.wpk);
             int k = 0;          // ring slots used (chunks with work, in order)
             int stalled = -1;   // test hook: the slot left empty
-            bool ok = ptx::mbar_wait_bounded(rbar, 0, a.wait_ns);   // chunk starts, from shared memory
+            bool ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(rbar, 0, a.wait_ns));   // chunk starts, from shared memory
             const int64_t wfirst = ok ? I_s[0] : 0;                   // the task's first packed block
             for (int c = 0; ok && c < nch; c++) {
                 const int lo = I_s[4 + c], hi = I_s[5 + c];
                 if (lo == hi) continue;   // no block of this task in chunk c
                 const int s = k % NS;
-                if (k >= NS && !ptx::mbar_wait_bounded(&empty[s], ((k / NS) - 1) & 1, a.wait_ns)) {
-                    ok = false;
-                    break;
-                }
-                if (aborted(misc)) { ok = false; break; }
+                const bool got = k < NS || ptx::mbar_wait_bounded(&empty[s], ((k / NS) - 1) & 1, a.wait_ns);
+                ok = __all_sync(0xffffffffu, got && !aborted(misc));
+                if (!ok) break;
                 if (c == a.stall_chunk) {   // never loaded: its consumer times out
                     stalled = k++;
                     continue;
                 }
                 // the X chunk and, beside it, the task's block values for this chunk
                 const uint32_t wbytes = (uint32_t)(hi - lo) * wblock;
-                ptx::mbar_arrive_expect_tx(&full[s], kStageBytes + wbytes);
-                ptx::tma_load_2d(base + s * kStageBytes, &xmap, c * TcCfg<T>::KC, (int32_t)n0, &full[s]);
-                ptx::bulk_load(W_s + s * a.wstage, wsrc + (wfirst + lo) * wblock, wbytes, &full[s]);
+                if (elected) {
+                    ptx::mbar_arrive_expect_tx(&full[s], kStageBytes + wbytes);
+                    ptx::tma_load_2d(base + s * kStageBytes, &xmap, c * TcCfg<T>::KC, (int32_t)n0, &full[s]);
+                    ptx::bulk_load(W_s + s * a.wstage, wsrc + (wfirst + lo) * wblock, wbytes, &full[s]);
+                }
                 k++;
             }
-            if (!ok) {
+            if (!ok && elected) {
                 set_status(a.status, DEV_TIMEOUT);
                 atomicExch(&misc[0], 1);
             }
@@ -204,11 +210,11 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
             ptx::mbar_wait_bounded(rbar, 0, kDrainNs);
         }
     } else if (warp <= NISS) {
-        // ---------------- MMA issuers: lane 0 of warps 1..NISS, each over a
+        // ---------------- MMA issuers: one lane of warps 1..NISS, each over a
         // contiguous range of the task's items (its accumulators), ranges
         // balanced by block count; every issuer walks every chunk and
         // commits the stage, so `empty` and `done` count NISS arrivals
-        if (lane == 0) {
+        {
             const int q = warp - 1;
             int i0 = 0, i1 = 0;
             {
@@ -229,7 +235,7 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
                 if (i1 == 0) i0 = 0;
             }
             const uint32_t ufirst = (uint32_t)i0, ucnt = (uint32_t)(i1 - i0);
-            bool ok = ptx::mbar_wait_bounded(rbar, 0, a.wait_ns) && !aborted(misc);
+            bool ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(rbar, 0, a.wait_ns) && !aborted(misc));
             const int32_t *ent = I_s + items_at + 4 * g_count;
             int k = 0;   // chunks consumed
             for (int c = 0; ok && c < nch; c++) {
@@ -237,10 +243,9 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
                 if (lo == hi) continue;
                 const int s = k % NS;
                 // fp32: wait for the split parts (the split warps waited for the copy)
-                if (!ptx::mbar_wait_bounded(F32 ? &split[s] : &full[s], (k / NS) & 1, a.wait_ns) || aborted(misc)) {
-                    ok = false;
-                    break;
-                }
+                const bool got = ptx::mbar_wait_bounded(F32 ? &split[s] : &full[s], (k / NS) & 1, a.wait_ns);
+                ok = __all_sync(0xffffffffu, got && !aborted(misc));
+                if (!ok) break;
                 tc5::fence_after();
                 const uint32_t stage = ptx::smem_addr(base + s * kStageBytes);
                 const uint32_t w_stage = ptx::smem_addr(W_s + s * a.wstage);
@@ -270,12 +275,13 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
                                 acc[jj] = ((vv[jj] >> 7) & 1u) == 0u;
                             }
 #pragma unroll
-                            for (int jj = 0; jj < 4; jj++) tc5::mma_ss<false>(dv[jj], adv[jj], bdv[jj], idesc, acc[jj]);
+                            for (int jj = 0; jj < 4; jj++)
+                                if (elected) tc5::mma_ss<false>(dv[jj], adv[jj], bdv[jj], idesc, acc[jj]);
                         }
                     }
                 }
                 for (; ucnt > 0 && e < hi; e++) {
-                    const uint32_t v = (uint32_t)ent[e];
+                    const uint32_t v = (uint32_t)__shfl_sync(0xffffffffu, ent[e], 0);   // uniform
                     const uint32_t g = (v >> 2) & 31u, first = (v >> 7) & 1u;
                     const uint64_t ad = a0 + (uint64_t)((v & 3u) * 2u);             // + (v & 3) * 32 bytes
                     const uint64_t bd = b0 + (uint64_t)((uint32_t)(e - lo) * wb16);
@@ -290,8 +296,9 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
                             const uint64_t bs = bd + (uint64_t)(ufirst * R * 2);   // ufirst * R rows of 32 bytes
 #pragma unroll 4
                             for (int sl = 0; sl < C / 16; sl++)
-                                tc5::mma_ss<false>(tmem + ufirst * R, ad + (uint64_t)(sl * 2), bs + (uint64_t)(sl * ns * 2),
-                                         idesc_s, (first == 0u) | (sl > 0));
+                                if (elected)
+                                    tc5::mma_ss<false>(tmem + ufirst * R, ad + (uint64_t)(sl * 2),
+                                                       bs + (uint64_t)(sl * ns * 2), idesc_s, (first == 0u) | (sl > 0));
                             continue;
                         }
                     }
@@ -304,26 +311,29 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
 #pragma unroll 2
                         for (int sl = 0; sl < C / 8; sl++) {
                             const uint64_t ka = (uint64_t)(sl * 2), kb = (uint64_t)(sl * (R * 2));   // 32 and R*32 bytes
-                            tc5::mma_ss<true>(d, ad + ka, bd + kb, idesc, (first == 0u) | (sl > 0));
-                            tc5::mma_ss<true>(d, ad + ka, bdl + kb, idesc, 1u);
-                            tc5::mma_ss<true>(d, adl + ka, bd + kb, idesc, 1u);
+                            if (elected) {
+                                tc5::mma_ss<true>(d, ad + ka, bd + kb, idesc, (first == 0u) | (sl > 0));
+                                tc5::mma_ss<true>(d, ad + ka, bdl + kb, idesc, 1u);
+                                tc5::mma_ss<true>(d, adl + ka, bd + kb, idesc, 1u);
+                            }
                         }
                     } else {
                         constexpr uint32_t idesc = tc5::idesc(false, TN, R);
 #pragma unroll 4
                         for (int sl = 0; sl < C / 16; sl++)
-                            tc5::mma_ss<false>(d, ad + (uint64_t)(sl * 2), bd + (uint64_t)(sl * (R * 2)), idesc,
-                                     (first == 0u) | (sl > 0));
+                            if (elected)
+                                tc5::mma_ss<false>(d, ad + (uint64_t)(sl * 2), bd + (uint64_t)(sl * (R * 2)), idesc,
+                                                   (first == 0u) | (sl > 0));
                     }
                 }
-                tc5::commit(&empty[s]);   // the stage is free once every issuer's MMAs completed
+                if (elected) tc5::commit(&empty[s]);   // the stage is free once every issuer's MMAs completed
                 k++;
             }
-            if (!ok) {
+            if (!ok && elected) {
                 set_status(a.status, DEV_TIMEOUT);
                 atomicExch(&misc[0], 1);
             }
-            tc5::commit(done);   // every MMA this issuer issued completes before its `done` arrival
+            if (elected) tc5::commit(done);   // every MMA this issuer issued completes before its `done` arrival
         }
     } else {
         // ---------------- the last four warps: fp32 split during the main
