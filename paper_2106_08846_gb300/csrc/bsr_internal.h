@@ -122,11 +122,10 @@ inline size_t dtype_size(bsr_dtype_t dt) { return dt == BSR_F32 ? 4 : 2; }
 
 // ---- builder (builder.cu)
 cudaError_t launch_builder_count(const void *W, bsr_dtype_t dt, int64_t M, int64_t K, int R, int C,
-                                 float thr, uint8_t *flags, int32_t *counts, int32_t *indptr,
-                                 cudaStream_t s);
-cudaError_t launch_builder_compact(const void *W, bsr_dtype_t dt, int64_t M, int64_t K, int R, int C,
-                                   const uint8_t *flags, const int32_t *indptr, int32_t *indices,
-                                   void *data, cudaStream_t s);
+                                 float thr, int32_t *counts, int32_t *indptr, int32_t *nnzb, cudaStream_t s);
+cudaError_t launch_builder_compact(const void *W, bsr_dtype_t dt, int64_t M, int64_t K, int R, int C, float thr,
+                                   const int32_t *first, int32_t *indices, void *data, cudaStream_t s);
+int64_t builder_segments(int64_t M, int64_t K, int R, int C, bsr_dtype_t dt);   // entries of `counts` / `first`
 
 // ---- SpMM kernels (spmm_*.cu)
 struct LaunchArgs {

@@ -1,0 +1,37 @@
+"""bsr_from_dense at the edges of its segments: blocks of the largest size in
+either direction, rows that are not 16-byte aligned, a misaligned W, one and
+many segments per block row, a partly filled last one; bit for bit against the
+oracle, NaN and threshold rule included."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from tests.gpu_util import assert_structure_equal, dtype_of, to_dev
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [  # R, C, M, K
+    (4096, 1, 8192, 6), (1, 4096, 3, 3 * 4096), (64, 64, 128, 64 * 5), (1, 1, 7, 2049), (1, 1, 3, 5000),
+    (2, 3, 10, 3 * 701), (8, 1, 16, 1026), (32, 1, 64, 4100), (5, 7, 15, 7 * 333), (16, 16, 32, 16 * 70),
+]
+
+
+@pytest.mark.parametrize("R,C,M,K", SHAPES)
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_builder_segments_match_the_oracle(R, C, M, K, dtype, offset):
+    import paper_2106_08846_gb300 as bsr
+    MB, KB = M // R, K // C
+    w = synth.make_weight("be", 8000 + R + C, M, K, R, C, dtype, 0,
+                          mask=synth.uniform_block_mask(8000 + R + C, MB, KB, max(1, (MB * KB) // 3)))
+    W = w.W.copy()
+    W.flat[0] = np.float32("nan") if dtype == "f32" else 0x7fc0
+    Wd = to_dev(W).flatten()
+    buf = torch.empty(M * K + 8, dtype=Wd.dtype, device="cuda")
+    at = buf[offset:offset + M * K].view(M, K)   # offset 1: no 16-byte loads
+    at.copy_(Wd.view(M, K))
+    for thr in (0.0, 0.03):
+        assert_structure_equal(bsr.bsr_from_dense(at, R, C, thr), oracle.bsr_from_dense(W, R, C, thr))
+    assert dtype_of(W) == dtype
