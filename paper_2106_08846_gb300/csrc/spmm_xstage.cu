@@ -158,23 +158,36 @@ struct Tile {
     }
 };
 
-// one output per lane: plain fp32 FMA, no operand pairs to form (measured
-// faster than the packed form for this load-bound tile)
-template <>
-struct Tile<1> {
-    float a[8];
+// One output per lane (load-bound: no operand pairs to form) and four (4 x 4
+// blocks of 768 x 768 at 80%, 1024 tokens: 17.6 us against 19.8 us packed):
+// plain fp32 multiply-adds. Packed ones read three 64-bit operands each, which
+// the register file sustains at 58% of the FP32 rate; eight outputs still take
+// them, since there the issue slots that plain ones need cost more (32x1 at
+// 16384 tokens 133 against 140 us).
+template <int TR>
+struct PlainTile {
+    float a[8][TR];
     __device__ __forceinline__ void zero() {
 #pragma unroll
-        for (int k = 0; k < 8; k++) a[k] = 0.f;
-    }
-    __device__ __forceinline__ void fma(const float (&x)[8], const f2_t (&wd)[1]) {
-        float w, w2;
-        unpack2(wd[0], w, w2);
+        for (int i = 0; i < 8; i++)
 #pragma unroll
-        for (int i = 0; i < 8; i++) a[i] = fmaf(x[i], w, a[i]);
+            for (int j = 0; j < TR; j++) a[i][j] = 0.f;
     }
-    __device__ __forceinline__ float get(int i, int) const { return a[i]; }
+    __device__ __forceinline__ void fma(const float (&x)[8], const f2_t (&wd)[TR]) {
+#pragma unroll
+        for (int j = 0; j < TR; j++) {
+            float w, w2;
+            unpack2(wd[j], w, w2);
+#pragma unroll
+            for (int i = 0; i < 8; i++) a[i][j] = fmaf(x[i], w, a[i][j]);
+        }
+    }
+    __device__ __forceinline__ float get(int i, int j) const { return a[i][j]; }
 };
+template <>
+struct Tile<1> : PlainTile<1> {};
+template <>
+struct Tile<4> : PlainTile<4> {};
 
 // The TR weights of one block column for this lane, each as a (w, w) pair.
 // With WD == 2 the packed values already hold every weight twice, so the
