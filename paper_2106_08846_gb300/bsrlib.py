@@ -98,13 +98,21 @@ def _check(status: int, where: str) -> None:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+# The current stream's handle and device without a Stream object (which takes
+# 2.9 us to make, as long as the whole C call); its long form where torch has none.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_cur_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        if _raw_stream is not None and _cur_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_cur_device())
+        return torch.cuda.current_stream().cuda_stream
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def dtype_code(dtype: torch.dtype) -> int:
@@ -204,34 +212,38 @@ def bsr_reserve(h: Handle, N_max: int) -> None:
     _check(load().bsr_reserve(h.ptr, N_max), "bsr_reserve")
 
 
-def bsr_spmm(h: Handle, X: torch.Tensor, bias: Optional[torch.Tensor], Y: torch.Tensor,
-             N: Optional[int] = None, stream=None) -> None:
-    """Y[N, M] = X[N, K] W^T + bias; X and Y both on the device or both in host memory."""
-    if X.dtype != h.dtype or Y.dtype != h.dtype:
+def _check_product(h: Handle, X: torch.Tensor, bias: Optional[torch.Tensor], Y: torch.Tensor, N: Optional[int]) -> int:
+    """The checks of one product's tensors; returns N."""
+    dt = h.dtype
+    if X.dtype is not dt or Y.dtype is not dt:
         raise TypeError("X and Y must have the handle's dtype")
     if not X.is_contiguous() or not Y.is_contiguous():
         raise ValueError("X and Y must be contiguous")
-    if bias is not None and (bias.dtype != torch.float32 or not bias.is_contiguous()):
+    if bias is not None and (bias.dtype is not torch.float32 or not bias.is_contiguous()):
         raise TypeError("bias must be a contiguous float32 tensor")
-    N = X.shape[0] if N is None else N
-    if X.shape[-1] != h.K or Y.shape[-1] != h.M or X.shape[0] < N or Y.shape[0] < N:
+    xs, ys = X.shape, Y.shape
+    if N is None:
+        N = xs[0]
+    if xs[-1] != h.K or ys[-1] != h.M or xs[0] < N or ys[0] < N:
         raise ValueError("X must be [N, K] and Y [N, M]")
-    _check(load().bsr_spmm(h.ptr, _ptr(X), _ptr(bias), _ptr(Y), N, _stream(stream)), "bsr_spmm")
+    return N
+
+
+def bsr_spmm(h: Handle, X: torch.Tensor, bias: Optional[torch.Tensor], Y: torch.Tensor,
+             N: Optional[int] = None, stream=None) -> None:
+    """Y[N, M] = X[N, K] W^T + bias; X and Y both on the device or both in host memory."""
+    N = _check_product(h, X, bias, Y, N)
+    st = (_lib or load()).bsr_spmm(h.ptr, X.data_ptr(), None if bias is None else bias.data_ptr(), Y.data_ptr(), N,
+                                   _stream(stream))
+    if st:
+        _check(st, "bsr_spmm")
 
 
 def bsr_spmm_noalloc(h: Handle, X: torch.Tensor, bias: Optional[torch.Tensor], Y: torch.Tensor,
                      N: Optional[int] = None, stream=None) -> None:
     """bsr_spmm without any device allocation (device X and Y only): split-row
     partials use the library's fixed scratch array (see include/bsr.h)."""
-    if X.dtype != h.dtype or Y.dtype != h.dtype:
-        raise TypeError("X and Y must have the handle's dtype")
-    if not X.is_contiguous() or not Y.is_contiguous():
-        raise ValueError("X and Y must be contiguous")
-    if bias is not None and (bias.dtype != torch.float32 or not bias.is_contiguous()):
-        raise TypeError("bias must be a contiguous float32 tensor")
-    N = X.shape[0] if N is None else N
-    if X.shape[-1] != h.K or Y.shape[-1] != h.M or X.shape[0] < N or Y.shape[0] < N:
-        raise ValueError("X must be [N, K] and Y [N, M]")
+    N = _check_product(h, X, bias, Y, N)
     _check(load().bsr_spmm_noalloc(h.ptr, _ptr(X), _ptr(bias), _ptr(Y), N, _stream(stream)), "bsr_spmm_noalloc")
 
 
