@@ -12,6 +12,14 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The first address at or after p (dynamic shared memory) on a 1024-byte
+// boundary, by pointer arithmetic: through an integer the compiler would lose
+// the address space and turn every access into a generic load or store (64-bit
+// addresses, a longer latency).
+__device__ __forceinline__ unsigned char *align_smem(unsigned char *p) {
+    return p + ((1024u - (smem_addr(p) & 1023u)) & 1023u);
+}
+
 // Programmatic dependent launch (see launch.cuh): let the next kernel of
 // the stream be scheduled; wait until the kernels this one depends on have
 // completed and their writes are visible. Both are no-ops for a kernel

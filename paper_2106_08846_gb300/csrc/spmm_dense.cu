@@ -177,8 +177,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatch<MAXB> b) {
     ptx::pdl_launch_dependents();
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *base =
-        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char *base = ptx::align_smem(smem_raw);
     const int ns = b.ns;
     const uint32_t stage_bytes = b.stage_bytes;
     float *bias_s = reinterpret_cast<float *>(base + (size_t)ns * stage_bytes);

@@ -238,8 +238,7 @@ k_gk(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ GkArgs a)
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int KS = F32 ? 8 : 16;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *base =
-        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char *base = ptx::align_smem(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(base + a.bar_off);
     uint64_t *empty = full + NS_MAX;   // the gather warps + every issuer's MMA commit
     uint64_t *afull = empty + NS_MAX;  // A buffer written (one gather group)

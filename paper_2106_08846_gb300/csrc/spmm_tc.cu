@@ -112,8 +112,7 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
     constexpr int NS = TcCfg<T>::NS;
     constexpr int NISS = TcCfg<T>::NISS;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *base =
-        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char *base = ptx::align_smem(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(base + a.bar_off);
     uint64_t *empty = full + NS;
     uint64_t *split = empty + NS;    // fp32: the stage's high/low parts are ready

@@ -140,8 +140,7 @@ k_tcp(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcpArgs 
     constexpr int SC = Cfg::SC;
     constexpr int NLW = Cfg::NLW;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *base =
-        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char *base = ptx::align_smem(smem_raw);
     uint64_t *xfull = reinterpret_cast<uint64_t *>(base + a.bar_off);
     uint64_t *xempty = xfull + NXMAX;   // the loaders copied the X buffer to tensor memory
     uint64_t *wfull = xempty + NXMAX;

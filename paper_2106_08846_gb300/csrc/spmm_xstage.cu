@@ -292,7 +292,7 @@ __device__ __forceinline__ void item_chunk(Tile<TR> &acc, const unsigned char *s
             const int lb = piece + S * jj;
             const int kk = idx[lb] * C - kbase;
             const float *wb = wbase + lb * C * R * WD;
-            if (TR < 8 && (cw & 3) == 0) {   // four columns per load, where registers allow
+            if ((TR < 8 || NRG == 1) && (cw & 3) == 0) {   // four columns per load, where registers allow
                 for (int c4 = cc0; c4 < cc0 + cw; c4 += 4) {
                     const unsigned char *xp = st + (St::off0(kk + c4) ^ tgx);
                     float4 xv[8];
@@ -310,7 +310,7 @@ __device__ __forceinline__ void item_chunk(Tile<TR> &acc, const unsigned char *s
                     }
                 }
             } else {
-                for (int cc = cc0; cc < cc0 + cw; cc++) {
+                auto one = [&](int cc) {
                     const unsigned char *xp = st + (St::off0(kk + cc) ^ tgx);
                     float x[8];
                     f2_t wd[TR];
@@ -318,6 +318,12 @@ __device__ __forceinline__ void item_chunk(Tile<TR> &acc, const unsigned char *s
                     for (int i = 0; i < 8; i++) x[i] = ld_x(xp + i * 1024, T());
                     load_wd<TR>(wb + cc * R * WD, wd);
                     acc.fma(x, wd);
+                };
+                if constexpr (NRG == 2) {
+#pragma unroll 4
+                    for (int cc = cc0; cc < cc0 + cw; cc++) one(cc);
+                } else {
+                    for (int cc = cc0; cc < cc0 + cw; cc++) one(cc);
                 }
             }
         }
@@ -619,7 +625,7 @@ __device__ __forceinline__ void xstage_cta(const CUtensorMap &xmap, const XsArgs
     using St = Stage<T>;
     extern __shared__ unsigned char smem_raw[];
     Shared sh;
-    sh.base = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    sh.base = ptx::align_smem(smem_raw);
     sh.full = reinterpret_cast<uint64_t *>(sh.base + a.bar_off);
     sh.empty = sh.full + NS;
     sh.wbar = sh.empty + NS;
