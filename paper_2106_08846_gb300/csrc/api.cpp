@@ -216,6 +216,9 @@ Schedule::~Schedule() {
         cudaFree(tc.d_stab[gi]);
     }
     cudaFree(d_indices);
+    cudaFree(xc.d_table);
+    cudaFree(xc.d_ints);
+    cudaFree(xc.d_src);
     cudaFree(dense.d_group_row);
     cudaFree(dense.d_group_pos);
     cudaFree(dense.d_table);

@@ -13,6 +13,7 @@
 #include "bsr.h"
 #include "dense.h"
 #include "gk.h"
+#include "xcol.h"
 #include "tc.h"
 #include "xstage.h"
 
@@ -64,6 +65,7 @@ struct Schedule {
     XsPlan xs;                          // xstage task footprints
     TcPlan tc;                          // tcgen05 task footprints
     GkPlan gk;                          // gathered-K tensor-core kernel, alongside the variant's own
+    XcPlan xc;                          // column-list SIMT kernel, alongside the xstage or tcgen05 variant
     DensePlan dense;                    // dense-tile tensor-core kernel, alongside the tcgen05 variant's own
     int n_slots = 0;
     int64_t empty_rows = 0, max_row = 0;

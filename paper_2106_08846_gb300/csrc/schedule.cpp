@@ -515,13 +515,14 @@ bsr_status_t build_schedule(Schedule &sc) {
         plan_xstage(sc);
     }
     if (sc.variant == V_XSTAGE && (int64_t)sc.xs_blob.size() > INT32_MAX) sc.variant = V_GENERIC;   // blob offsets are int32
-    // the dense-tile kernel (bf16 tensor-core schedules) and
+    // the dense-tile kernel (bf16 tensor-core schedules), the column-list kernel
+    // (fp32 32x1 blocks) and
     // the gathered-K kernel, after the variant's own packed values (the
     // generic kernel's: a copy of the caller's block values)
     if (sc.variant == V_TC)
         plan_gk(sc, plan_dense(sc, sc.tc_w_total));
     else if (sc.variant == V_XSTAGE)
-        plan_gk(sc, (int64_t)sc.xs_blob.size() * 4);
+        plan_gk(sc, plan_xcol(sc, (int64_t)sc.xs_blob.size() * 4));
     else
         plan_gk(sc, sc.nnzb * sc.R * sc.C * (int64_t)dtype_size(sc.dt));
     if (sc.variant == V_GENERIC) {
@@ -542,7 +543,9 @@ bsr_status_t build_schedule(Schedule &sc) {
         upload(&sc.d_vmap, sc.vmap) != cudaSuccess ||
         upload(&sc.dense.d_group_row, sc.dense.group_row) != cudaSuccess ||
         upload(&sc.dense.d_group_pos, sc.dense.group_pos) != cudaSuccess ||
-        upload(&sc.dense.d_table, sc.dense.table) != cudaSuccess) {
+        upload(&sc.dense.d_table, sc.dense.table) != cudaSuccess ||
+        upload(&sc.xc.d_table, sc.xc.table) != cudaSuccess || upload(&sc.xc.d_ints, sc.xc.ints) != cudaSuccess ||
+        upload(&sc.xc.d_src, sc.xc.src) != cudaSuccess) {
         cudaGetLastError();
         return BSR_ERR_ALLOC;
     }
@@ -579,6 +582,7 @@ bsr_status_t pack_data(Handle &h) {
     // template, then this handle's block values)
     size_t bytes = sc.variant == V_TC ? (size_t)sc.tc_w_total : sc.variant == V_XSTAGE ? sc.xs_blob.size() * 4 : raw_bytes;
     if (sc.dense.ok) bytes = std::max(bytes, (size_t)(sc.dense.w_off + sc.dense.w_bytes));
+    if (sc.xc.ok) bytes = std::max(bytes, (size_t)(sc.xc.off + sc.xc.bytes));
     if (sc.gk.ok) bytes = std::max(bytes, (size_t)sc.gk.total_bytes);
     if (bytes == 0) return BSR_OK;
     if (cudaMalloc(&h.data_packed, bytes) != cudaSuccess) {
@@ -622,6 +626,7 @@ bsr_status_t pack_data(Handle &h) {
             e = pack_xstage_data(h.data, sc.dt, sc.d_items, sc.d_xs_perm, sc.d_xs_vdst, (int64_t)sc.items.size(),
                                  sc.R, sc.C, (float *)h.data_packed, 0);
     }
+    if (e == cudaSuccess && sc.xc.ok) e = pack_xcol_data(sc, h.data, h.data_packed, 0);
     if (e == cudaSuccess && sc.dense.ok) e = pack_dense_data(sc, h.data, h.data_packed, 0);
     // the gathered-K kernel's operands: zero padding, then the block values
     int64_t gk_lo = -1;
@@ -652,14 +657,15 @@ int launches_per_call(const Schedule &sc, int64_t N) {
 // token (blocks x R x C); a CTA's fixed cost (pipeline fill, streaming the
 // X tile, staging, epilogue) is worth about kFixed of them, which is about
 // two 32x1 rows of a 768-wide weight at 80% block sparsity.
-int choose_tasks(const Schedule &sc, int64_t N) {
+int choose_tasks(const Schedule &sc, int64_t N, double *cost_out) {
     static const int forced = [] {
         const char *v = getenv("BSR_XS_G");
         return v ? atoi(v) : 0;
     }();
     auto fits = [&](int G) { return sc.xs_blob_off[g_index(G)] >= 0; };   // blobs exist for G
-    for (int gi = 0; gi < kXsTaskSizes; gi++)
-        if (forced == kXsG[gi] && fits(forced)) return forced;
+    if (!cost_out)
+        for (int gi = 0; gi < kXsTaskSizes; gi++)
+            if (forced == kXsG[gi] && fits(forced)) return forced;
     const double kFixed = 10000.0;
     const int64_t tiles = (N + kXsTokens - 1) / kXsTokens;
     const int64_t items = (int64_t)sc.items.size();
@@ -680,6 +686,7 @@ int choose_tasks(const Schedule &sc, int64_t N) {
             best = G;
         }
     }
+    if (cost_out) *cost_out = best_cost;
     return best;
 }
 
@@ -724,12 +731,14 @@ int choose_tc_tasks(const Schedule &sc, int64_t N, double *cost_out) {
 // Products of the dense-tile kernel share grids whatever their shapes (the
 // other classes are below it).
 constexpr int kDenseClass = 1 << 28;
+constexpr int kXcolClass = 1 << 27;
 
 int fusion_class(const Schedule &sc, int64_t N, int *G) {
     if (choose_gk(sc, N) >= 0) {   // a grid of its own
         *G = 0;
         return -1;
     }
+    if (choose_tcp(sc, N) < 0 && (*G = choose_xcol(sc, N)) >= 0) return kXcolClass + *G;
     if (sc.variant == V_XSTAGE) {
         *G = choose_tasks(sc, N);
         return 2 * xstage_fusion_key(sc, *G);
@@ -781,7 +790,7 @@ cudaError_t launch_spmm_batch(const LaunchArgs *as, int n) {
             if (e != cudaSuccess) return e;
             continue;
         }
-        cudaError_t e = tc ? (m == 1 ? launch_tc(grp[0], gs[0]) : launch_tc_batch(grp.data(), gs.data(), m))
+        cudaError_t e = key >= kXcolClass ? launch_xcol(grp.data(), gs.data(), m) : tc ? (m == 1 ? launch_tc(grp[0], gs[0]) : launch_tc_batch(grp.data(), gs.data(), m))
                            : (m == 1 ? launch_xstage(grp[0], gs[0]) : launch_xstage_batch(grp.data(), gs.data(), m));
         if (e != cudaSuccess) return e;
         for (const LaunchArgs &a : grp)
@@ -795,8 +804,11 @@ cudaError_t launch_spmm(const LaunchArgs &a) {
     if (gG >= 0) return launch_gk(a, gG);   // every block row is an item: nothing to reduce
     cudaError_t e;
     const int tG = a.sc->variant == V_TC ? choose_tcp(*a.sc, a.N) : -1;
+    const int xG = tG < 0 ? choose_xcol(*a.sc, a.N) : -1;
     if (tG >= 0)
         e = launch_tcp(a, tG);
+    else if (xG >= 0)
+        e = launch_xcol(&a, &xG, 1);
     else if (const int g = choose_dense(*a.sc, a.N); g > 0)
         return launch_dense(&a, &g, 1);   // no split rows, no reduce pass
     else if (a.sc->variant == V_TC)

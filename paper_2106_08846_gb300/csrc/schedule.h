@@ -21,6 +21,10 @@ cudaError_t launch_spmm(const LaunchArgs &a);
 // runs alone. *G receives the task size chosen for N.
 int fusion_class(const Schedule &sc, int64_t N, int *G);
 
+// Task size of the per-task SIMT kernel for N tokens; *cost: the model's cost of
+// it, in multiply-adds per token.
+int choose_tasks(const Schedule &sc, int64_t N, double *cost = nullptr);
+
 // Task size of the block-by-block tensor-core kernel for N tokens; *cost: the
 // model's cost of it, in MMA units.
 int choose_tc_tasks(const Schedule &sc, int64_t N, double *cost = nullptr);

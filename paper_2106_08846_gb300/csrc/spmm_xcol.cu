@@ -1,0 +1,457 @@
+// SIMT kernel over column lists for fp32 one-column blocks of 32 rows ("xcol").
+//
+// A warp multiplies an item (a block row) with 8 TT tokens: lane = tg + 8 rg,
+// tg picks tokens tg, tg + 8, ..., rg a group of 8 output rows. Per column a
+// lane loads TT activations and 8 weights from shared memory and does 8 TT
+// multiply-adds, packed in pairs of tokens.
+//
+// What bounds it: the FP32 pipe as the register file feeds it. A packed
+// multiply-add reads three 64-bit operands; with the weight pair kept over
+// consecutive instructions (tokens inside, outputs outside) it takes 2.5 cycles
+// instead of 2, with the activations kept 3.4; plain ones run at 87% of the
+// rate but leave no issue slots for the loads. Shared memory delivers 32 words
+// a cycle whatever is broadcast: TT + 8 words for 8 TT multiply-adds, equal to
+// the pipe's need at TT = 8 and 79% of it at TT = 14, the largest tile that
+// three warps a scheduler have registers for.
+//
+// Persistent: one CTA per SM walks units (task of G items, token tile). The
+// producer warp streams X chunks (two TMA boxes of 32 columns) and, beside
+// each, the items' packed columns of that chunk through a ring; every consumer
+// warp waits for chunks, works through its columns and frees them, and goes on
+// to the next unit when its own tile is stored: no barrier over all warps.
+// Items of a task are neighbours in length, so warps stay within the ring of
+// one another.
+//
+// Measured (us, back to back, the per-task kernel in brackets): see
+// choose_xcol.
+//
+// Every wait is bounded by the global timer; a timeout sets the device status
+// word, stops the CTA's roles, lets the issued copies land and returns.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <atomic>
+#include <mutex>
+
+#include "bsr_internal.h"
+#include "launch.cuh"
+#include "ptx.cuh"
+
+namespace bsr {
+
+namespace {
+
+constexpr int NW = kXcWarps;
+constexpr int kThreads = 32 * (NW + 1);
+constexpr int kStagesMax = kXcStagesMax;
+constexpr uint64_t kDrainNs = 200000000ull;
+
+struct XcArgs {
+    const int32_t *table;        // per item and chunk: the packed chunk's start / 16, in order (and the end)
+    const unsigned char *packed;
+    const Item *items;
+    const float *bias;
+    float *Y, *ws;
+    int *status;
+    int64_t M;
+    uint64_t wait_ns;
+    int n_items, n_tasks;
+    unsigned tiles;
+    int stall_chunk;
+};
+
+template <int MAXB>
+struct XcBatch {
+    int n, ns;
+    uint32_t stage_bytes;   // a stage: two X boxes, then the items' packed chunks, item_bytes apart
+    uint32_t item_bytes;
+    int nch;
+    int64_t N;
+    unsigned start[MAXB + 1];
+    XcArgs args[MAXB];
+};
+
+typedef unsigned long long f2_t;   // two packed fp32
+__device__ __forceinline__ f2_t pack2(float lo, float hi) {
+    f2_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f2_t v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+// (volatile: in the order written)
+__device__ __forceinline__ f2_t ffma2(f2_t a, f2_t b, f2_t c) {
+    f2_t d;
+    asm volatile("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
+__device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
+__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, uint64_t limit_ns, const int *flag) {
+    if (ptx::mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = ptx::globaltimer();
+    while (true) {
+        if (ptx::mbar_try_wait(bar, parity)) return true;
+        if (aborted(flag) || ptx::globaltimer() - t0 > limit_ns) return false;
+    }
+}
+
+struct Unit {
+    int i0, n;    // first item, items
+    int64_t n0;   // first token
+};
+template <int TT>
+__device__ __forceinline__ Unit unit_at(const XcArgs &a, unsigned v) {
+    Unit u;   // the tasks of a token tile side by side: their reads of X meet in L2
+    const unsigned tile = v / (unsigned)a.n_tasks;
+    const int task = (int)(v - tile * (unsigned)a.n_tasks);
+    u.i0 = xcol_first(task, a.n_tasks, a.n_items);
+    u.n = xcol_first(task + 1, a.n_tasks, a.n_items) - u.i0;
+    u.n0 = (int64_t)tile * (8 * TT);
+    return u;
+}
+
+// One column: TT activations at p and 8 weights at w (the lane's first four
+// outputs, and 16 further its last four).
+template <int TT>
+__device__ __forceinline__ void column(f2_t (&acc)[TT / 2][8], const unsigned char *p, const float *w) {
+    f2_t x[TT / 2];
+#pragma unroll
+    for (int i = 0; i < TT / 2; i++)
+        x[i] = pack2(*reinterpret_cast<const float *>(p + 2 * i * 1024),
+                     *reinterpret_cast<const float *>(p + (2 * i + 1) * 1024));
+    const float4 a = *reinterpret_cast<const float4 *>(w), b = *reinterpret_cast<const float4 *>(w + 16);
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        const f2_t wj = pack2(v[j], v[j]);
+#pragma unroll
+        for (int i = 0; i < TT / 2; i++) acc[i][j] = ffma2(x[i], wj, acc[i][j]);
+    }
+}
+
+template <int MAXB, int TT>
+__global__ void __launch_bounds__(kThreads, 1)
+k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch<MAXB> b) {
+    ptx::pdl_launch_dependents();
+    constexpr uint32_t kX = 2 * kXcBox;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *base = ptx::align_smem(smem_raw);
+    __shared__ uint64_t full[kStagesMax], empty[kStagesMax];
+    __shared__ int stop;
+    const int ns = b.ns;
+    const uint32_t stage_bytes = b.stage_bytes;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < ns; s++) {
+            ptx::mbar_init(&full[s], 1);
+            ptx::mbar_init(&empty[s], NW);
+        }
+        stop = 0;
+        ptx::fence_barrier_init();
+    }
+    __syncthreads();
+    const unsigned units = b.start[b.n];
+    const bool elected = ptx::elect_one();
+    auto halt = [&](int *status) {
+        if (elected) {
+            if (!aborted(&stop)) set_status(status, DEV_TIMEOUT);
+            atomicExch(&stop, 1);
+        }
+    };
+    const int nch = b.nch;
+    unsigned u = blockIdx.x;
+    int h = 0, s = 0;
+
+    if (warp == NW) {
+        // ---------------- producer: lane g copies item g's columns
+        uint32_t phase = 1;   // the parity of `empty` that a first use of a stage passes at once
+        uint32_t stalled = 0; // test hook: stages whose load was left out
+        int issued = 0;
+        bool ok = true, waited = false;
+        if (elected) ptx::prefetch_tensormap(&xmap);
+        for (; ok && u < units; u += gridDim.x) {
+            while (u >= b.start[h + 1]) h++;
+            const XcArgs &a = b.args[h];
+            const Unit un = unit_at<TT>(a, u - b.start[h]);
+            const int32_t *tab = a.table + (int64_t)(un.i0 + min(lane, un.n - 1)) * nch;
+            int at = __ldg(tab);
+            auto load_w = [&](int c, int st, int from, int to) {
+                const uint32_t bytes = lane < un.n ? (uint32_t)(to - from) * 16 : 0;
+                const uint32_t all = __reduce_add_sync(0xffffffffu, bytes);
+                if (elected) ptx::mbar_arrive_expect_tx(&full[st], 2 * TT * 1024 + all);
+                __syncwarp();
+                if (bytes)
+                    ptx::bulk_load(base + (size_t)st * stage_bytes + kX + lane * b.item_bytes,
+                                   a.packed + (int64_t)from * 16, bytes, &full[st]);
+                __syncwarp();
+            };
+            // the first columns do not depend on earlier kernels
+            const int ahead = waited ? 0 : min(ns, nch);
+            if (!waited) {
+                int from = at;
+                for (int c = 0; c < ahead; c++) {
+                    const int to = __ldg(tab + c + 1);
+                    if (c != a.stall_chunk) load_w(c, c, from, to);
+                    from = to;
+                }
+                ptx::pdl_wait();   // X may be an earlier kernel's output
+                waited = true;
+            }
+            for (int c = 0; c < nch; c++) {
+                const int next = __ldg(tab + c + 1);
+                // (the stages loaded ahead are free, and their X tiles always
+                // follow: a barrier phase is never left half loaded)
+                if (c >= ahead) {
+                    const bool got = wait_or_abort(&empty[s], phase, a.wait_ns, &stop);
+                    if (!__all_sync(0xffffffffu, got && !aborted(&stop))) {
+                        halt(a.status);
+                        ok = false;
+                        break;
+                    }
+                }
+                if (c == a.stall_chunk) {   // never loaded: its consumers time out
+                    stalled |= 1u << s;
+                } else {
+                    if (c >= ahead) load_w(c, s, at, next);
+                    if (elected) {
+                        unsigned char *st = base + (size_t)s * stage_bytes;
+                        ptx::tma_load_2d(st, &xmap, c * kXcChunk, (int32_t)un.n0, &full[s]);
+                        ptx::tma_load_2d(st + kXcBox, &xmap, c * kXcChunk + 32, (int32_t)un.n0, &full[s]);
+                    }
+                }
+                issued++;
+                if (++s == ns) {
+                    s = 0;
+                    phase ^= 1;
+                }
+                at = next;
+            }
+        }
+        // no copy may outlive the CTA (a stage that was consumed has landed long ago)
+        for (int k = max(0, issued - ns); k < issued; k++)
+            if (!((stalled >> (k % ns)) & 1)) ptx::mbar_wait_bounded(&full[k % ns], (uint32_t)(k / ns) & 1, kDrainNs);
+        return;
+    }
+
+    // ---------------- consumers
+    const int tg = lane & 7, rg = lane >> 3;
+    const uint32_t tgx = (uint32_t)tg << 4;
+    uint32_t phase = 0;
+    bool fresh = false;   // Y, the bias and the workspace may be touched
+    for (; u < units; u += gridDim.x) {
+        while (u >= b.start[h + 1]) h++;
+        const XcArgs &a = b.args[h];
+        const Unit un = unit_at<TT>(a, u - b.start[h]);
+        const bool has = warp < un.n;
+        f2_t acc[TT / 2][8];   // pairs of tokens
+#pragma unroll
+        for (int i = 0; i < TT / 2; i++)
+#pragma unroll
+            for (int j = 0; j < 8; j++) acc[i][j] = 0ull;
+        for (int c = 0; c < nch; c++) {
+            if (!__all_sync(0xffffffffu, ptx::mbar_try_wait(&full[s], phase))) {
+                const bool got = wait_or_abort(&full[s], phase, a.wait_ns * (fresh ? 1 : 2), &stop);
+                if (!__all_sync(0xffffffffu, got && !aborted(&stop))) {
+                    halt(a.status);
+                    return;
+                }
+            }
+            if (has) {
+                const unsigned char *st = base + (size_t)s * stage_bytes;
+                const unsigned char *xs = st + tg * 128;
+                const int4 *hdr = reinterpret_cast<const int4 *>(st + kX + warp * b.item_bytes);
+                int n = hdr->x;   // columns; then their places, then their weights
+                const int4 *oc = hdr + 1;
+                const float *w = reinterpret_cast<const float *>(oc + ((n + 3) >> 2)) + 4 * rg;
+                for (; n >= 4; n -= 4, w += 4 * 32) {
+                    const int4 o = *oc++;
+                    column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
+                    column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
+                    asm volatile("" ::: "memory");   // two columns' operands at a time: no more fit the registers
+                    column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
+                    column<TT>(acc, xs + ((uint32_t)o.w ^ tgx), w + 96);
+                    asm volatile("" ::: "memory");
+                }
+                if (n > 0) {
+                    const int4 o = *oc;
+                    column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
+                    if (n > 1) column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
+                    if (n > 2) column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&empty[s]);
+            if (++s == ns) {
+                s = 0;
+                phase ^= 1;
+            }
+        }
+        if (!fresh) {
+            ptx::pdl_wait();   // the bias, Y and the workspace may be an earlier kernel's
+            fresh = true;
+        }
+        if (!has) continue;
+        // ---- the bias, and the item's rows of Y (or of its slot of the
+        // workspace, for a piece of a split row)
+        const Item it = a.items[un.i0 + warp];
+        const bool partial = it.slot >= 0;
+        const int64_t pitch = partial ? 32 : a.M;
+        float *out = partial ? a.ws + (int64_t)it.slot * b.N * 32 : a.Y + (int64_t)it.row * 32;
+        const float *bias = a.bias && !partial ? a.bias + (int64_t)it.row * 32 : nullptr;
+        float bv[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) bv[j] = bias ? __ldg(bias + (j < 4 ? 4 * rg + j : 16 + 4 * rg + j - 4)) : 0.f;
+#pragma unroll
+        for (int i = 0; i < TT; i++) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                float even, odd;
+                unpack2(acc[i >> 1][j], even, odd);
+                v[j] = i & 1 ? odd : even;
+            }
+            const int64_t t = un.n0 + tg + 8 * i;
+            if (t < b.N) {
+                float *dst = out + t * pitch + 4 * rg;
+                *reinterpret_cast<float4 *>(dst) = make_float4(v[0] + bv[0], v[1] + bv[1], v[2] + bv[2], v[3] + bv[3]);
+                *reinterpret_cast<float4 *>(dst + 16) =
+                    make_float4(v[4] + bv[4], v[5] + bv[5], v[6] + bv[6], v[7] + bv[7]);
+            }
+        }
+    }
+}
+
+// Weights of every packed column: src[2 k] = float offset of its R weights,
+// src[2 k + 1] = its stored block.
+__global__ void k_pack_xcol(const float *__restrict__ data, const int32_t *__restrict__ src, int64_t n, int R,
+                            float *__restrict__ out) {
+    const int64_t total = n * R;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = e / R;
+        const int r = (int)(e - k * R);
+        out[(int64_t)src[2 * k] + r] = data[(int64_t)src[2 * k + 1] * R + r];
+    }
+}
+__global__ void k_pack_xcol_ints(const int32_t *__restrict__ pairs, int64_t n, int32_t *__restrict__ out) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+        out[pairs[2 * k]] = pairs[2 * k + 1];
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+        else
+            cudaGetLastError();
+    });
+    return fn;
+}
+
+template <typename K>
+cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const uint64_t bit = 1ull << (dev & 63);
+    if (done.load() & bit) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kXcMaxSmem - 1024);
+    if (e == cudaSuccess) done.fetch_or(bit);
+    return e;
+}
+
+template <int MAXB, int TT>
+cudaError_t launch(const LaunchArgs *las, int n) {
+    XcBatch<MAXB> b;
+    b.n = 0;
+    b.N = las[0].N;
+    const int64_t K = las[0].sc->K;
+    b.nch = (int)((K + kXcChunk - 1) / kXcChunk);
+    b.item_bytes = 0;
+    int64_t units = 0;
+    for (int i = 0; i < n; i++) {
+        const LaunchArgs &la = las[i];
+        const Schedule &sc = *la.sc;
+        if (la.N == 0 || sc.items.empty()) continue;
+        XcArgs &a = b.args[b.n];
+        a.table = sc.xc.d_table;
+        a.packed = static_cast<const unsigned char *>(la.data) + sc.xc.off;
+        a.items = sc.d_items;
+        a.bias = la.bias;
+        a.Y = static_cast<float *>(la.Y);
+        a.ws = la.ws;
+        a.status = la.status;
+        a.M = sc.M;
+        a.wait_ns = la.wait_ns;
+        a.n_items = (int)sc.items.size();
+        a.n_tasks = (a.n_items + NW - 1) / NW;
+        a.tiles = (unsigned)((la.N + 8 * TT - 1) / (8 * TT));
+        a.stall_chunk = la.stall_chunk;
+        b.start[b.n] = (unsigned)units;
+        units += (int64_t)a.tiles * a.n_tasks;
+        b.item_bytes = std::max(b.item_bytes, sc.xc.item_bytes);
+        b.n++;
+        if (units > INT32_MAX) return cudaErrorInvalidConfiguration;
+    }
+    if (b.n == 0) return cudaSuccess;
+    b.start[b.n] = (unsigned)units;
+    b.stage_bytes = xcol_stage_bytes(b.item_bytes);
+    b.ns = (int)std::min<uint32_t>(kXcStagesMax, kXcRoom / b.stage_bytes);
+    if (b.ns < 1) return cudaErrorInvalidConfiguration;
+    auto enc = encode_fn();
+    if (!enc) return cudaErrorNotSupported;
+    CUtensorMap map;
+    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)b.N}, strides[1] = {(cuuint64_t)K * 4};
+    const cuuint32_t box[2] = {32, 8 * TT}, estr[2] = {1, 1};
+    if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(las[0].X), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    static std::atomic<uint64_t> attr_set{0};
+    cudaError_t e = allow_smem(k_xcol<MAXB, TT>, attr_set);
+    if (e != cudaSuccess) return e;
+    const unsigned grid = (unsigned)std::min<int64_t>(units, las[0].sc->sm_count);
+    return launch_kernel(k_xcol<MAXB, TT>, dim3(grid), dim3(kThreads), b.ns * b.stage_bytes + 1024, las[0].stream, map,
+                         b);
+}
+
+template <int TT>
+cudaError_t launch_n(const LaunchArgs *las, int n) {
+    return n == 1 ? launch<1, TT>(las, 1) : launch<kXcBatchMax, TT>(las, n);
+}
+
+}  // namespace
+
+cudaError_t pack_xcol_data(const Schedule &sc, const void *data, void *packed, cudaStream_t s) {
+    const XcPlan &pl = sc.xc;
+    unsigned char *out = static_cast<unsigned char *>(packed) + pl.off;
+    const int64_t ni = (int64_t)pl.ints.size() / 2, nc = (int64_t)pl.src.size() / 2;
+    if (ni)
+        k_pack_xcol_ints<<<(int)std::min<int64_t>((ni + 255) / 256, 4096), 256, 0, s>>>(pl.d_ints, ni,
+                                                                                       reinterpret_cast<int32_t *>(out));
+    if (nc)
+        k_pack_xcol<<<(int)std::min<int64_t>((nc * sc.R + 255) / 256, 1 << 16), 256, 0, s>>>(
+            static_cast<const float *>(data), pl.d_src, nc, sc.R, reinterpret_cast<float *>(out));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_xcol(const LaunchArgs *las, const int *tiles, int n) {
+    if (n <= 0) return cudaSuccess;
+    if (n > kXcBatchMax) return cudaErrorInvalidValue;
+    switch (kXcTT[tiles[0]]) {
+        case 8: return launch_n<8>(las, n);
+        case 12: return launch_n<12>(las, n);
+        case 14: return launch_n<14>(las, n);
+    }
+    return cudaErrorInvalidConfiguration;
+}
+
+}  // namespace bsr

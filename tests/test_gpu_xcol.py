@@ -1,0 +1,17 @@
+"""The column-list SIMT kernel for fp32 32x1 blocks at each of its token tiles
+(forced: by itself it takes large calls only)."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.mark.parametrize("tile", [0, 1, 2])
+def test_xcol_parity_at_tile(tile):
+    r = subprocess.run([sys.executable, "-m", "tests.xcol_check"], cwd=ROOT, env=dict(os.environ, BSR_XC_TILE=str(tile)),
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
