@@ -22,8 +22,16 @@
 // Items of a task are neighbours in length, so warps stay within the ring of
 // one another.
 //
-// Measured (us, back to back, the per-task kernel in brackets): see
-// choose_xcol.
+// So that an output is not one long chain of additions, a warp adds its tile to
+// a running sum after every segment of chunks (about 52 columns). Registers and
+// shared memory are full; the sums live in tensor memory, which nothing else
+// uses here: a warp reaches 32 lanes of it, so up to three tiles of 112 columns.
+//
+// (With 112 accumulators the largest tile spills a dozen registers around that
+// addition: one chain per output runs 85.5 us where this takes 98.1, but its
+// relative error at 102 columns is 1.8e-7 instead of 1.3e-7, at 512 4.0e-7.)
+//
+// Measured, with the per-task kernel beside it: see choose_xcol.
 //
 // Every wait is bounded by the global timer; a timeout sets the device status
 // word, stops the CTA's roles, lets the issued copies land and returns.
@@ -37,6 +45,7 @@
 #include "bsr_internal.h"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "tcgen05.cuh"
 
 namespace bsr {
 
@@ -45,6 +54,8 @@ namespace {
 constexpr int NW = kXcWarps;
 constexpr int kThreads = 32 * (NW + 1);
 constexpr int kStagesMax = kXcStagesMax;
+constexpr uint32_t kTmemCols = 512;   // three warps a lane quarter, a tile's 112 columns each (a power of two)
+constexpr uint32_t kTileCols = 8 * kXcTT[kXcTileSizes - 1];   // of the largest tile
 constexpr uint64_t kDrainNs = 200000000ull;
 
 struct XcArgs {
@@ -57,6 +68,7 @@ struct XcArgs {
     int64_t M;
     uint64_t wait_ns;
     int n_items, n_tasks;
+    int seg;                     // chunks per segment
     unsigned tiles;
     int stall_chunk;
 };
@@ -142,6 +154,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
     unsigned char *base = ptx::align_smem(smem_raw);
     __shared__ uint64_t full[kStagesMax], empty[kStagesMax];
     __shared__ int stop;
+    __shared__ uint32_t tmem_s;
     const int ns = b.ns;
     const uint32_t stage_bytes = b.stage_bytes;
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -153,7 +166,10 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
         stop = 0;
         ptx::fence_barrier_init();
     }
+    if (warp == 0) tc5::alloc(&tmem_s, kTmemCols);
+    tc5::fence_before();
     __syncthreads();
+    tc5::fence_after();
     const unsigned units = b.start[b.n];
     const bool elected = ptx::elect_one();
     auto halt = [&](int *status) {
@@ -234,94 +250,143 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
         // no copy may outlive the CTA (a stage that was consumed has landed long ago)
         for (int k = max(0, issued - ns); k < issued; k++)
             if (!((stalled >> (k % ns)) & 1)) ptx::mbar_wait_bounded(&full[k % ns], (uint32_t)(k / ns) & 1, kDrainNs);
-        return;
-    }
-
-    // ---------------- consumers
-    const int tg = lane & 7, rg = lane >> 3;
-    const uint32_t tgx = (uint32_t)tg << 4;
-    uint32_t phase = 0;
-    bool fresh = false;   // Y, the bias and the workspace may be touched
-    for (; u < units; u += gridDim.x) {
-        while (u >= b.start[h + 1]) h++;
-        const XcArgs &a = b.args[h];
-        const Unit un = unit_at<TT>(a, u - b.start[h]);
-        const bool has = warp < un.n;
-        f2_t acc[TT / 2][8];   // pairs of tokens
+        __syncwarp();
+    } else {
+        // ---------------- consumers
+        const int tg = lane & 7, rg = lane >> 3;
+        const uint32_t tgx = (uint32_t)tg << 4;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (; ok && u < units; u += gridDim.x) {
+            while (u >= b.start[h + 1]) h++;
+            const XcArgs &a = b.args[h];
+            const bool has = warp < unit_at<TT>(a, u - b.start[h]).n;
+            f2_t acc[TT / 2][8];   // pairs of tokens
 #pragma unroll
-        for (int i = 0; i < TT / 2; i++)
+            for (int i = 0; i < TT / 2; i++)
 #pragma unroll
-            for (int j = 0; j < 8; j++) acc[i][j] = 0ull;
-        for (int c = 0; c < nch; c++) {
-            if (!__all_sync(0xffffffffu, ptx::mbar_try_wait(&full[s], phase))) {
-                const bool got = wait_or_abort(&full[s], phase, a.wait_ns * (fresh ? 1 : 2), &stop);
-                if (!__all_sync(0xffffffffu, got && !aborted(&stop))) {
-                    halt(a.status);
-                    return;
+                for (int j = 0; j < 8; j++) acc[i][j] = 0ull;
+            auto sums = [&]() {   // this warp's running sums
+                return tmem_s + ((uint32_t)(32 * (warp & 3)) << 16) +
+                       (uint32_t)(warp >> 2) * kTileCols;
+            };
+            auto add_sums = [&]() {   // acc += the running sums
+                const uint32_t at = sums();
+#pragma unroll
+                for (int k = 0; k < 8 * TT; k += 8) {
+                    uint32_t v[8];
+                    tc5::ld8(at + k, v);
+                    tc5::ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        asm volatile("" : "+r"(v[2 * e]), "+r"(v[2 * e + 1]));   // no use moves above the wait
+                        f2_t &t = acc[(k / 2 + e) / 8][(k / 2 + e) % 8];
+                        float even, odd;
+                        unpack2(t, even, odd);
+                        t = pack2(even + __uint_as_float(v[2 * e]), odd + __uint_as_float(v[2 * e + 1]));
+                    }
+                }
+            };
+            for (int c = 0, c1 = a.seg; c < nch; c++) {
+                if (!__all_sync(0xffffffffu, ptx::mbar_try_wait(&full[s], phase))) {
+                    const bool got = wait_or_abort(&full[s], phase, 2 * a.wait_ns, &stop);
+                    ok = __all_sync(0xffffffffu, got && !aborted(&stop));
+                    if (!ok) {
+                        halt(a.status);
+                        break;
+                    }
+                }
+                if (has) {
+                    const unsigned char *st = base + (size_t)s * stage_bytes;
+                    const unsigned char *xs = st + tg * 128;
+                    const int4 *hdr = reinterpret_cast<const int4 *>(st + kX + warp * b.item_bytes);
+                    int n = hdr->x;   // columns; then their places, then their weights
+                    const int4 *oc = hdr + 1;
+                    const float *w = reinterpret_cast<const float *>(oc + ((n + 3) >> 2)) + 4 * rg;
+                    for (; n >= 4; n -= 4, w += 4 * 32) {
+                        const int4 o = *oc++;
+                        column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
+                        column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
+                        asm volatile("" ::: "memory");   // two columns' operands at a time: no more fit the registers
+                        column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
+                        column<TT>(acc, xs + ((uint32_t)o.w ^ tgx), w + 96);
+                        asm volatile("" ::: "memory");
+                    }
+                    if (n > 0) {
+                        const int4 o = *oc;
+                        column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
+                        if (n > 1) column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
+                        if (n > 2) column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&empty[s]);
+                if (++s == ns) {
+                    s = 0;
+                    phase ^= 1;
+                }
+                if (c + 1 == c1 && c1 < nch) {
+                    if (c1 > a.seg) add_sums();
+                    const uint32_t at = sums();
+#pragma unroll
+                    for (int k = 0; k < 8 * TT; k += 8) {
+                        uint32_t v[8];
+#pragma unroll
+                        for (int e = 0; e < 4; e++) {
+                            f2_t &t = acc[(k / 2 + e) / 8][(k / 2 + e) % 8];
+                            float even, odd;
+                            unpack2(t, even, odd);
+                            v[2 * e] = __float_as_uint(even);
+                            v[2 * e + 1] = __float_as_uint(odd);
+                            t = 0ull;
+                        }
+                        tc5::st8(at + k, v);
+                    }
+                    tc5::st_wait();
+                    c1 += a.seg;
                 }
             }
-            if (has) {
-                const unsigned char *st = base + (size_t)s * stage_bytes;
-                const unsigned char *xs = st + tg * 128;
-                const int4 *hdr = reinterpret_cast<const int4 *>(st + kX + warp * b.item_bytes);
-                int n = hdr->x;   // columns; then their places, then their weights
-                const int4 *oc = hdr + 1;
-                const float *w = reinterpret_cast<const float *>(oc + ((n + 3) >> 2)) + 4 * rg;
-                for (; n >= 4; n -= 4, w += 4 * 32) {
-                    const int4 o = *oc++;
-                    column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
-                    column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
-                    asm volatile("" ::: "memory");   // two columns' operands at a time: no more fit the registers
-                    column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
-                    column<TT>(acc, xs + ((uint32_t)o.w ^ tgx), w + 96);
-                    asm volatile("" ::: "memory");
-                }
-                if (n > 0) {
-                    const int4 o = *oc;
-                    column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
-                    if (n > 1) column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
-                    if (n > 2) column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&empty[s]);
-            if (++s == ns) {
-                s = 0;
-                phase ^= 1;
-            }
-        }
-        if (!fresh) {
+            if (!ok) break;
+            if (nch > a.seg) add_sums();
             ptx::pdl_wait();   // the bias, Y and the workspace may be an earlier kernel's
-            fresh = true;
-        }
-        if (!has) continue;
-        // ---- the bias, and the item's rows of Y (or of its slot of the
-        // workspace, for a piece of a split row)
-        const Item it = a.items[un.i0 + warp];
-        const bool partial = it.slot >= 0;
-        const int64_t pitch = partial ? 32 : a.M;
-        float *out = partial ? a.ws + (int64_t)it.slot * b.N * 32 : a.Y + (int64_t)it.row * 32;
-        const float *bias = a.bias && !partial ? a.bias + (int64_t)it.row * 32 : nullptr;
-        float bv[8];
+            if (!has) continue;
+            // (the unit once more: the registers are the columns' until here)
+            const Unit un = unit_at<TT>(a, u - b.start[h]);
+            // ---- the bias, and the item's rows of Y (or of its slot of the
+            // workspace, for a piece of a split row)
+            const Item it = a.items[un.i0 + warp];
+            const bool partial = it.slot >= 0;
+            const int64_t pitch = partial ? 32 : a.M;
+            float *out = partial ? a.ws + (int64_t)it.slot * b.N * 32 : a.Y + (int64_t)it.row * 32;
+            const float *bias = a.bias && !partial ? a.bias + (int64_t)it.row * 32 : nullptr;
+            float bv[8];
 #pragma unroll
-        for (int j = 0; j < 8; j++) bv[j] = bias ? __ldg(bias + (j < 4 ? 4 * rg + j : 16 + 4 * rg + j - 4)) : 0.f;
+            for (int j = 0; j < 8; j++) bv[j] = bias ? __ldg(bias + (j < 4 ? 4 * rg + j : 16 + 4 * rg + j - 4)) : 0.f;
 #pragma unroll
-        for (int i = 0; i < TT; i++) {
-            float v[8];
+            for (int i = 0; i < TT; i++) {
+                float v[8];
 #pragma unroll
-            for (int j = 0; j < 8; j++) {
-                float even, odd;
-                unpack2(acc[i >> 1][j], even, odd);
-                v[j] = i & 1 ? odd : even;
+                for (int j = 0; j < 8; j++) {
+                    float even, odd;
+                    unpack2(acc[i >> 1][j], even, odd);
+                    v[j] = i & 1 ? odd : even;
+                }
+                const int64_t t = un.n0 + tg + 8 * i;
+                if (t < b.N) {
+                    float *dst = out + t * pitch + 4 * rg;
+                    *reinterpret_cast<float4 *>(dst) = make_float4(v[0] + bv[0], v[1] + bv[1], v[2] + bv[2], v[3] + bv[3]);
+                    *reinterpret_cast<float4 *>(dst + 16) =
+                        make_float4(v[4] + bv[4], v[5] + bv[5], v[6] + bv[6], v[7] + bv[7]);
+                }
             }
-            const int64_t t = un.n0 + tg + 8 * i;
-            if (t < b.N) {
-                float *dst = out + t * pitch + 4 * rg;
-                *reinterpret_cast<float4 *>(dst) = make_float4(v[0] + bv[0], v[1] + bv[1], v[2] + bv[2], v[3] + bv[3]);
-                *reinterpret_cast<float4 *>(dst + 16) =
-                    make_float4(v[4] + bv[4], v[5] + bv[5], v[6] + bv[6], v[7] + bv[7]);
-            }
         }
+        __syncwarp();
+    }
+    tc5::fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc5::fence_after();
+        tc5::dealloc(tmem_s, kTmemCols);
     }
 }
 
@@ -393,6 +458,7 @@ cudaError_t launch(const LaunchArgs *las, int n) {
         a.wait_ns = la.wait_ns;
         a.n_items = (int)sc.items.size();
         a.n_tasks = (a.n_items + NW - 1) / NW;
+        a.seg = sc.xc.seg;
         a.tiles = (unsigned)((la.N + 8 * TT - 1) / (8 * TT));
         a.stall_chunk = la.stall_chunk;
         b.start[b.n] = (unsigned)units;

@@ -33,6 +33,7 @@ struct XcPlan {
     bool ok = false;
     int64_t off = -1, bytes = 0;       // place in the handle's packed buffer
     uint32_t item_bytes = 0;           // largest packed chunk of an item
+    int seg = 1;                       // chunks per segment (one chain of additions)
     std::vector<int32_t> table;        // per item and chunk: its start / 16 (and the end)
     std::vector<int32_t> ints;         // (place / 4 bytes, value) of the packed buffer's integers
     std::vector<int32_t> src;          // per column: its weights' place / 4 bytes, its block

@@ -48,6 +48,13 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     }
     pl.table.push_back((int32_t)(at / 4));
     pl.bytes = at * 4;
+    // equal segments of about 52 columns: outputs are then no further from 64
+    // bits than the per-task kernel's, which shares a row among warps (relative
+    // error at 102 columns in one chain 1.8e-7, at 512 4.0e-7; the per-task
+    // kernel's 1.3e-7)
+    const double mean = (double)sc.nnzb / (double)n_items;
+    const int64_t segs = std::min<int64_t>(nch, std::max<int64_t>(1, (int64_t)(mean / 52.0 + 0.999)));
+    pl.seg = (int)((nch + segs - 1) / segs);
     if (2 * xcol_stage_bytes(pl.item_bytes) > kXcRoom) return base;   // a ring of two stages
     pl.ok = true;
     return pl.off + pl.bytes;
@@ -55,14 +62,14 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
 
 // The tile that minimises the busiest scheduler's cycles, where that beats the
 // per-task kernel. A task's items sit one per warp, ceil(items / 4) to a
-// scheduler; a column takes it about 10 TT + 25 cycles, a chunk 100, a unit's
+// scheduler; a column takes it about 11.5 TT + 25 cycles, a chunk 100, a unit's
 // stores 60 TT; the per-task kernel pays about 0.85 cycles per unit of its own
 // model. Fitted to (us, this kernel and the per-task one): 1024 x 1024 at 90%,
-// 16384 tokens 85.8 and 123 (TT = 14; 12: 107, 8: 119), 4096 tokens 30.3 and
-// 36.5 (TT = 12); at 50%, 16384 tokens 333 and 659; 768 x 768 at 70%, 3000
-// tokens 29.4 and 37.3 (TT = 8); 1536 x 1536 at 95%, 4000 tokens 46.8 and 38.9
-// (few columns per unit: stays); 768 x 768 at 50%, 1024 tokens 43.2 and 30.5
-// (24 items leave most SMs idle: stays). The model is 3 to 15% under.
+// 16384 tokens 98.1 and 123 (TT = 14), 4096 tokens 30.5 and 36.5 (TT = 12); at
+// 50%, 16384 tokens 377 and 659; 768 x 768 at 70%, 3000 tokens 30.4 and 37.3
+// (TT = 8); 1536 x 1536 at 95%, 4000 tokens 47 and 38.9 (few columns per unit:
+// stays); 768 x 768 at 50%, 1024 tokens 43 and 30.5 (24 items leave most SMs
+// idle: stays).
 int choose_xcol(const Schedule &sc, int64_t N) {
     static const int mode = [] {
         const char *v = getenv("BSR_XC");
@@ -89,7 +96,7 @@ int choose_xcol(const Schedule &sc, int64_t N) {
         const int TT = kXcTT[ti];
         const int64_t units = ((N + 8 * TT - 1) / (8 * TT)) * tasks;
         const double rounds = (double)((units + sc.sm_count - 1) / sc.sm_count);
-        const double cost = 1.1 * (rounds * (warps * columns * (10.0 * TT + 25.0) + 100.0 * chunks + 60.0 * TT) + 4000.0);
+        const double cost = rounds * (warps * columns * (11.5 * TT + 25.0) + 100.0 * chunks + 60.0 * TT) + 4000.0;
         if (cost < best_cost) {
             best_cost = cost;
             best = ti;
