@@ -48,8 +48,8 @@ struct DensePlan {
 struct Schedule;
 struct LaunchArgs;
 
-// Fills sc.dense (after the tensor-core plan; `base`: the first free byte of
-// the packed buffer); returns the buffer's new end.
+// Fills sc.dense (after the variant's plan; `base`: the first free byte of the
+// packed buffer); returns the buffer's new end.
 int64_t plan_dense(Schedule &sc, int64_t base);
 // Row groups per task for a call of N tokens, with kDnPair where pairs of
 // CTAs run it (0: the kernel does not run it).

@@ -12,7 +12,8 @@ int64_t plan_dense(Schedule &sc, int64_t base) {
     DensePlan &pl = sc.dense;
     pl.ok = false;
     const bool shape_ok = kDnGroup % sc.R == 0 || sc.R % kDnGroup == 0;
-    if (sc.variant != V_TC || sc.dt != BSR_BF16 || sc.M % kDnGroup || sc.K % 8 || !shape_ok) return base;
+    if ((sc.variant != V_TC && sc.variant != V_XSTAGE) || sc.dt != BSR_BF16 || sc.M % kDnGroup || sc.K % 8 || !shape_ok)
+        return base;
     const int64_t n_groups = sc.M / kDnGroup, nch = (sc.K + kDnChunk - 1) / kDnChunk;
     if (n_groups > INT32_MAX / 32 || nch > 1 << 20) return base;
     // per row group, the chunks that hold a kept block (a byte each)
@@ -98,7 +99,10 @@ int64_t plan_dense(Schedule &sc, int64_t base) {
 // 16x16 blocks of 1024 x 1024 at 99% (24 against 40 us at 16384 tokens), and
 // lost on 16x16 blocks of 4096 x 4096 at 97% (60 against 40 us at 2048
 // tokens: every chunk has a block of some row, and the dense tiles do 33
-// times the kept multiply-adds).
+// times the kept multiply-adds). Narrow blocks too sparse for the block-by-
+// block kernel have the per-task SIMT kernel beside this one, at about 0.85
+// cycles per unit of its model: 32x1 of 1024 x 1024 at 95%, 16384 tokens, 26.2
+// against 69 us.
 int choose_dense(const Schedule &sc, int64_t N) {
     static const int mode = [] {
         const char *v = getenv("BSR_DENSE");
@@ -145,9 +149,15 @@ int choose_dense(const Schedule &sc, int64_t N) {
             }
         }
     }
-    double by_blocks = 0.0;
-    choose_tc_tasks(sc, N, &by_blocks);
-    if (mode != 1 && by_blocks > 0 && best_cost > 300.0 * by_blocks) best = 0;
+    double other = 0.0;   // the variant's own kernel
+    if (sc.variant == V_TC) {
+        choose_tc_tasks(sc, N, &other);
+        other *= 300.0;
+    } else {
+        choose_tasks(sc, N, &other);
+        other *= 0.85;
+    }
+    if (mode != 1 && other > 0 && best_cost > other) best = 0;
     if (N < (int64_t)1 << 48) pl.last.store((uint64_t)N << 16 | (uint64_t)best, std::memory_order_relaxed);
     return best;
 }

@@ -515,14 +515,14 @@ bsr_status_t build_schedule(Schedule &sc) {
         plan_xstage(sc);
     }
     if (sc.variant == V_XSTAGE && (int64_t)sc.xs_blob.size() > INT32_MAX) sc.variant = V_GENERIC;   // blob offsets are int32
-    // the dense-tile kernel (bf16 tensor-core schedules), the column-list kernel
+    // the dense-tile kernel (bf16), the column-list kernel
     // (fp32 32x1 blocks) and
     // the gathered-K kernel, after the variant's own packed values (the
     // generic kernel's: a copy of the caller's block values)
     if (sc.variant == V_TC)
         plan_gk(sc, plan_dense(sc, sc.tc_w_total));
     else if (sc.variant == V_XSTAGE)
-        plan_gk(sc, plan_xcol(sc, (int64_t)sc.xs_blob.size() * 4));
+        plan_gk(sc, plan_xcol(sc, plan_dense(sc, (int64_t)sc.xs_blob.size() * 4)));
     else
         plan_gk(sc, sc.nnzb * sc.R * sc.C * (int64_t)dtype_size(sc.dt));
     if (sc.variant == V_GENERIC) {
@@ -738,7 +738,10 @@ int fusion_class(const Schedule &sc, int64_t N, int *G) {
         *G = 0;
         return -1;
     }
-    if (choose_tcp(sc, N) < 0 && (*G = choose_xcol(sc, N)) >= 0) return kXcolClass + *G;
+    if (choose_tcp(sc, N) < 0) {
+        if ((*G = choose_dense(sc, N)) > 0) return kDenseClass + (*G & kDnPair);
+        if ((*G = choose_xcol(sc, N)) >= 0) return kXcolClass + *G;
+    }
     if (sc.variant == V_XSTAGE) {
         *G = choose_tasks(sc, N);
         return 2 * xstage_fusion_key(sc, *G);
@@ -748,7 +751,6 @@ int fusion_class(const Schedule &sc, int64_t N, int *G) {
             *G = 0;
             return -1;
         }
-        if ((*G = choose_dense(sc, N)) > 0) return kDenseClass + (*G & kDnPair);
         *G = choose_tc_tasks(sc, N);
         return 2 * tc_fusion_key(sc) + 1;
     }

@@ -68,3 +68,26 @@ def test_dense_batch_of_different_shapes_is_bitwise_the_single_calls():
         assert np.array_equal(to_host(Y), single)
         check_product(single, oracle.bsr_from_dense(w.W, w.R, w.C), X, w.bias, w.M)
         assert h.check_device_status() == 0
+
+
+@pytest.mark.parametrize("R,C,N", [(32, 1, 3000), (1, 1, 700), (4, 4, 129)])
+def test_dense_takes_sparse_narrow_weights_of_the_simt_variant(R, C, N):
+    """bf16 blocks too sparse for the block-by-block kernel (1/12 fill): the
+    schedule's variant stays the SIMT kernel, calls may run on dense tiles;
+    either way the product is the oracle's, and a batch is the single calls."""
+    import paper_2106_08846_gb300 as bsr
+    M, K = 768, 1024
+    ws = [synth.make_weight("dx", 7800 + i, M, K, R, C, "bf16", 0,
+                            mask=synth.uniform_block_mask(7800 + i, M // R, K // C, (M // R) * (K // C) * (3 + i) // 100))
+          for i in range(2)]
+    hs = [bsr.bsr_create(*build_on_gpu(w.W, R, C), R, C, M, K) for w in ws]
+    assert all(h.schedule()["variant"] == "xstage" for h in hs)
+    X = synth.activations(7801, N, K, "bf16")
+    Xd, b = to_dev(X), to_dev(ws[0].bias)
+    Ys = [torch.empty((N, M), dtype=torch.bfloat16, device="cuda") for _ in ws]
+    bsr.bsr_spmm_batch(hs, Xd, [b, None], Ys, N)
+    rows = np.unique(np.concatenate([np.arange(0, N, 13), np.arange(N - 130 if N > 130 else 0, N)]))
+    for i, (h, w, Y) in enumerate(zip(hs, ws, Ys)):
+        single = to_host(h.spmm(Xd, b if i == 0 else None))
+        assert np.array_equal(to_host(Y), single)
+        check_product(single, oracle.bsr_from_dense(w.W, R, C), X, ws[0].bias if i == 0 else None, M, rows=rows)
