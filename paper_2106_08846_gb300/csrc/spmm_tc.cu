@@ -13,7 +13,7 @@
 //                         (repacked at create time into the MMA's K-major
 //                         layout, in task-chunk order); chunks without blocks
 //                         are neither loaded nor visited.
-//   warp 1 (one thread)  owns the tensor memory (G * R fp32 columns, one
+//   warp 1 (fp32: 1..4)  owns the tensor memory (G * R fp32 columns, one
 //                         block row per R columns) and issues the MMAs from
 //                         the work list (per chunk, one packed entry per
 //                         block: column offset, item, first-block flag, stack
@@ -21,18 +21,24 @@
 //                         block is a stack: one MMA per K slice with
 //                         N = items x R over their adjacent accumulators. A
 //                         tcgen05.commit per chunk releases the stage.
-//   warps 2..5           fp32: write the tf32 low parts of every landed X
-//                         stage into a twin buffer (the MMAs read the stage
-//                         itself as the high parts) for the issuer's
-//                         high x high + high x low + low x high; then the
-//                         epilogue: each reads its 32 TMEM lanes (tokens),
+//   the last four warps  fp32: split every landed X stage into tf32 high and
+//                         low parts in tensor memory, the A operands of the
+//                         issuers' high x high + high x low + low x high; then
+//                         the epilogue: each reads its 32 TMEM lanes (tokens),
 //                         adds the bias, converts, stages 16-column groups in
 //                         the idle X ring and one thread stores them to Y by
 //                         2-D TMA (split rows write fp32 partials directly).
 //
 // Two CTAs share an SM, so that one CTA's set-up, stage round trips and
-// epilogue overlap the other's MMAs: bf16 uses a 3-stage ring, fp32 a 2-stage
-// ring (plus the low twins).
+// epilogue overlap the other's MMAs: bf16 uses a 3-stage ring; fp32 as many
+// stages as fit (tc_ring), and one CTA where its accumulators need more than
+// half of the tensor memory.
+// What bounded fp32: shared memory. With A in shared memory a block's MMAs each
+// read its 4 KB a K slice (16x16 at 90%: 86 KB a chunk, 675 of its 1270 cycles),
+// beside the split's reads and writes. With A in tensor memory the split reads X
+// once and the MMAs only their blocks: 1024 x 1024 at 90%, 16384 tokens, 16x16
+// 84.9 -> 75.7 us, 32x32 73.1 -> 57.4; 64x32 at 80%, 4096 tokens 25.3 -> 17.3;
+// 32x32 of 768 x 768 at 80%, 1024 tokens 11.3 -> 9.4.
 // Launched with programmatic stream serialisation: set-up and the work list
 // come before the wait for the previous kernel; X, bias, Y after it. Every
 // wait is bounded by the global timer; a timeout sets the device status word,
@@ -64,11 +70,12 @@ constexpr uint32_t kStageBytes = TN * 128;   // 16 KB: 128 token rows of 128 byt
 template <typename T>
 struct TcCfg {
     static constexpr int KC = 128 / (int)sizeof(T);
-    static constexpr int NS = sizeof(T) == 4 ? kTcStagesF32 : kTcStages;
+    static constexpr int NSMAX = sizeof(T) == 4 ? kTcStagesF32 : kTcStages;   // fp32: a.ns of them (as many as fit)
     static constexpr int NISS = tc_issuers(sizeof(T) == 4);   // MMA-issuing warps (lane 0 of each)
     static constexpr int NTHREADS = tc_threads(sizeof(T) == 4);
 };
 constexpr uint64_t kDrainNs = 200000000ull;
+constexpr size_t kTcYStaging = 65536;   // two rounds of fp32 Y staging, in the idle ring
 
 struct TcArgs {
     CUtensorMap ymap;         // Y [N, M] in 16-column x 128-row boxes, for the epilogue's TMA stores
@@ -85,6 +92,7 @@ struct TcArgs {
     int C, nchunks;
     uint32_t w_off, trec_smem, bias_off, bar_off, misc_off;
     uint32_t tmem_cols;
+    int ns, nslot;            // fp32: ring stages; A slots in tensor memory (64 columns each, after the accumulators)
     uint64_t wait_ns;
     int stall_chunk;
 };
@@ -109,14 +117,15 @@ template <typename T, int R>
 __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a, unsigned cta) {
     ptx::pdl_launch_dependents();
     constexpr bool F32 = sizeof(T) == 4;
-    constexpr int NS = TcCfg<T>::NS;
+    const int NS = F32 ? a.ns : TcCfg<T>::NSMAX;
+    const int nslot = F32 ? a.nslot : 1;
     constexpr int NISS = TcCfg<T>::NISS;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = ptx::align_smem(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(base + a.bar_off);
     uint64_t *empty = full + NS;
-    uint64_t *split = empty + NS;    // fp32: the stage's high/low parts are ready
-    uint64_t *done = split + NS;     // every MMA completed
+    uint64_t *split = empty + NS;    // fp32: an A slot's high/low parts are ready
+    uint64_t *done = split + NS;     // every MMA completed (nslot <= NS)
     uint64_t *rbar = done + 1;       // task record landed
     int *misc = reinterpret_cast<int *>(base + a.misc_off);   // [0] abort flag, [1] TMEM address
     int *itab = misc + 4;                                     // per item: row p0 p1 slot - len
@@ -140,7 +149,7 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
         for (int s = 0; s < NS; s++) {
             ptx::mbar_init(&full[s], 1);
             ptx::mbar_init(&empty[s], NISS);
-            ptx::mbar_init(&split[s], 1);
+            ptx::mbar_init(&split[s], 4);   // the split warps
         }
         ptx::mbar_init(done, NISS);
         ptx::mbar_init(rbar, 1);
@@ -162,6 +171,7 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
     __syncthreads();
     tc5::fence_after();
     const uint32_t tmem = (uint32_t)misc[1];
+    const uint32_t a_col = (uint32_t)max(32, a.G * R);           // fp32: the A slots' first column
     const uint32_t wblock = (uint32_t)R * C * (F32 ? 8 : 2);   // bytes of one block's B operand(s)
 
     if (warp == 0) {
@@ -176,29 +186,31 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
             }
             ptx::pdl_wait();   // X may be an earlier kernel's output
             const unsigned char *wsrc = static_cast<const unsigned char *>(a.wpk);
-            int k = 0;          // ring slots used (chunks with work, in order)
+            int k = 0, s = 0;   // ring slots used (chunks with work, in order); the next one's stage
+            uint32_t phase = 1; // parity of `empty` that a first use of a stage passes at once
             int stalled = -1;   // test hook: the slot left empty
             bool ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(rbar, 0, a.wait_ns));   // chunk starts, from shared memory
             const int64_t wfirst = ok ? I_s[0] : 0;                   // the task's first packed block
             for (int c = 0; ok && c < nch; c++) {
                 const int lo = I_s[4 + c], hi = I_s[5 + c];
                 if (lo == hi) continue;   // no block of this task in chunk c
-                const int s = k % NS;
-                const bool got = k < NS || ptx::mbar_wait_bounded(&empty[s], ((k / NS) - 1) & 1, a.wait_ns);
+                const bool got = ptx::mbar_wait_bounded(&empty[s], phase, a.wait_ns);
                 ok = __all_sync(0xffffffffu, got && !aborted(misc));
                 if (!ok) break;
-                if (c == a.stall_chunk) {   // never loaded: its consumer times out
-                    stalled = k++;
-                    continue;
-                }
                 // the X chunk and, beside it, the task's block values for this chunk
                 const uint32_t wbytes = (uint32_t)(hi - lo) * wblock;
-                if (elected) {
+                if (c == a.stall_chunk) {   // never loaded: its consumer times out
+                    stalled = k;
+                } else if (elected) {
                     ptx::mbar_arrive_expect_tx(&full[s], kStageBytes + wbytes);
                     ptx::tma_load_2d(base + s * kStageBytes, &xmap, c * TcCfg<T>::KC, (int32_t)n0, &full[s]);
                     ptx::bulk_load(W_s + s * a.wstage, wsrc + (wfirst + lo) * wblock, wbytes, &full[s]);
                 }
                 k++;
+                if (++s == NS) {
+                    s = 0;
+                    phase ^= 1;
+                }
             }
             if (!ok && elected) {
                 set_status(a.status, DEV_TIMEOUT);
@@ -236,13 +248,14 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
             const uint32_t ufirst = (uint32_t)i0, ucnt = (uint32_t)(i1 - i0);
             bool ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(rbar, 0, a.wait_ns) && !aborted(misc));
             const int32_t *ent = I_s + items_at + 4 * g_count;
-            int k = 0;   // chunks consumed
+            int s = 0, sl_ = 0;             // stage; fp32: A slot
+            uint32_t phase = 0, sphase = 0;
             for (int c = 0; ok && c < nch; c++) {
                 const int lo = I_s[4 + c], hi = I_s[5 + c];
                 if (lo == hi) continue;
-                const int s = k % NS;
                 // fp32: wait for the split parts (the split warps waited for the copy)
-                const bool got = ptx::mbar_wait_bounded(F32 ? &split[s] : &full[s], (k / NS) & 1, a.wait_ns);
+                const bool got =
+                    ptx::mbar_wait_bounded(F32 ? &split[sl_] : &full[s], F32 ? sphase : phase, a.wait_ns);
                 ok = __all_sync(0xffffffffu, got && !aborted(misc));
                 if (!ok) break;
                 tc5::fence_after();
@@ -306,14 +319,17 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
                     if constexpr (F32) {
                         // 3xTF32: high x high + high x low + low x high, K = 8 per MMA
                         constexpr uint32_t idesc = tc5::idesc(true, TN, R);
-                        const uint64_t adl = ad + (uint64_t)(NS * kStageBytes >> 4), bdl = bd + (uint64_t)((uint32_t)R * C * 4 >> 4);
+                        // (A from tensor memory: its 4 KB a K slice would be read
+                        // from shared memory by every MMA)
+                        const uint64_t bdl = bd + (uint64_t)((uint32_t)R * C * 4 >> 4);
+                        const uint32_t ah = tmem + a_col + (uint32_t)(sl_ * 64) + (v & 3u) * 8u;
 #pragma unroll 2
                         for (int sl = 0; sl < C / 8; sl++) {
-                            const uint64_t ka = (uint64_t)(sl * 2), kb = (uint64_t)(sl * (R * 2));   // 32 and R*32 bytes
+                            const uint64_t kb = (uint64_t)(sl * (R * 2));   // R * 32 bytes
                             if (elected) {
-                                tc5::mma_ss<true>(d, ad + ka, bd + kb, idesc, (first == 0u) | (sl > 0));
-                                tc5::mma_ss<true>(d, ad + ka, bdl + kb, idesc, 1u);
-                                tc5::mma_ss<true>(d, adl + ka, bd + kb, idesc, 1u);
+                                tc5::mma_ts<true>(d, ah + 8 * sl, bd + kb, idesc, (first == 0u) | (sl > 0));
+                                tc5::mma_ts<true>(d, ah + 8 * sl, bdl + kb, idesc, 1u);
+                                tc5::mma_ts<true>(d, ah + 32 + 8 * sl, bd + kb, idesc, 1u);
                             }
                         }
                     } else {
@@ -325,8 +341,15 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
                                                    (first == 0u) | (sl > 0));
                     }
                 }
-                if (elected) tc5::commit(&empty[s]);   // the stage is free once every issuer's MMAs completed
-                k++;
+                if (elected) tc5::commit(&empty[s]);   // the stage (and A slot) is free once every issuer's MMAs completed
+                if (++s == NS) {
+                    s = 0;
+                    phase ^= 1;
+                }
+                if (F32 && ++sl_ == nslot) {
+                    sl_ = 0;
+                    sphase ^= 1;
+                }
             }
             if (!ok && elected) {
                 set_status(a.status, DEV_TIMEOUT);
@@ -345,34 +368,58 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
         }
         bool split_ok = true;
         if constexpr (F32) {
-            // x = high + low per element of every loaded stage: the low part
-            // into the stage's twin buffer (same swizzled layout); the high
-            // part is the stage itself, since kind::tf32 MMAs use only the
-            // top 19 bits of each fp32 element (round-to-nearest would leave
-            // about 2^-11 relative error per product, far outside the fp32
-            // tolerance the parity tests check)
-            split_ok = ptx::mbar_wait_bounded(rbar, 0, a.wait_ns);
-            int k = 0;
+            // x = high + low per element of every loaded stage, one token row a
+            // thread, into an A slot: high is x with the low 13 mantissa bits
+            // cleared (kind::tf32 uses the top 19 bits of each element), low the
+            // exact rest (rounding instead would leave about 2^-11 relative
+            // error per product, far outside the fp32 tolerance)
+            split_ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(rbar, 0, a.wait_ns));
+            const int row = 32 * (warp & 3) + lane;
+            const uint32_t slots = tmem + a_col + ((uint32_t)(32 * (warp & 3)) << 16);
+            int s = 0, slot = 0, used = 0, fs = 0;   // fs: the stage of the chunk nslot ago
+            uint32_t phase = 0, fphase = 0;
             for (int c = 0; split_ok && c < nch; c++) {
                 if (I_s[4 + c] == I_s[5 + c]) continue;
-                const int s = k % NS;
-                const bool got = ptx::mbar_wait_bounded(&full[s], (k / NS) & 1, a.wait_ns) && !aborted(misc);
-                if (ptx::named_barrier_or(2, 128, !got)) { split_ok = false; break; }
-                float4 *hi4 = reinterpret_cast<float4 *>(base + s * kStageBytes);
-                float4 *lo4 = reinterpret_cast<float4 *>(base + (NS + s) * kStageBytes);
-#pragma unroll
-                for (int j = 0; j < (int)(kStageBytes / 16 / 128); j++) {
-                    const int q4 = et + 128 * j;
-                    const float4 x = hi4[q4];
-                    const float4 h = tf32_high(x);
-                    lo4[q4] = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+                bool got = ptx::mbar_wait_bounded(&full[s], phase, a.wait_ns);
+                if (used >= nslot) {   // the slot's last chunk has been multiplied
+                    got = ptx::mbar_wait_bounded(&empty[fs], fphase, a.wait_ns) && got;
+                    if (++fs == NS) {
+                        fs = 0;
+                        fphase ^= 1;
+                    }
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor cores
-                ptx::named_barrier(2, 128);
-                if (et == 0) ptx::mbar_arrive(&split[s]);
-                k++;
+                split_ok = __all_sync(0xffffffffu, got && !aborted(misc));
+                if (!split_ok) break;
+                tc5::fence_after();
+                const float4 *x4 = reinterpret_cast<const float4 *>(base + s * kStageBytes + row * 128);
+                uint32_t hi[32], lo[32];
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const float4 x = x4[j ^ (row & 7)];
+                    const float4 h = tf32_high(x);
+                    hi[4 * j] = __float_as_uint(h.x);
+                    hi[4 * j + 1] = __float_as_uint(h.y);
+                    hi[4 * j + 2] = __float_as_uint(h.z);
+                    hi[4 * j + 3] = __float_as_uint(h.w);
+                    lo[4 * j] = __float_as_uint(x.x - h.x);
+                    lo[4 * j + 1] = __float_as_uint(x.y - h.y);
+                    lo[4 * j + 2] = __float_as_uint(x.z - h.z);
+                    lo[4 * j + 3] = __float_as_uint(x.w - h.w);
+                }
+                tc5::st32(slots + (uint32_t)(slot * 64), hi);
+                tc5::st32(slots + (uint32_t)(slot * 64 + 32), lo);
+                tc5::st_wait();
+                tc5::fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&split[slot]);
+                used++;
+                if (++s == NS) {
+                    s = 0;
+                    phase ^= 1;
+                }
+                if (++slot == nslot) slot = 0;
             }
-            if (!split_ok && et == 0) {
+            if (!split_ok && lane == 0) {
                 set_status(a.status, DEV_TIMEOUT);
                 atomicExch(&misc[0], 1);
             }
@@ -395,7 +442,7 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
         // partials to the workspace directly.
         constexpr uint32_t kGroupBytes = TN * 16 * sizeof(T);
         constexpr uint32_t kRoundBytes = 4 * kGroupBytes;
-        static_assert(2 * kRoundBytes <= (F32 ? 2 : 1) * NS * kStageBytes, "Y staging exceeds the X ring");
+        static_assert(2 * kRoundBytes <= (F32 ? kTcYStaging : kTcStages * kStageBytes), "Y staging exceeds the ring");
         int round = 0;
         for (int c0 = 0; c0 < g_count * R && !stop; c0 += 64, round++) {
             unsigned char *buf = base + (round & 1) * kRoundBytes;
@@ -591,11 +638,19 @@ uint32_t tmem_cols_for(int cols) {
     return n;
 }
 
+constexpr size_t kSmemPerSm = 233472;   // 228 KB, of which 1 KB is reserved per CTA
+
+// Shared memory of a CTA beside the ring: record, bias, barriers, item table, alignment.
+size_t tc_fixed_bytes(int R, int G, size_t ibytes, int ns) {
+    return ((ibytes + 15) & ~size_t(15)) + (((size_t)G * R * 4 + 15) & ~size_t(15)) + (3 * ns + 2) * 8 +
+           (4 + 6 * 32) * 4 + 1024;
+}
+
 // Kernel arguments and dynamic shared-memory bytes of one product at task
 // size G (nothing to launch: smem = 0).
 template <typename T, int R>
 cudaError_t make_tc_args(const LaunchArgs &la, int G, TcArgs &a, uint32_t &smem) {
-    constexpr int NS = TcCfg<T>::NS, KC = TcCfg<T>::KC;
+    constexpr int KC = TcCfg<T>::KC;
     const Schedule &sc = *la.sc;
     const int n_items = (int)sc.items.size();
     smem = 0;
@@ -617,16 +672,19 @@ cudaError_t make_tc_args(const LaunchArgs &la, int G, TcArgs &a, uint32_t &smem)
     a.M = sc.M;
     a.C = sc.ex_C;   // the execution block width (64 for re-blocked narrow blocks)
     a.nchunks = (int)((sc.K + KC - 1) / KC);
-    a.w_off = (sizeof(T) == 4 ? 2 : 1) * NS * kStageBytes;
-    a.trec_smem = a.w_off + NS * a.wstage;
+    const TcRing ring = tc_ring(R, G, a.wstage, sc.tc.task_ibytes[gidx], sc.dt);
+    const int NS = a.ns = ring.ns;
+    a.nslot = ring.nslot;
+    a.w_off = NS * kStageBytes;
+    a.trec_smem = ring.bytes;
     a.bias_off = a.trec_smem + (uint32_t)((sc.tc.task_ibytes[gidx] + 15) & ~size_t(15));
     a.bar_off = a.bias_off + (uint32_t)(((size_t)G * R * 4 + 15) & ~size_t(15));
     a.misc_off = a.bar_off + (3 * NS + 2) * 8;
-    a.tmem_cols = tmem_cols_for(G * R);
+    a.tmem_cols = ring.tmem_cols;
     a.wait_ns = la.wait_ns;
     a.stall_chunk = la.stall_chunk;
     smem = a.misc_off + (4 + 6 * 32) * 4 + 1024;
-    if (smem > (uint32_t)kTcMaxSmem || G * R > kTcTmemCols) return cudaErrorInvalidConfiguration;
+    if (smem > (uint32_t)kTcMaxSmem || ring.ns < 1) return cudaErrorInvalidConfiguration;
     return encode_y<T>(la.Y, la.N, sc.M, &a.ymap);
 }
 
@@ -725,18 +783,44 @@ int tc_g_index(int G) {
     return 0;
 }
 
+// The ring of a task size. bf16: three stages. fp32: two A slots in tensor
+// memory where they and the accumulators fit half of it, with as many stages as
+// let two CTAs share an SM; else four slots and up to kTcStagesF32 stages.
+TcRing tc_ring(int R, int G, size_t wbytes, size_t ibytes, bsr_dtype_t dt) {
+    const size_t wstage = (wbytes + 15) & ~size_t(15), stage = kStageBytes + wstage;
+    TcRing r = {};
+    if (dt == BSR_BF16) {
+        r.ns = G * R <= kTcTmemCols ? kTcStages : 0;
+        r.tmem_cols = tmem_cols_for(G * R);
+        r.bytes = (uint32_t)(kTcStages * stage);
+        return r;
+    }
+    const size_t fixed = tc_fixed_bytes(R, G, ibytes, kTcStagesF32);
+    const int acc = std::max(32, G * R);
+    auto stages = [&](size_t room) { return room > fixed ? (int)std::min<size_t>(kTcStagesF32, (room - fixed) / stage) : 0; };
+    if (acc + 2 * 64 <= kTcTmemCols / 2 && stages(kSmemPerSm / 2 - 1024) >= 2) {
+        r.ns = stages(kSmemPerSm / 2 - 1024);
+        r.nslot = 2;
+    } else if (acc + 2 * 64 <= kTcTmemCols) {
+        r.ns = stages(kTcMaxSmem);
+        r.nslot = acc + 4 * 64 <= kTcTmemCols && r.ns >= 4 ? 4 : 2;
+        if (r.ns < 2) r.ns = 0;
+    }
+    r.tmem_cols = tmem_cols_for(acc + r.nslot * 64);
+    r.bytes = (uint32_t)std::max<size_t>(r.ns * stage, kTcYStaging);
+    return r;
+}
+
 size_t tc_smem_bytes(int R, int G, size_t wstage, size_t ibytes, bsr_dtype_t dt) {
-    const size_t ring = dt == BSR_F32 ? (size_t)2 * kTcStagesF32 * kStageBytes : (size_t)kTcStages * kStageBytes;
-    const int ns = dt == BSR_F32 ? kTcStagesF32 : kTcStages;
-    return ring + ns * ((wstage + 15) & ~size_t(15)) + ((ibytes + 15) & ~size_t(15)) +
-           (((size_t)G * R * 4 + 15) & ~size_t(15)) + (3 * ns + 2) * 8 + (4 + 6 * 32) * 4 + 1024;
+    const TcRing r = tc_ring(R, G, wstage, ibytes, dt);
+    if (r.ns < 1) return (size_t)kTcMaxSmem + 1;   // does not fit
+    return r.bytes + tc_fixed_bytes(R, G, ibytes, r.ns);
 }
 
 int tc_ctas_per_sm(int R, int G, size_t wbytes, size_t ibytes, bsr_dtype_t dt) {
-    constexpr size_t kSmemPerSm = 233472;   // 228 KB, of which 1 KB is reserved per CTA
     const size_t per_cta = tc_smem_bytes(R, G, wbytes, ibytes, dt) + 1024;
     const int by_smem = (int)(kSmemPerSm / per_cta);
-    const int by_tmem = kTcTmemCols / (int)tmem_cols_for(G * R);
+    const int by_tmem = kTcTmemCols / (int)std::max<uint32_t>(32, tc_ring(R, G, wbytes, ibytes, dt).tmem_cols);
     const int bound = 2;   // the kernel's __launch_bounds__
     return std::max(1, std::min(bound, std::min(by_smem, by_tmem)));
 }

@@ -14,8 +14,7 @@ namespace bsr {
 constexpr int kTcTokens = 128;         // tokens per CTA = MMA M = TMEM lanes
 constexpr int kTcChunk = 64;           // K columns per ring stage (one 128-byte swizzle row of bf16)
 constexpr int kTcStages = 3;           // ring depth (bf16; two CTAs per SM)
-constexpr int kTcStagesF32 = 2;        // ring depth (fp32: each stage has a twin for the low parts; two
-                                       // stages let two CTAs share an SM and overlap their stage latencies)
+constexpr int kTcStagesF32 = 6;        // most ring stages (fp32; tc_ring)
 constexpr int kTcMaxSmem = 232448;     // 227 KB
 constexpr int kTcpIssuers = 4;         // MMA-issuing threads of the persistent kernel (one per warp)
 constexpr int kTcpProgHeader = 16;     // ints before a stage program's MMAs: per issuer its first MMA, and the end
@@ -79,6 +78,11 @@ inline int64_t tc_pad4(int64_t n) { return (n + 3) & ~int64_t(3); }
 // Block shapes the tensor-core kernels run; MK: the weight's elements (M K).
 bool tc_supports(int R, int C, bsr_dtype_t dt, int64_t K, int64_t MK);
 int tc_g_index(int G);
+struct TcRing {
+    int ns, nslot;        // stages (0: does not fit); fp32: A slots in tensor memory
+    uint32_t bytes, tmem_cols;
+};
+TcRing tc_ring(int R, int G, size_t wbytes, size_t ibytes, bsr_dtype_t dt);
 size_t tc_smem_bytes(int R, int G, size_t wbytes, size_t ibytes, bsr_dtype_t dt);
 // CTAs of the tensor-core kernel that fit one SM at once (shared memory,
 // tensor memory and the kernel's launch bound), for a task size's footprint.
