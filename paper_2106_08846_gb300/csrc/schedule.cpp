@@ -740,7 +740,10 @@ int fusion_class(const Schedule &sc, int64_t N, int *G) {
     }
     if (choose_tcp(sc, N) < 0) {
         if ((*G = choose_dense(sc, N)) > 0) return kDenseClass + (*G & kDnPair);
-        if ((*G = choose_xcol(sc, N)) >= 0) return kXcolClass + *G;
+        if (choose_xcol(sc, N)) {
+            *G = 0;
+            return kXcolClass;
+        }
     }
     if (sc.variant == V_XSTAGE) {
         *G = choose_tasks(sc, N);
@@ -792,7 +795,7 @@ cudaError_t launch_spmm_batch(const LaunchArgs *as, int n) {
             if (e != cudaSuccess) return e;
             continue;
         }
-        cudaError_t e = key >= kXcolClass ? launch_xcol(grp.data(), gs.data(), m) : tc ? (m == 1 ? launch_tc(grp[0], gs[0]) : launch_tc_batch(grp.data(), gs.data(), m))
+        cudaError_t e = key >= kXcolClass ? launch_xcol(grp.data(), m) : tc ? (m == 1 ? launch_tc(grp[0], gs[0]) : launch_tc_batch(grp.data(), gs.data(), m))
                            : (m == 1 ? launch_xstage(grp[0], gs[0]) : launch_xstage_batch(grp.data(), gs.data(), m));
         if (e != cudaSuccess) return e;
         for (const LaunchArgs &a : grp)
@@ -806,11 +809,10 @@ cudaError_t launch_spmm(const LaunchArgs &a) {
     if (gG >= 0) return launch_gk(a, gG);   // every block row is an item: nothing to reduce
     cudaError_t e;
     const int tG = a.sc->variant == V_TC ? choose_tcp(*a.sc, a.N) : -1;
-    const int xG = tG < 0 ? choose_xcol(*a.sc, a.N) : -1;
     if (tG >= 0)
         e = launch_tcp(a, tG);
-    else if (xG >= 0)
-        e = launch_xcol(&a, &xG, 1);
+    else if (choose_xcol(*a.sc, a.N))
+        e = launch_xcol(&a, 1);
     else if (const int g = choose_dense(*a.sc, a.N); g > 0)
         return launch_dense(&a, &g, 1);   // no split rows, no reduce pass
     else if (a.sc->variant == V_TC)

@@ -16,22 +16,30 @@
 //
 // Persistent: one CTA per SM walks units (task of G items, token tile). The
 // producer warp streams X chunks (two TMA boxes of 32 columns) and, beside
-// each, the items' packed columns of that chunk through a ring; every consumer
-// warp waits for chunks, works through its columns and frees them, and goes on
-// to the next unit when its own tile is stored: no barrier over all warps.
-// Items of a task are neighbours in length, so warps stay within the ring of
-// one another.
+// each, the task's packed columns of that chunk (one bulk copy; one for each item
+// took the producer longer than the warps: with 8 items a task, 2048 x 2048 at 70%,
+// 2000 tokens 128 us, then 120) through a ring; every consumer warp waits for
+// chunks, works through its columns and frees them, and goes on to the next unit
+// when its own tile is stored: no barrier over all warps.
+// Which items make a task and how many tokens a tile changes no output's bits, so a
+// launch chooses both for all of its products together: few items a task spread a
+// small call over the SMs (768 x 768 at 50%, 1024 tokens 43 -> 30 us), 48 products
+// of 1024 tokens fill the GPU with larger ones (plan of 48 weights at 50 to 95%, of
+// which those at 50% run here, 616 -> 486 us).
+// Items of a task are neighbours in length, so warps stay within the ring of one
+// another.
 //
 // So that an output is not one long chain of additions, a warp adds its tile to
-// a running sum after every segment of chunks (about 52 columns). Registers and
-// shared memory are full; the sums live in tensor memory, which nothing else
-// uses here: a warp reaches 32 lanes of it, so up to three tiles of 112 columns.
+// a running sum after every segment of chunks (at most about 40 columns, or one
+// chunk). A tile of 64 tokens has registers for a second set; for the larger ones
+// registers and shared memory are full and the sums live in tensor memory, which
+// nothing else uses here: a warp reaches 32 lanes of it, so up to three tiles of
+// 112 columns. An addition there costs the largest tile about 1900 cycles (it
+// spills a dozen registers around it): one chain per output would run 1024 x 1024
+// at 90%, 16384 tokens in 86 us where this takes 101, with a relative error of
+// 1.8e-7 instead of 1.15e-7 (the per-task kernel's: 1.33e-7).
 //
-// (With 112 accumulators the largest tile spills a dozen registers around that
-// addition: one chain per output runs 85.5 us where this takes 98.1, but its
-// relative error at 102 columns is 1.8e-7 instead of 1.3e-7, at 512 4.0e-7.)
-//
-// Measured, with the per-task kernel beside it: see choose_xcol.
+// Measured, with the per-task kernel beside it: choose_xcol.
 //
 // Every wait is bounded by the global timer; a timeout sets the device status
 // word, stops the CTA's roles, lets the issued copies land and returns.
@@ -59,7 +67,7 @@ constexpr uint32_t kTileCols = 8 * kXcTT[kXcTileSizes - 1];   // of the largest 
 constexpr uint64_t kDrainNs = 200000000ull;
 
 struct XcArgs {
-    const int32_t *table;        // per item and chunk: the packed chunk's start / 16, in order (and the end)
+    const int32_t *table;        // per chunk and item: the packed chunk's start / 16, in order (and the end)
     const unsigned char *packed;
     const Item *items;
     const float *bias;
@@ -76,8 +84,7 @@ struct XcArgs {
 template <int MAXB>
 struct XcBatch {
     int n, ns;
-    uint32_t stage_bytes;   // a stage: two X boxes, then the items' packed chunks, item_bytes apart
-    uint32_t item_bytes;
+    uint32_t stage_bytes;   // a stage: two X boxes, then the items' packed chunks
     int nch;
     int64_t N;
     unsigned start[MAXB + 1];
@@ -100,6 +107,12 @@ __device__ __forceinline__ f2_t ffma2(f2_t a, f2_t b, f2_t c) {
     return d;
 }
 
+__device__ __forceinline__ f2_t fadd2(f2_t a, f2_t b) {
+    f2_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 __device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
 __device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
 __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, uint64_t limit_ns, const int *flag) {
@@ -111,6 +124,13 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, ui
     }
 }
 
+// The unit a CTA takes in its k-th turn (>= `units`: none). Several products come
+// longest first: to and fro over the grid, so that a CTA's units add up to the
+// same as another's.
+__device__ __forceinline__ unsigned turn_unit(unsigned k, int products) {
+    return k * gridDim.x + (products > 1 && k & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+}
+
 struct Unit {
     int i0, n;    // first item, items
     int64_t n0;   // first token
@@ -119,9 +139,13 @@ template <int TT>
 __device__ __forceinline__ Unit unit_at(const XcArgs &a, unsigned v) {
     Unit u;   // the tasks of a token tile side by side: their reads of X meet in L2
     const unsigned tile = v / (unsigned)a.n_tasks;
-    const int task = (int)(v - tile * (unsigned)a.n_tasks);
-    u.i0 = xcol_first(task, a.n_tasks, a.n_items);
-    u.n = xcol_first(task + 1, a.n_tasks, a.n_items) - u.i0;
+    unsigned task = v - tile * (unsigned)a.n_tasks;
+    // where the grid is whole tiles, a CTA would have the same task (the longest,
+    // say) in every turn: another one in each
+    if (a.n_tasks > 1 && gridDim.x % (unsigned)a.n_tasks == 0)
+        task = (task + tile / (gridDim.x / (unsigned)a.n_tasks)) % (unsigned)a.n_tasks;
+    u.i0 = xcol_first((int)task, a.n_tasks, a.n_items);
+    u.n = xcol_first((int)task + 1, a.n_tasks, a.n_items) - u.i0;
     u.n0 = (int64_t)tile * (8 * TT);
     return u;
 }
@@ -155,6 +179,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
     __shared__ uint64_t full[kStagesMax], empty[kStagesMax];
     __shared__ int stop;
     __shared__ uint32_t tmem_s;
+    __shared__ uint32_t place[kStagesMax][NW];   // where a stage's items begin
     const int ns = b.ns;
     const uint32_t stage_bytes = b.stage_bytes;
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -179,46 +204,44 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
         }
     };
     const int nch = b.nch;
-    unsigned u = blockIdx.x;
     int h = 0, s = 0;
 
     if (warp == NW) {
-        // ---------------- producer: lane g copies item g's columns
+        // ---------------- producer
         uint32_t phase = 1;   // the parity of `empty` that a first use of a stage passes at once
         uint32_t stalled = 0; // test hook: stages whose load was left out
         int issued = 0;
         bool ok = true, waited = false;
         if (elected) ptx::prefetch_tensormap(&xmap);
-        for (; ok && u < units; u += gridDim.x) {
+        for (unsigned k = 0, u; ok && k * gridDim.x < units; k++) {
+            if ((u = turn_unit(k, b.n)) >= units) break;
             while (u >= b.start[h + 1]) h++;
             const XcArgs &a = b.args[h];
             const Unit un = unit_at<TT>(a, u - b.start[h]);
-            const int32_t *tab = a.table + (int64_t)(un.i0 + min(lane, un.n - 1)) * nch;
+            // (the task's packed chunk is one range; lane g knows where item g's begins)
+            const int32_t *tab = a.table + un.i0 + min(lane, un.n);
             int at = __ldg(tab);
-            auto load_w = [&](int c, int st, int from, int to) {
-                const uint32_t bytes = lane < un.n ? (uint32_t)(to - from) * 16 : 0;
-                const uint32_t all = __reduce_add_sync(0xffffffffu, bytes);
-                if (elected) ptx::mbar_arrive_expect_tx(&full[st], 2 * TT * 1024 + all);
+            auto load_w = [&](int st, int v) {
+                const int from = __shfl_sync(0xffffffffu, v, 0), to = __shfl_sync(0xffffffffu, v, un.n);
+                if (lane < NW) place[st][lane] = (uint32_t)(v - from) * 16;
                 __syncwarp();
-                if (bytes)
-                    ptx::bulk_load(base + (size_t)st * stage_bytes + kX + lane * b.item_bytes,
-                                   a.packed + (int64_t)from * 16, bytes, &full[st]);
+                if (elected) {
+                    const uint32_t bytes = (uint32_t)(to - from) * 16;
+                    ptx::mbar_arrive_expect_tx(&full[st], 2 * TT * 1024 + bytes);
+                    ptx::bulk_load(base + (size_t)st * stage_bytes + kX, a.packed + (int64_t)from * 16, bytes, &full[st]);
+                }
                 __syncwarp();
             };
             // the first columns do not depend on earlier kernels
             const int ahead = waited ? 0 : min(ns, nch);
             if (!waited) {
-                int from = at;
-                for (int c = 0; c < ahead; c++) {
-                    const int to = __ldg(tab + c + 1);
-                    if (c != a.stall_chunk) load_w(c, c, from, to);
-                    from = to;
-                }
+                for (int c = 0; c < ahead; c++)
+                    if (c != a.stall_chunk) load_w(c, __ldg(tab + (int64_t)c * a.n_items));
                 ptx::pdl_wait();   // X may be an earlier kernel's output
                 waited = true;
             }
             for (int c = 0; c < nch; c++) {
-                const int next = __ldg(tab + c + 1);
+                const int next = c + 1 < nch ? __ldg(tab + (int64_t)(c + 1) * a.n_items) : 0;
                 // (the stages loaded ahead are free, and their X tiles always
                 // follow: a barrier phase is never left half loaded)
                 if (c >= ahead) {
@@ -232,7 +255,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                 if (c == a.stall_chunk) {   // never loaded: its consumers time out
                     stalled |= 1u << s;
                 } else {
-                    if (c >= ahead) load_w(c, s, at, next);
+                    if (c >= ahead) load_w(s, at);
                     if (elected) {
                         unsigned char *st = base + (size_t)s * stage_bytes;
                         ptx::tma_load_2d(st, &xmap, c * kXcChunk, (int32_t)un.n0, &full[s]);
@@ -257,7 +280,8 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
         const uint32_t tgx = (uint32_t)tg << 4;
         uint32_t phase = 0;
         bool ok = true;
-        for (; ok && u < units; u += gridDim.x) {
+        for (unsigned k = 0, u; ok && k * gridDim.x < units; k++) {
+            if ((u = turn_unit(k, b.n)) >= units) break;
             while (u >= b.start[h + 1]) h++;
             const XcArgs &a = b.args[h];
             const bool has = warp < unit_at<TT>(a, u - b.start[h]).n;
@@ -266,24 +290,37 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
             for (int i = 0; i < TT / 2; i++)
 #pragma unroll
                 for (int j = 0; j < 8; j++) acc[i][j] = 0ull;
+            constexpr bool kRegSums = TT == 8;   // the running sums fit the registers
+            f2_t total[kRegSums ? TT / 2 : 1][8];
+            if constexpr (kRegSums) {
+#pragma unroll
+                for (int i = 0; i < TT / 2; i++)
+#pragma unroll
+                    for (int j = 0; j < 8; j++) total[i][j] = 0x8000000080000000ull;   // -0: adds nothing, to any value
+            }
             auto sums = [&]() {   // this warp's running sums
                 return tmem_s + ((uint32_t)(32 * (warp & 3)) << 16) +
                        (uint32_t)(warp >> 2) * kTileCols;
             };
             auto add_sums = [&]() {   // acc += the running sums
                 const uint32_t at = sums();
+                tc5::st_wait();
+                // (as many loads at once as there are registers)
+                constexpr int L = TT == 12 ? 16 : 8;
 #pragma unroll
-                for (int k = 0; k < 8 * TT; k += 8) {
-                    uint32_t v[8];
-                    tc5::ld8(at + k, v);
+                for (int k = 0; k < 8 * TT; k += L) {
+                    uint32_t v[L / 8][8];
+#pragma unroll
+                    for (int l = 0; l < L / 8; l++) tc5::ld8(at + k + 8 * l, v[l]);
                     tc5::ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        asm volatile("" : "+r"(v[2 * e]), "+r"(v[2 * e + 1]));   // no use moves above the wait
+                    for (int e = 0; e < L / 2; e++) {
+                        uint32_t &v0 = v[e / 4][2 * (e % 4)], &v1 = v[e / 4][2 * (e % 4) + 1];
+                        asm volatile("" : "+r"(v0), "+r"(v1));   // no use moves above the wait
                         f2_t &t = acc[(k / 2 + e) / 8][(k / 2 + e) % 8];
                         float even, odd;
                         unpack2(t, even, odd);
-                        t = pack2(even + __uint_as_float(v[2 * e]), odd + __uint_as_float(v[2 * e + 1]));
+                        t = pack2(even + __uint_as_float(v0), odd + __uint_as_float(v1));
                     }
                 }
             };
@@ -299,7 +336,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                 if (has) {
                     const unsigned char *st = base + (size_t)s * stage_bytes;
                     const unsigned char *xs = st + tg * 128;
-                    const int4 *hdr = reinterpret_cast<const int4 *>(st + kX + warp * b.item_bytes);
+                    const int4 *hdr = reinterpret_cast<const int4 *>(st + kX + place[s][warp]);
                     int n = hdr->x;   // columns; then their places, then their weights
                     const int4 *oc = hdr + 1;
                     const float *w = reinterpret_cast<const float *>(oc + ((n + 3) >> 2)) + 4 * rg;
@@ -325,7 +362,16 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                     s = 0;
                     phase ^= 1;
                 }
-                if (c + 1 == c1 && c1 < nch) {
+                if (kRegSums && c + 1 == c1 && c1 < nch) {
+#pragma unroll
+                    for (int i = 0; i < (kRegSums ? TT / 2 : 1); i++)
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            total[i][j] = fadd2(acc[i][j], total[i][j]);
+                            acc[i][j] = 0ull;
+                        }
+                    c1 += a.seg;
+                } else if (!kRegSums && c + 1 == c1 && c1 < nch) {
                     if (c1 > a.seg) add_sums();
                     const uint32_t at = sums();
 #pragma unroll
@@ -342,12 +388,18 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                         }
                         tc5::st8(at + k, v);
                     }
-                    tc5::st_wait();
                     c1 += a.seg;
                 }
             }
             if (!ok) break;
-            if (nch > a.seg) add_sums();
+            if constexpr (kRegSums) {
+#pragma unroll
+                for (int i = 0; i < TT / 2; i++)
+#pragma unroll
+                    for (int j = 0; j < 8; j++) acc[i][j] = fadd2(acc[i][j], total[i][j]);
+            } else if (nch > a.seg) {
+                add_sums();
+            }
             ptx::pdl_wait();   // the bias, Y and the workspace may be an earlier kernel's
             if (!has) continue;
             // (the unit once more: the registers are the columns' until here)
@@ -434,13 +486,13 @@ cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
 }
 
 template <int MAXB, int TT>
-cudaError_t launch(const LaunchArgs *las, int n) {
+cudaError_t launch(const LaunchArgs *las, int n, int G) {
     XcBatch<MAXB> b;
     b.n = 0;
     b.N = las[0].N;
     const int64_t K = las[0].sc->K;
     b.nch = (int)((K + kXcChunk - 1) / kXcChunk);
-    b.item_bytes = 0;
+    uint32_t item_bytes = 0;
     int64_t units = 0;
     for (int i = 0; i < n; i++) {
         const LaunchArgs &la = las[i];
@@ -457,19 +509,19 @@ cudaError_t launch(const LaunchArgs *las, int n) {
         a.M = sc.M;
         a.wait_ns = la.wait_ns;
         a.n_items = (int)sc.items.size();
-        a.n_tasks = (a.n_items + NW - 1) / NW;
+        a.n_tasks = (a.n_items + G - 1) / G;
         a.seg = sc.xc.seg;
         a.tiles = (unsigned)((la.N + 8 * TT - 1) / (8 * TT));
         a.stall_chunk = la.stall_chunk;
         b.start[b.n] = (unsigned)units;
         units += (int64_t)a.tiles * a.n_tasks;
-        b.item_bytes = std::max(b.item_bytes, sc.xc.item_bytes);
+        item_bytes = std::max(item_bytes, sc.xc.item_bytes);
         b.n++;
         if (units > INT32_MAX) return cudaErrorInvalidConfiguration;
     }
     if (b.n == 0) return cudaSuccess;
     b.start[b.n] = (unsigned)units;
-    b.stage_bytes = xcol_stage_bytes(b.item_bytes);
+    b.stage_bytes = xcol_stage_bytes(item_bytes, G);
     b.ns = (int)std::min<uint32_t>(kXcStagesMax, kXcRoom / b.stage_bytes);
     if (b.ns < 1) return cudaErrorInvalidConfiguration;
     auto enc = encode_fn();
@@ -490,8 +542,8 @@ cudaError_t launch(const LaunchArgs *las, int n) {
 }
 
 template <int TT>
-cudaError_t launch_n(const LaunchArgs *las, int n) {
-    return n == 1 ? launch<1, TT>(las, 1) : launch<kXcBatchMax, TT>(las, n);
+cudaError_t launch_n(const LaunchArgs *las, int n, int G) {
+    return n == 1 ? launch<1, TT>(las, 1, G) : launch<kXcBatchMax, TT>(las, n, G);
 }
 
 }  // namespace
@@ -509,13 +561,21 @@ cudaError_t pack_xcol_data(const Schedule &sc, const void *data, void *packed, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_xcol(const LaunchArgs *las, const int *tiles, int n) {
+cudaError_t launch_xcol(const LaunchArgs *las, int n) {
     if (n <= 0) return cudaSuccess;
     if (n > kXcBatchMax) return cudaErrorInvalidValue;
-    switch (kXcTT[tiles[0]]) {
-        case 8: return launch_n<8>(las, n);
-        case 12: return launch_n<12>(las, n);
-        case 14: return launch_n<14>(las, n);
+    // the longest units first
+    LaunchArgs sorted[kXcBatchMax];
+    const Schedule *scs[kXcBatchMax];
+    std::copy(las, las + n, sorted);
+    auto length = [](const LaunchArgs &la) { return (double)la.sc->nnzb / (double)std::max<size_t>(la.sc->items.size(), 1); };
+    std::stable_sort(sorted, sorted + n, [&](const LaunchArgs &x, const LaunchArgs &y) { return length(x) > length(y); });
+    for (int i = 0; i < n; i++) scs[i] = sorted[i].sc;
+    const XcShape sh = xcol_shape(scs, n, las[0].N);
+    switch (kXcTT[sh.tile]) {
+        case 8: return launch_n<8>(sorted, n, sh.G);
+        case 12: return launch_n<12>(sorted, n, sh.G);
+        case 14: return launch_n<14>(sorted, n, sh.G);
     }
     return cudaErrorInvalidConfiguration;
 }

@@ -23,9 +23,10 @@ constexpr int kXcBatchMax = 64;        // products in one fused launch
 constexpr int kXcTileSizes = 3;
 constexpr int kXcTT[kXcTileSizes] = {8, 12, 14};   // tokens per lane; 8 times as many per unit
 
-// A task is up to kXcWarps items (block rows, or pieces of them), one per warp.
-// An item's columns are packed chunk by chunk (64 columns of K), one bulk copy
-// each:
+// A task is up to kXcWarps items (block rows, or pieces of them), one per warp; a
+// launch chooses how many, and its tile: neither changes an output's bits.
+// Columns are packed chunk by chunk (64 columns of K) and in a chunk item by item,
+// so that a task's part of a chunk is one bulk copy:
 //   int32 n, 0, 0, 0   columns in this chunk
 //   int32 [n]          byte offsets of theirs in the X tile, padded to 4
 //   float [n][32]      their weights
@@ -34,11 +35,11 @@ struct XcPlan {
     int64_t off = -1, bytes = 0;       // place in the handle's packed buffer
     uint32_t item_bytes = 0;           // largest packed chunk of an item
     int seg = 1;                       // chunks per segment (one chain of additions)
-    std::vector<int32_t> table;        // per item and chunk: its start / 16 (and the end)
+    std::vector<int32_t> table;        // per chunk and item: its start / 16 (and the end)
     std::vector<int32_t> ints;         // (place / 4 bytes, value) of the packed buffer's integers
     std::vector<int32_t> src;          // per column: its weights' place / 4 bytes, its block
     int32_t *d_table = nullptr, *d_ints = nullptr, *d_src = nullptr;
-    mutable std::atomic<uint64_t> last{0};   // choose_xcol's last answer
+    mutable std::atomic<uint64_t> last{0};   // choose_xcol's last answer: N << 16 | (yes: 1)
 };
 
 // The first item of task t of `tasks`: equal counts, in item order.
@@ -48,18 +49,23 @@ __host__ __device__
 inline int xcol_first(int t, int tasks, int items) { return (int)((int64_t)t * items / tasks); }
 
 // A ring stage: the X tile's two boxes, then the items' packed chunks.
-inline uint32_t xcol_stage_bytes(uint32_t item_bytes) { return (2 * kXcBox + kXcWarps * item_bytes + 1023) & ~1023u; }
+inline uint32_t xcol_stage_bytes(uint32_t item_bytes, int G) { return (2 * kXcBox + G * item_bytes + 1023) & ~1023u; }
 
 struct Schedule;
 struct LaunchArgs;
 
 // Fills sc.xc (after the items); returns the packed buffer's new end.
 int64_t plan_xcol(Schedule &sc, int64_t base);
-// Tile size of a call of N tokens (index into kXcTT), or -1: the kernel does
-// not run it. Products with equal answers can share a grid.
-int choose_xcol(const Schedule &sc, int64_t N);
+// Whether the kernel runs a call of N tokens.
+bool choose_xcol(const Schedule &sc, int64_t N);
+// Tile (index into kXcTT) and items per task of one grid of n products.
+struct XcShape {
+    int tile, G;
+    double cycles;   // the model's, of the busiest SM
+};
+XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N);
 cudaError_t pack_xcol_data(const Schedule &sc, const void *data, void *packed, cudaStream_t s);
-// n products that share X, N, K and the stream (equal tiles): one grid.
-cudaError_t launch_xcol(const LaunchArgs *las, const int *tiles, int n);
+// n products that share X, N, K and the stream: one grid.
+cudaError_t launch_xcol(const LaunchArgs *las, int n);
 
 }  // namespace bsr

@@ -1,6 +1,7 @@
 // Plan and dispatch of the column-list kernel (xcol.h): packed columns, and the
 // tile size of a call.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include "bsr_internal.h"
@@ -26,10 +27,12 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
         pl.ints.push_back((int32_t)place);
         pl.ints.push_back((int32_t)v);
     };
-    for (const Item &it : sc.items) {
-        int32_t p = it.p0;
-        for (int64_t c = 0; c < nch; c++) {
-            int32_t p1 = p;
+    std::vector<int32_t> next(sc.items.size());   // per item: its first block not packed yet
+    for (size_t i = 0; i < sc.items.size(); i++) next[i] = sc.items[i].p0;
+    for (int64_t c = 0; c < nch; c++) {
+        for (size_t i = 0; i < sc.items.size(); i++) {
+            const Item &it = sc.items[i];
+            int32_t &p = next[i], p1 = p;
             while (p1 < it.p1 && sc.indices[(size_t)p1] < (c + 1) * kXcChunk) p1++;
             const int64_t n = p1 - p, vals = at + 4 + ((n + 3) & ~int64_t(3));
             pl.table.push_back((int32_t)(at / 4));
@@ -48,62 +51,103 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     }
     pl.table.push_back((int32_t)(at / 4));
     pl.bytes = at * 4;
-    // equal segments of about 52 columns: outputs are then no further from 64
-    // bits than the per-task kernel's, which shares a row among warps (relative
-    // error at 102 columns in one chain 1.8e-7, at 512 4.0e-7; the per-task
-    // kernel's 1.3e-7)
-    const double mean = (double)sc.nnzb / (double)n_items;
-    const int64_t segs = std::min<int64_t>(nch, std::max<int64_t>(1, (int64_t)(mean / 52.0 + 0.999)));
+    // equal segments of at most 40 columns, or one chunk: outputs are then no
+    // further from 64 bits than the per-task kernel's, which shares a row among
+    // warps (relative errors of ten sizes 0.98 to 1.37e-7, the per-task kernel's 1.16
+    // to 1.43e-7; at 52 columns 1.17 to 1.47e-7, in one chain of 102 1.8e-7)
+    const double per_chunk = (double)sc.nnzb / (double)(n_items * nch);
+    const int64_t most = per_chunk * (double)nch <= 40.0 ? nch : std::max<int64_t>(1, (int64_t)(40.0 / per_chunk));
+    const int64_t segs = (nch + most - 1) / most;
     pl.seg = (int)((nch + segs - 1) / segs);
-    if (2 * xcol_stage_bytes(pl.item_bytes) > kXcRoom) return base;   // a ring of two stages
+    if (2 * xcol_stage_bytes(pl.item_bytes, kXcWarps) > kXcRoom) return base;   // a ring of two stages
     pl.ok = true;
     return pl.off + pl.bytes;
 }
 
-// The tile that minimises the busiest scheduler's cycles, where that beats the
-// per-task kernel. A task's items sit one per warp, ceil(items / 4) to a
-// scheduler; a column takes it about 11.5 TT + 25 cycles, a chunk 100, a unit's
-// stores 60 TT; the per-task kernel pays about 0.85 cycles per unit of its own
-// model. Fitted to (us, this kernel and the per-task one): 1024 x 1024 at 90%,
-// 16384 tokens 98.1 and 123 (TT = 14), 4096 tokens 30.5 and 36.5 (TT = 12); at
-// 50%, 16384 tokens 377 and 659; 768 x 768 at 70%, 3000 tokens 30.4 and 37.3
-// (TT = 8); 1536 x 1536 at 95%, 4000 tokens 47 and 38.9 (few columns per unit:
-// stays); 768 x 768 at 50%, 1024 tokens 43 and 30.5 (24 items leave most SMs
-// idle: stays).
-int choose_xcol(const Schedule &sc, int64_t N) {
-    static const int mode = [] {
-        const char *v = getenv("BSR_XC");
-        return v && *v ? atoi(v) : -1;   // 0: never
-    }();
-    static const int forced = [] {
+// The tile and the items per task that minimise the busiest SM's cycles. A task's
+// items sit one per warp, ceil(items / 4) to a scheduler; a column takes it 11.9
+// TT cycles (a lone warp 24 more, 75 with the largest tile, which spills), a chunk
+// 470, the rest of a unit 385 TT, a running sum in tensor memory 135 TT (one is in
+// the 385), a launch 6000: fitted to 80 times of six sizes,
+// every tile and 3 to 11 items, to 6% of them in the mean. One product's units run in rounds; those
+// of several, longest first and to and fro, fill the SMs to about half of the
+// longest.
+XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N) {
+    static const int forced_tile = [] {
         const char *v = getenv("BSR_XC_TILE");   // index into kXcTT
         return v && *v ? atoi(v) : -1;
     }();
-    const XcPlan &pl = sc.xc;
-    if (!pl.ok || N <= 0 || mode == 0) return -1;
-    if (forced >= 0 && forced < kXcTileSizes) return forced;
-    // (the choice for the last N asked, which is what a steady stream of calls asks again)
-    const uint64_t memo = pl.last.load(std::memory_order_relaxed);
-    if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return (int)(memo & 0xffff) - 1;
-    const int64_t items = (int64_t)sc.items.size(), tasks = (items + kXcWarps - 1) / kXcWarps;
-    const double warps = (double)(((items + tasks - 1) / tasks + 3) / 4);
-    const double columns = (double)sc.nnzb / (double)items, chunks = (double)((sc.K + kXcChunk - 1) / kXcChunk);
-    double per_task = 0.0;
-    choose_tasks(sc, N, &per_task);
-    double best_cost = 0.85 * per_task;
-    int best = -1;
-    for (int ti = 0; ti < kXcTileSizes; ti++) {
-        const int TT = kXcTT[ti];
-        const int64_t units = ((N + 8 * TT - 1) / (8 * TT)) * tasks;
-        const double rounds = (double)((units + sc.sm_count - 1) / sc.sm_count);
-        const double cost = rounds * (warps * columns * (11.5 * TT + 25.0) + 100.0 * chunks + 60.0 * TT) + 4000.0;
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = ti;
+    static const int forced_G = [] {
+        const char *v = getenv("BSR_XC_G");   // items per task
+        return v && *v ? atoi(v) : -1;
+    }();
+    constexpr int kG[] = {kXcWarps, 8, 6, 4, 3, 2, 1};
+    XcShape best = {0, kXcWarps, -1.0};
+    const double sms = (double)scs[0]->sm_count;
+    const double chunks = (double)((scs[0]->K + kXcChunk - 1) / kXcChunk);
+    uint32_t item_bytes = 0;
+    for (int i = 0; i < n; i++) item_bytes = std::max(item_bytes, scs[i]->xc.item_bytes);
+    for (int G : kG) {
+        if (forced_G >= 1 && forced_G <= kXcWarps ? G != forced_G : 2 * xcol_stage_bytes(item_bytes, G) > kXcRoom) continue;
+        for (int ti = 0; ti < kXcTileSizes; ti++) {
+            if (forced_tile >= 0 && forced_tile < kXcTileSizes && ti != forced_tile) continue;
+            const int TT = kXcTT[ti];
+            const int64_t tiles = (N + 8 * TT - 1) / (8 * TT);
+            double sum = 0.0, longest = 0.0;
+            int64_t units = 0;
+            for (int i = 0; i < n; i++) {
+                const int64_t items = (int64_t)scs[i]->items.size(), tasks = (items + G - 1) / G;
+                if (!items) continue;
+                const double warps = (double)(((items + tasks - 1) / tasks + 3) / 4);
+                const double unit = (double)scs[i]->nnzb / (double)items * (11.9 * TT * warps + (warps > 1 ? 0.0 : TT == 14 ? 75.0 : 24.0)) +
+                                    470.0 * chunks + 385.0 * TT +
+                                    (TT > 8 ? 135.0 * TT * std::max(0.0, std::ceil(chunks / scs[i]->xc.seg) - 2.0) : 0.0);
+                units += tiles * tasks;
+                sum += unit * (double)(tiles * tasks);
+                longest = std::max(longest, unit);
+            }
+            const double cost = n == 1 ? longest * std::ceil((double)units / sms)
+                                       : std::max(longest, sum / sms + (units > sms ? 0.5 * longest : 0.0));
+            // (fewer items a task read X more often: for 3% at least)
+            if (best.cycles < 0 || cost < (G == best.G ? 1.0 : 0.97) * best.cycles) best = {ti, G, cost};
         }
     }
-    if (N < (int64_t)1 << 48) pl.last.store((uint64_t)N << 16 | (uint64_t)(best + 1), std::memory_order_relaxed);
+    best.cycles += 6000.0;
     return best;
+}
+
+// Against the per-task kernel, which takes its tasks' work and about 8500 + 4000 / G
+// cycles for each (G items a task; partly filled waves overlap). Measured (us, this
+// kernel and the per-task one): 1024 x 1024 at 90%, 16384 tokens 101 and 123, 4096
+// tokens 29.9 and 36.6; at 50%, 16384 tokens 360 and 656; 2048 x 2048 at 70%, 2000
+// tokens 125 and 203; 4096 x 4096 at 90%, 512 tokens 56 and 101; 768 x 768 at 70%,
+// 3000 tokens 28.3 and 37.4; at 50%, 1024 tokens 30.0 and 30.5. At 80%, 2000 tokens
+// 22.8 and 19.2; at 70%, 1024 tokens 21 and 13.3; 1024 x 768 at 50%, 500 tokens 30
+// and 15.6 (an item's columns are one warp's): these stay.
+bool choose_xcol(const Schedule &sc, int64_t N) {
+    static const int mode = [] {
+        const char *v = getenv("BSR_XC");
+        return v && *v ? atoi(v) : -1;   // 0: never, 1: always
+    }();
+    static const bool forced = [] {
+        const char *v = getenv("BSR_XC_TILE");
+        return v && *v;
+    }();
+    const XcPlan &pl = sc.xc;
+    if (!pl.ok || N <= 0 || mode == 0) return false;
+    if (forced || mode == 1) return true;
+    // (the choice for the last N asked, which is what a steady stream of calls asks again)
+    const uint64_t memo = pl.last.load(std::memory_order_relaxed);
+    if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return memo & 1;
+    const Schedule *one = &sc;
+    double cost = 0.0;
+    const int G = choose_tasks(sc, N, &cost);
+    const int64_t items = (int64_t)sc.items.size(), tasks = (items + G - 1) / G;
+    const double waves = (double)((N + kXsTokens - 1) / kXsTokens * tasks) / (double)sc.sm_count;
+    const double work = (double)sc.nnzb * sc.R * sc.C / (double)tasks;
+    const bool yes = xcol_shape(&one, 1, N).cycles < std::max(1.0, waves) * (8500.0 + 4000.0 / G + work);
+    if (N < (int64_t)1 << 48) pl.last.store((uint64_t)N << 16 | (uint64_t)yes, std::memory_order_relaxed);
+    return yes;
 }
 
 }  // namespace bsr

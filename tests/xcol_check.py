@@ -1,5 +1,6 @@
 """Parity sweep of the column-list SIMT kernel, for a process started with
-BSR_XC_TILE (one token tile). Run by tests/test_gpu_xcol.py in a subprocess;
+BSR_XC_TILE (one token tile) or BSR_XC=1 and perhaps BSR_XC_G (items per
+task). Run by tests/test_gpu_xcol.py in a subprocess;
 exit status 0 when every output is right."""
 import os
 import sys
@@ -51,12 +52,12 @@ def main() -> int:
                 continue
             print(f"{name}: ok", flush=True)
             h.destroy()
-    # two products of one grid are bit for bit the single calls
-    ws = [synth.make_weight("xb", 9200 + i, 416, 512, 32, 1, "f32", s) for i, s in enumerate((50, 90))]
+    # three products of one grid (not by length) are bit for bit the single calls
+    ws = [synth.make_weight("xb", 9200 + i, 416, 512, 32, 1, "f32", s) for i, s in enumerate((50, 90, 70))]
     hs = [bsr.bsr_create(*build_on_gpu(w.W, 32, 1), 32, 1, w.M, w.K) for w in ws]
     X = to_dev(synth.activations(9201, 700, 512, "f32"))
     Ys = [torch.empty((700, w.M), device="cuda") for w in ws]
-    bsr.bsr_spmm_batch(hs, X, None, Ys, 700)
+    bsr.bsr_spmm_batch(hs[::-1], X, None, Ys[::-1], 700)
     fails += sum(not torch.equal(h.spmm(X), Y) for h, Y in zip(hs, Ys))
     # a chunk that is never loaded: bounded waits, BSR_ERR_TIMEOUT, usable context
     os.environ.update(BSR_WAIT_LIMIT_NS="2000000", BSR_TEST_STALL_CHUNK="3")
