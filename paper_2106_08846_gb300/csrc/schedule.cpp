@@ -285,7 +285,7 @@ void plan_tc(Schedule &sc) {
         off.clear();
         order.clear();
         stack.clear();
-        sc.tc.task_cost_max[gi] = 0;
+        sc.tc.task_cost_max[gi] = sc.tc.task_chunks_max[gi] = 0;
         sc.tc.stacks[gi] = 0;
         size_t wmax = 0, imax = 0, swmax = 0;
         const int64_t n_tasks = (n_items + G - 1) / G;
@@ -339,8 +339,10 @@ void plan_tc(Schedule &sc) {
             }
             // stacks, and the task's MMA cost
             double cost = 0.0;
+            int64_t visited = 0;
             for (int64_t c = 0; c < nch; c++) {
                 std::vector<int32_t> &pc = per_chunk[(size_t)c];
+                visited += !pc.empty();
                 bool st = can_stack && g_count >= 2 && g_count * sc.R <= 256 && (int)pc.size() == g_count;
                 for (int g = 0; st && g < g_count; g++)
                     st = ((pc[(size_t)g] >> 2) & 31) == g && (pc[(size_t)g] & 3) == (pc[0] & 3) &&
@@ -356,6 +358,7 @@ void plan_tc(Schedule &sc) {
                 for (int g = 0; g < (int)pc.size(); g++) stack.push_back(st ? (g << 16) | g_count : 1);
             }
             sc.tc.task_cost_max[gi] = std::max(sc.tc.task_cost_max[gi], (int64_t)std::ceil(cost));
+            sc.tc.task_chunks_max[gi] = std::max(sc.tc.task_chunks_max[gi], visited);
             for (int g = 0; g < g_count; g++) {
                 const Item &it = sc.items[(size_t)mem[(size_t)g]];
                 rec[items_at + 4 * (size_t)g + 0] = it.row;
@@ -697,7 +700,13 @@ int choose_tasks(const Schedule &sc, int64_t N, double *cost_out) {
 // barriers, work list, first stage round trip, epilogue: several microseconds
 // in per-CTA phase stamps) is counted as kOverheadMma MMA units, a
 // conservative weight: at 32 the model preferred five waves of two-row tasks
-// to three waves of four-row tasks on Zipf rows, measured 9% slower.
+// to three waves of four-row tasks on Zipf rows, measured 9% slower. fp32 counts
+// its chunks (copy, split and MMAs in turn: about 700 cycles, 30 units) and the
+// accumulator columns its epilogue reads beside a fixed cost, more of it where no
+// second CTA hides it; on 22 sizes this takes the fastest task size of each.
+// Without the chunks 16x16 of 1024 x 1024 took tasks of four rows, which read X
+// twice as often as eight: at 16384 tokens and 50% 179 us instead of 157, at 70%
+// 149 instead of 127.
 int choose_tc_tasks(const Schedule &sc, int64_t N, double *cost_out) {
     static const int forced = [] {
         const char *v = getenv("BSR_TC_G");
@@ -715,10 +724,13 @@ int choose_tc_tasks(const Schedule &sc, int64_t N, double *cost_out) {
         const int G = kTcG[gi];
         if (!fits(G)) continue;
         const int64_t ctas = tiles * (int64_t)sc.tc.rec_off[gi].size();
-        const int64_t slots = (int64_t)sc.sm_count *
-                              tc_ctas_per_sm(sc.ex_R, G, sc.tc.task_wbytes[gi], sc.tc.task_ibytes[gi], sc.dt);
+        const int per_sm = tc_ctas_per_sm(sc.ex_R, G, sc.tc.task_wbytes[gi], sc.tc.task_ibytes[gi], sc.dt);
+        const int64_t slots = (int64_t)sc.sm_count * per_sm;
         const double waves = (double)((ctas + slots - 1) / slots);
-        const double cost = waves * (kOverheadMma + (double)sc.tc.task_cost_max[gi]);
+        const double overhead = sc.dt == BSR_F32 ? 30.0 * (double)sc.tc.task_chunks_max[gi] + 0.8 * G * sc.ex_R +
+                                                       (per_sm > 1 ? 80.0 : 480.0)
+                                                 : kOverheadMma;
+        const double cost = waves * (overhead + (double)sc.tc.task_cost_max[gi]);
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = G;

@@ -40,6 +40,7 @@ struct TcPlan {
     size_t task_wbytes[kTcTaskSizes] = {};   // W ring stage bytes
     size_t task_ibytes[kTcTaskSizes] = {};
     int64_t task_cost_max[kTcTaskSizes] = {};     // MMA cost of the most loaded task (units: one N <= 64 MMA)
+    int64_t task_chunks_max[kTcTaskSizes] = {};   // chunks of the task that visits most
     int64_t stacks[kTcTaskSizes] = {};            // stacked chunks over all tasks
     std::vector<int32_t> rec[kTcTaskSizes];       // all task records of this G
     std::vector<int32_t> rec_off[kTcTaskSizes];   // per task: offset (ints, multiple of 4)
