@@ -754,7 +754,7 @@ int fusion_class(const Schedule &sc, int64_t N, int *G) {
         if ((*G = choose_dense(sc, N)) > 0) return kDenseClass + (*G & kDnPair);
         if (choose_xcol(sc, N)) {
             *G = 0;
-            return kXcolClass;
+            return kXcolClass + sc.R;
         }
     }
     if (sc.variant == V_XSTAGE) {
@@ -807,8 +807,13 @@ cudaError_t launch_spmm_batch(const LaunchArgs *as, int n) {
             if (e != cudaSuccess) return e;
             continue;
         }
-        cudaError_t e = key >= kXcolClass ? launch_xcol(grp.data(), m) : tc ? (m == 1 ? launch_tc(grp[0], gs[0]) : launch_tc_batch(grp.data(), gs.data(), m))
-                           : (m == 1 ? launch_xstage(grp[0], gs[0]) : launch_xstage_batch(grp.data(), gs.data(), m));
+        cudaError_t e;
+        if (key >= kXcolClass)
+            e = launch_xcol(grp.data(), m);
+        else if (tc)
+            e = m == 1 ? launch_tc(grp[0], gs[0]) : launch_tc_batch(grp.data(), gs.data(), m);
+        else
+            e = m == 1 ? launch_xstage(grp[0], gs[0]) : launch_xstage_batch(grp.data(), gs.data(), m);
         if (e != cudaSuccess) return e;
         for (const LaunchArgs &a : grp)
             if (!a.sc->splits.empty() && (e = launch_reduce(a)) != cudaSuccess) return e;

@@ -1,9 +1,11 @@
-// SIMT kernel over column lists for fp32 one-column blocks of 32 rows ("xcol").
+// SIMT kernel over column lists for fp32 blocks of 32 or 16 rows and up to four
+// columns ("xcol").
 //
 // A warp multiplies an item (a block row) with 8 TT tokens: lane = tg + 8 rg,
 // tg picks tokens tg, tg + 8, ..., rg a group of 8 output rows. Per column a
 // lane loads TT activations and 8 weights from shared memory and does 8 TT
-// multiply-adds, packed in pairs of tokens.
+// multiply-adds, packed in pairs of tokens. For blocks of 16 rows a lane has 4
+// outputs and TT = 16 tokens: the same multiply-adds, 20 words instead of 16.
 //
 // What bounds it: the FP32 pipe as the register file feeds it. A packed
 // multiply-add reads three 64-bit operands; with the weight pair kept over
@@ -150,30 +152,35 @@ __device__ __forceinline__ Unit unit_at(const XcArgs &a, unsigned v) {
     return u;
 }
 
-// One column: TT activations at p and 8 weights at w (the lane's first four
+// One column: TT activations at p and NR weights at w (the lane's first four
 // outputs, and 16 further its last four).
-template <int TT>
-__device__ __forceinline__ void column(f2_t (&acc)[TT / 2][8], const unsigned char *p, const float *w) {
+template <int TT, int NR>
+__device__ __forceinline__ void column(f2_t (&acc)[TT / 2][NR], const unsigned char *p, const float *w) {
     f2_t x[TT / 2];
 #pragma unroll
     for (int i = 0; i < TT / 2; i++)
         x[i] = pack2(*reinterpret_cast<const float *>(p + 2 * i * 1024),
                      *reinterpret_cast<const float *>(p + (2 * i + 1) * 1024));
-    const float4 a = *reinterpret_cast<const float4 *>(w), b = *reinterpret_cast<const float4 *>(w + 16);
-    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    float v[NR];
 #pragma unroll
-    for (int j = 0; j < 8; j++) {
+    for (int j = 0; j < NR; j += 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(w + 4 * j);
+        v[j] = q.x, v[j + 1] = q.y, v[j + 2] = q.z, v[j + 3] = q.w;
+    }
+#pragma unroll
+    for (int j = 0; j < NR; j++) {
         const f2_t wj = pack2(v[j], v[j]);
 #pragma unroll
         for (int i = 0; i < TT / 2; i++) acc[i][j] = ffma2(x[i], wj, acc[i][j]);
     }
 }
 
-template <int MAXB, int TT>
+template <int MAXB, int TT, int NR>
 __global__ void __launch_bounds__(kThreads, 1)
 k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch<MAXB> b) {
     ptx::pdl_launch_dependents();
     constexpr uint32_t kX = 2 * kXcBox;
+    constexpr int R = 4 * NR;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = ptx::align_smem(smem_raw);
     __shared__ uint64_t full[kStagesMax], empty[kStagesMax];
@@ -285,18 +292,18 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
             while (u >= b.start[h + 1]) h++;
             const XcArgs &a = b.args[h];
             const bool has = warp < unit_at<TT>(a, u - b.start[h]).n;
-            f2_t acc[TT / 2][8];   // pairs of tokens
+            f2_t acc[TT / 2][NR];   // pairs of tokens
 #pragma unroll
             for (int i = 0; i < TT / 2; i++)
 #pragma unroll
-                for (int j = 0; j < 8; j++) acc[i][j] = 0ull;
-            constexpr bool kRegSums = TT == 8;   // the running sums fit the registers
-            f2_t total[kRegSums ? TT / 2 : 1][8];
+                for (int j = 0; j < NR; j++) acc[i][j] = 0ull;
+            constexpr bool kRegSums = TT * NR == 64;   // the running sums fit the registers
+            f2_t total[kRegSums ? TT / 2 : 1][NR];
             if constexpr (kRegSums) {
 #pragma unroll
                 for (int i = 0; i < TT / 2; i++)
 #pragma unroll
-                    for (int j = 0; j < 8; j++) total[i][j] = 0x8000000080000000ull;   // -0: adds nothing, to any value
+                    for (int j = 0; j < NR; j++) total[i][j] = 0x8000000080000000ull;   // -0: adds nothing, to any value
             }
             auto sums = [&]() {   // this warp's running sums
                 return tmem_s + ((uint32_t)(32 * (warp & 3)) << 16) +
@@ -308,7 +315,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                 // (as many loads at once as there are registers)
                 constexpr int L = TT == 12 ? 16 : 8;
 #pragma unroll
-                for (int k = 0; k < 8 * TT; k += L) {
+                for (int k = 0; k < NR * TT; k += L) {
                     uint32_t v[L / 8][8];
 #pragma unroll
                     for (int l = 0; l < L / 8; l++) tc5::ld8(at + k + 8 * l, v[l]);
@@ -317,7 +324,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                     for (int e = 0; e < L / 2; e++) {
                         uint32_t &v0 = v[e / 4][2 * (e % 4)], &v1 = v[e / 4][2 * (e % 4) + 1];
                         asm volatile("" : "+r"(v0), "+r"(v1));   // no use moves above the wait
-                        f2_t &t = acc[(k / 2 + e) / 8][(k / 2 + e) % 8];
+                        f2_t &t = acc[(k / 2 + e) / NR][(k / 2 + e) % NR];
                         float even, odd;
                         unpack2(t, even, odd);
                         t = pack2(even + __uint_as_float(v0), odd + __uint_as_float(v1));
@@ -340,20 +347,20 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                     int n = hdr->x;   // columns; then their places, then their weights
                     const int4 *oc = hdr + 1;
                     const float *w = reinterpret_cast<const float *>(oc + ((n + 3) >> 2)) + 4 * rg;
-                    for (; n >= 4; n -= 4, w += 4 * 32) {
+                    for (; n >= 4; n -= 4, w += 4 * R) {
                         const int4 o = *oc++;
-                        column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
-                        column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
+                        column<TT, NR>(acc, xs + ((uint32_t)o.x ^ tgx), w);
+                        column<TT, NR>(acc, xs + ((uint32_t)o.y ^ tgx), w + R);
                         asm volatile("" ::: "memory");   // two columns' operands at a time: no more fit the registers
-                        column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
-                        column<TT>(acc, xs + ((uint32_t)o.w ^ tgx), w + 96);
+                        column<TT, NR>(acc, xs + ((uint32_t)o.z ^ tgx), w + 2 * R);
+                        column<TT, NR>(acc, xs + ((uint32_t)o.w ^ tgx), w + 3 * R);
                         asm volatile("" ::: "memory");
                     }
                     if (n > 0) {
                         const int4 o = *oc;
-                        column<TT>(acc, xs + ((uint32_t)o.x ^ tgx), w);
-                        if (n > 1) column<TT>(acc, xs + ((uint32_t)o.y ^ tgx), w + 32);
-                        if (n > 2) column<TT>(acc, xs + ((uint32_t)o.z ^ tgx), w + 64);
+                        column<TT, NR>(acc, xs + ((uint32_t)o.x ^ tgx), w);
+                        if (n > 1) column<TT, NR>(acc, xs + ((uint32_t)o.y ^ tgx), w + R);
+                        if (n > 2) column<TT, NR>(acc, xs + ((uint32_t)o.z ^ tgx), w + 2 * R);
                     }
                 }
                 __syncwarp();
@@ -366,7 +373,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
 #pragma unroll
                     for (int i = 0; i < (kRegSums ? TT / 2 : 1); i++)
 #pragma unroll
-                        for (int j = 0; j < 8; j++) {
+                        for (int j = 0; j < NR; j++) {
                             total[i][j] = fadd2(acc[i][j], total[i][j]);
                             acc[i][j] = 0ull;
                         }
@@ -375,11 +382,11 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                     if (c1 > a.seg) add_sums();
                     const uint32_t at = sums();
 #pragma unroll
-                    for (int k = 0; k < 8 * TT; k += 8) {
+                    for (int k = 0; k < NR * TT; k += 8) {
                         uint32_t v[8];
 #pragma unroll
                         for (int e = 0; e < 4; e++) {
-                            f2_t &t = acc[(k / 2 + e) / 8][(k / 2 + e) % 8];
+                            f2_t &t = acc[(k / 2 + e) / NR][(k / 2 + e) % NR];
                             float even, odd;
                             unpack2(t, even, odd);
                             v[2 * e] = __float_as_uint(even);
@@ -396,7 +403,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
 #pragma unroll
                 for (int i = 0; i < TT / 2; i++)
 #pragma unroll
-                    for (int j = 0; j < 8; j++) acc[i][j] = fadd2(acc[i][j], total[i][j]);
+                    for (int j = 0; j < NR; j++) acc[i][j] = fadd2(acc[i][j], total[i][j]);
             } else if (nch > a.seg) {
                 add_sums();
             }
@@ -408,17 +415,17 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
             // workspace, for a piece of a split row)
             const Item it = a.items[un.i0 + warp];
             const bool partial = it.slot >= 0;
-            const int64_t pitch = partial ? 32 : a.M;
-            float *out = partial ? a.ws + (int64_t)it.slot * b.N * 32 : a.Y + (int64_t)it.row * 32;
-            const float *bias = a.bias && !partial ? a.bias + (int64_t)it.row * 32 : nullptr;
-            float bv[8];
+            const int64_t pitch = partial ? R : a.M;
+            float *out = partial ? a.ws + (int64_t)it.slot * b.N * R : a.Y + (int64_t)it.row * R;
+            const float *bias = a.bias && !partial ? a.bias + (int64_t)it.row * R : nullptr;
+            float bv[NR];
 #pragma unroll
-            for (int j = 0; j < 8; j++) bv[j] = bias ? __ldg(bias + (j < 4 ? 4 * rg + j : 16 + 4 * rg + j - 4)) : 0.f;
+            for (int j = 0; j < NR; j++) bv[j] = bias ? __ldg(bias + (j < 4 ? 4 * rg + j : 16 + 4 * rg + j - 4)) : 0.f;
 #pragma unroll
             for (int i = 0; i < TT; i++) {
-                float v[8];
+                float v[NR];
 #pragma unroll
-                for (int j = 0; j < 8; j++) {
+                for (int j = 0; j < NR; j++) {
                     float even, odd;
                     unpack2(acc[i >> 1][j], even, odd);
                     v[j] = i & 1 ? odd : even;
@@ -426,9 +433,10 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                 const int64_t t = un.n0 + tg + 8 * i;
                 if (t < b.N) {
                     float *dst = out + t * pitch + 4 * rg;
-                    *reinterpret_cast<float4 *>(dst) = make_float4(v[0] + bv[0], v[1] + bv[1], v[2] + bv[2], v[3] + bv[3]);
-                    *reinterpret_cast<float4 *>(dst + 16) =
-                        make_float4(v[4] + bv[4], v[5] + bv[5], v[6] + bv[6], v[7] + bv[7]);
+#pragma unroll
+                    for (int j = 0; j < NR; j += 4)
+                        *reinterpret_cast<float4 *>(dst + 4 * j) =
+                            make_float4(v[j] + bv[j], v[j + 1] + bv[j + 1], v[j + 2] + bv[j + 2], v[j + 3] + bv[j + 3]);
                 }
             }
         }
@@ -443,14 +451,15 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
 }
 
 // Weights of every packed column: src[2 k] = float offset of its R weights,
-// src[2 k + 1] = its stored block.
-__global__ void k_pack_xcol(const float *__restrict__ data, const int32_t *__restrict__ src, int64_t n, int R,
+// src[2 k + 1] = C times its stored block, plus its column in it.
+__global__ void k_pack_xcol(const float *__restrict__ data, const int32_t *__restrict__ src, int64_t n, int R, int C,
                             float *__restrict__ out) {
     const int64_t total = n * R;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t k = e / R;
         const int r = (int)(e - k * R);
-        out[(int64_t)src[2 * k] + r] = data[(int64_t)src[2 * k + 1] * R + r];
+        const int32_t q = src[2 * k + 1], block = q / C;
+        out[(int64_t)src[2 * k] + r] = data[((int64_t)block * R + r) * C + (q - block * C)];
     }
 }
 __global__ void k_pack_xcol_ints(const int32_t *__restrict__ pairs, int64_t n, int32_t *__restrict__ out) {
@@ -485,7 +494,7 @@ cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
     return e;
 }
 
-template <int MAXB, int TT>
+template <int MAXB, int TT, int NR>
 cudaError_t launch(const LaunchArgs *las, int n, int G) {
     XcBatch<MAXB> b;
     b.n = 0;
@@ -534,16 +543,16 @@ cudaError_t launch(const LaunchArgs *las, int n, int G) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     static std::atomic<uint64_t> attr_set{0};
-    cudaError_t e = allow_smem(k_xcol<MAXB, TT>, attr_set);
+    cudaError_t e = allow_smem(k_xcol<MAXB, TT, NR>, attr_set);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<int64_t>(units, las[0].sc->sm_count);
-    return launch_kernel(k_xcol<MAXB, TT>, dim3(grid), dim3(kThreads), b.ns * b.stage_bytes + 1024, las[0].stream, map,
+    return launch_kernel(k_xcol<MAXB, TT, NR>, dim3(grid), dim3(kThreads), b.ns * b.stage_bytes + 1024, las[0].stream, map,
                          b);
 }
 
-template <int TT>
+template <int TT, int NR>
 cudaError_t launch_n(const LaunchArgs *las, int n, int G) {
-    return n == 1 ? launch<1, TT>(las, 1, G) : launch<kXcBatchMax, TT>(las, n, G);
+    return n == 1 ? launch<1, TT, NR>(las, 1, G) : launch<kXcBatchMax, TT, NR>(las, n, G);
 }
 
 }  // namespace
@@ -557,7 +566,7 @@ cudaError_t pack_xcol_data(const Schedule &sc, const void *data, void *packed, c
                                                                                        reinterpret_cast<int32_t *>(out));
     if (nc)
         k_pack_xcol<<<(int)std::min<int64_t>((nc * sc.R + 255) / 256, 1 << 16), 256, 0, s>>>(
-            static_cast<const float *>(data), pl.d_src, nc, sc.R, reinterpret_cast<float *>(out));
+            static_cast<const float *>(data), pl.d_src, nc, sc.R, sc.C, reinterpret_cast<float *>(out));
     return cudaGetLastError();
 }
 
@@ -568,14 +577,15 @@ cudaError_t launch_xcol(const LaunchArgs *las, int n) {
     LaunchArgs sorted[kXcBatchMax];
     const Schedule *scs[kXcBatchMax];
     std::copy(las, las + n, sorted);
-    auto length = [](const LaunchArgs &la) { return (double)la.sc->nnzb / (double)std::max<size_t>(la.sc->items.size(), 1); };
+    auto length = [](const LaunchArgs &la) { return (double)la.sc->nnzb * la.sc->C / (double)std::max<size_t>(la.sc->items.size(), 1); };
     std::stable_sort(sorted, sorted + n, [&](const LaunchArgs &x, const LaunchArgs &y) { return length(x) > length(y); });
     for (int i = 0; i < n; i++) scs[i] = sorted[i].sc;
     const XcShape sh = xcol_shape(scs, n, las[0].N);
+    if (scs[0]->R == 16) return launch_n<kXcTT16, 4>(sorted, n, sh.G);
     switch (kXcTT[sh.tile]) {
-        case 8: return launch_n<8>(sorted, n, sh.G);
-        case 12: return launch_n<12>(sorted, n, sh.G);
-        case 14: return launch_n<14>(sorted, n, sh.G);
+        case 8: return launch_n<8, 8>(sorted, n, sh.G);
+        case 12: return launch_n<12, 8>(sorted, n, sh.G);
+        case 14: return launch_n<14, 8>(sorted, n, sh.G);
     }
     return cudaErrorInvalidConfiguration;
 }

@@ -1,5 +1,5 @@
-// The column-list SIMT kernel (spmm_xcol.cu) for fp32 32x1 blocks: parameters
-// shared with the schedule.
+// The column-list SIMT kernel (spmm_xcol.cu) for fp32 blocks of 16 or 32 rows:
+// parameters shared with the schedule.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -21,7 +21,8 @@ constexpr uint32_t kXcRoom = kXcMaxSmem - 2048;   // of it for the ring
 constexpr int kXcStagesMax = 8;
 constexpr int kXcBatchMax = 64;        // products in one fused launch
 constexpr int kXcTileSizes = 3;
-constexpr int kXcTT[kXcTileSizes] = {8, 12, 14};   // tokens per lane; 8 times as many per unit
+constexpr int kXcTT[kXcTileSizes] = {8, 12, 14};   // tokens per lane (blocks of 32 rows); 8 times as many per unit
+constexpr int kXcTT16 = 16;            // of 16 rows
 
 // A task is up to kXcWarps items (block rows, or pieces of them), one per warp; a
 // launch chooses how many, and its tile: neither changes an output's bits.
@@ -29,12 +30,13 @@ constexpr int kXcTT[kXcTileSizes] = {8, 12, 14};   // tokens per lane; 8 times a
 // so that a task's part of a chunk is one bulk copy:
 //   int32 n, 0, 0, 0   columns in this chunk
 //   int32 [n]          byte offsets of theirs in the X tile, padded to 4
-//   float [n][32]      their weights
+//   float [n][R]       their weights
 struct XcPlan {
     bool ok = false;
     int64_t off = -1, bytes = 0;       // place in the handle's packed buffer
     uint32_t item_bytes = 0;           // largest packed chunk of an item
     int seg = 1;                       // chunks per segment (one chain of additions)
+    bool even = false;                 // items of about equal length
     std::vector<int32_t> table;        // per chunk and item: its start / 16 (and the end)
     std::vector<int32_t> ints;         // (place / 4 bytes, value) of the packed buffer's integers
     std::vector<int32_t> src;          // per column: its weights' place / 4 bytes, its block
@@ -58,14 +60,14 @@ struct LaunchArgs;
 int64_t plan_xcol(Schedule &sc, int64_t base);
 // Whether the kernel runs a call of N tokens.
 bool choose_xcol(const Schedule &sc, int64_t N);
-// Tile (index into kXcTT) and items per task of one grid of n products.
+// Tile (index into kXcTT; 32 rows) and items per task of one grid of n products.
 struct XcShape {
     int tile, G;
     double cycles;   // the model's, of the busiest SM
 };
 XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N);
 cudaError_t pack_xcol_data(const Schedule &sc, const void *data, void *packed, cudaStream_t s);
-// n products that share X, N, K and the stream: one grid.
+// n products that share X, N, K, R and the stream: one grid.
 cudaError_t launch_xcol(const LaunchArgs *las, int n);
 
 }  // namespace bsr

@@ -13,8 +13,10 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     XcPlan &pl = sc.xc;
     pl.ok = false;
     const int64_t n_items = (int64_t)sc.items.size();
-    if (sc.dt != BSR_F32 || sc.C != 1 || sc.R != 32 || sc.K % 4 || n_items == 0 || sc.variant != V_XSTAGE ||
-        sc.nnzb > INT32_MAX / 256)
+    // (wider blocks: the per-task kernel loads four activations at a time; 16x16 of
+    // 768 x 768 at 70%, 4000 tokens 53 us against 71 here, 32x8 at 80% 36 against 39)
+    if (sc.dt != BSR_F32 || (sc.R != 16 && sc.R != 32) || sc.C > 4 || kXcChunk % sc.C || sc.K % 4 || n_items == 0 ||
+        sc.variant != V_XSTAGE || sc.nnzb > INT32_MAX / 256 / sc.C)
         return base;
     const int64_t nch = (sc.K + kXcChunk - 1) / kXcChunk;
     pl.off = (base + 1023) & ~int64_t(1023);
@@ -33,17 +35,19 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
         for (size_t i = 0; i < sc.items.size(); i++) {
             const Item &it = sc.items[i];
             int32_t &p = next[i], p1 = p;
-            while (p1 < it.p1 && sc.indices[(size_t)p1] < (c + 1) * kXcChunk) p1++;
-            const int64_t n = p1 - p, vals = at + 4 + ((n + 3) & ~int64_t(3));
+            while (p1 < it.p1 && (int64_t)sc.indices[(size_t)p1] * sc.C < (c + 1) * kXcChunk) p1++;
+            const int64_t n = (int64_t)(p1 - p) * sc.C, vals = at + 4 + ((n + 3) & ~int64_t(3));
             pl.table.push_back((int32_t)(at / 4));
             put(at, n);
-            for (int64_t k = 0; k < n; k++, p++) {
-                const int kk = (int)(sc.indices[(size_t)p] - c * kXcChunk), b = kk & 31;
+            for (int64_t k = 0; k < n; k++) {
+                const int64_t block = p + k / sc.C, in = k % sc.C;
+                const int kk = (int)(sc.indices[(size_t)block] * (int64_t)sc.C + in - c * kXcChunk), b = kk & 31;
                 put(at + 4 + k, ((b >> 2) << 4 | (b & 3) << 2) + (kk >> 5) * (int64_t)kXcBox);
-                pl.src.push_back((int32_t)(vals + 32 * k));
-                pl.src.push_back(p);
+                pl.src.push_back((int32_t)(vals + sc.R * k));
+                pl.src.push_back((int32_t)(block * sc.C + in));
             }
-            const int64_t end = vals + 32 * n;
+            p = p1;
+            const int64_t end = vals + sc.R * n;
             pl.item_bytes = std::max(pl.item_bytes, (uint32_t)((end - at) * 4));
             at = end;
             if (at > (int64_t)INT32_MAX / 2) return base;
@@ -55,10 +59,17 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     // further from 64 bits than the per-task kernel's, which shares a row among
     // warps (relative errors of ten sizes 0.98 to 1.37e-7, the per-task kernel's 1.16
     // to 1.43e-7; at 52 columns 1.17 to 1.47e-7, in one chain of 102 1.8e-7)
-    const double per_chunk = (double)sc.nnzb / (double)(n_items * nch);
+    const double per_chunk = (double)sc.nnzb * sc.C / (double)(n_items * nch);
     const int64_t most = per_chunk * (double)nch <= 40.0 ? nch : std::max<int64_t>(1, (int64_t)(40.0 / per_chunk));
     const int64_t segs = (nch + most - 1) / most;
     pl.seg = (int)((nch + segs - 1) / segs);
+    double longest = 0.0, apart = 0.0;   // of the items' blocks; from their mean
+    const double mean = (double)sc.nnzb / (double)n_items;
+    for (const Item &it : sc.items) {
+        longest = std::max(longest, (double)(it.p1 - it.p0));
+        apart += std::abs((double)(it.p1 - it.p0) - mean);
+    }
+    pl.even = longest <= 1.5 * mean && apart <= 0.25 * (double)sc.nnzb;
     if (2 * xcol_stage_bytes(pl.item_bytes, kXcWarps) > kXcRoom) return base;   // a ring of two stages
     pl.ok = true;
     return pl.off + pl.bytes;
@@ -90,17 +101,19 @@ XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N) {
     for (int G : kG) {
         if (forced_G >= 1 && forced_G <= kXcWarps ? G != forced_G : 2 * xcol_stage_bytes(item_bytes, G) > kXcRoom) continue;
         for (int ti = 0; ti < kXcTileSizes; ti++) {
-            if (forced_tile >= 0 && forced_tile < kXcTileSizes && ti != forced_tile) continue;
+            const bool half = scs[0]->R == 16;   // one tile, whose lanes do as many multiply-adds as the first's
+            if (half ? ti > 0 : forced_tile >= 0 && forced_tile < kXcTileSizes && ti != forced_tile) continue;
             const int TT = kXcTT[ti];
-            const int64_t tiles = (N + 8 * TT - 1) / (8 * TT);
+            const int64_t tokens = 8 * (half ? kXcTT16 : TT), tiles = (N + tokens - 1) / tokens;
             double sum = 0.0, longest = 0.0;
             int64_t units = 0;
             for (int i = 0; i < n; i++) {
                 const int64_t items = (int64_t)scs[i]->items.size(), tasks = (items + G - 1) / G;
                 if (!items) continue;
                 const double warps = (double)(((items + tasks - 1) / tasks + 3) / 4);
-                const double unit = (double)scs[i]->nnzb / (double)items * (11.9 * TT * warps + (warps > 1 ? 0.0 : TT == 14 ? 75.0 : 24.0)) +
-                                    470.0 * chunks + 385.0 * TT +
+                const double mean = (double)scs[i]->nnzb * scs[i]->C / (double)items;
+                const double column = 11.9 * TT * warps + (warps > 1 ? 0.0 : TT == 14 ? 75.0 : 24.0);
+                const double unit = mean * column + 470.0 * chunks + 385.0 * TT +
                                     (TT > 8 ? 135.0 * TT * std::max(0.0, std::ceil(chunks / scs[i]->xc.seg) - 2.0) : 0.0);
                 units += tiles * tasks;
                 sum += unit * (double)(tiles * tasks);
@@ -123,7 +136,10 @@ XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N) {
 // tokens 125 and 203; 4096 x 4096 at 90%, 512 tokens 56 and 101; 768 x 768 at 70%,
 // 3000 tokens 28.3 and 37.4; at 50%, 1024 tokens 30.0 and 30.5. At 80%, 2000 tokens
 // 22.8 and 19.2; at 70%, 1024 tokens 21 and 13.3; 1024 x 768 at 50%, 500 tokens 30
-// and 15.6 (an item's columns are one warp's): these stay.
+// and 15.6 (an item's columns are one warp's): these stay. Blocks of 16 rows: 16x1 of
+// 1024 x 1024 at 90%, 16384 tokens 115 and 134; of 768 x 768 at 70%, 3000 tokens 32
+// and 41; 16x4 of 1024 x 1024 at 80%, 3000 tokens 43 and 60; 32x2 at 90%, 8000 tokens
+// 59 and 72.
 bool choose_xcol(const Schedule &sc, int64_t N) {
     static const int mode = [] {
         const char *v = getenv("BSR_XC");
@@ -139,6 +155,11 @@ bool choose_xcol(const Schedule &sc, int64_t N) {
     // (the choice for the last N asked, which is what a steady stream of calls asks again)
     const uint64_t memo = pl.last.load(std::memory_order_relaxed);
     if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return memo & 1;
+    // rows of unequal length stay, because an item is one warp's here (pruned at
+    // random, the longest row is below 1.5 means from about 40 columns on, and rows
+    // are 0.15 means apart or less; 16x1 Zipf rows of 1024 x 1024 at 80%, 3000 tokens
+    // 141 us, per-task 73)
+    if (!pl.even) return false;
     const Schedule *one = &sc;
     double cost = 0.0;
     const int G = choose_tasks(sc, N, &cost);

@@ -1,4 +1,4 @@
-"""The column-list SIMT kernel for fp32 32x1 blocks at each of its token tiles and
+"""The column-list SIMT kernel for fp32 blocks of 16 and 32 rows at each of its token tiles and
 several task sizes (forced: by itself it takes only calls it is faster on), and
 with both chosen per launch (one product and three then differ in them)."""
 import os

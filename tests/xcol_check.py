@@ -7,7 +7,10 @@ import sys
 
 import numpy as np
 
-SHAPES = [(32, 64, 1), (352, 100, 63), (384, 1000, 64), (1024, 768, 113), (160, 260, 1000), (736, 512, 4000)]   # M, K, N
+SHAPES = [(32, 1, 32, 64, 1), (32, 1, 352, 100, 63), (32, 1, 384, 1000, 64), (32, 1, 1024, 768, 113),
+          (32, 1, 160, 260, 1000), (32, 1, 736, 512, 4000), (32, 4, 352, 264, 400),
+          (16, 1, 16, 64, 1), (16, 1, 176, 100, 127), (16, 1, 384, 1000, 129), (16, 4, 352, 528, 1000),
+          (16, 4, 736, 260, 300), (16, 2, 512, 768, 2000)]   # R, C, M, K, N
 
 
 def main() -> int:
@@ -19,21 +22,21 @@ def main() -> int:
     from paper_2106_08846_gb300 import bsrlib as b
     from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
     fails = 0
-    for k, (M, K, N) in enumerate(SHAPES):
+    for k, (R, C, M, K, N) in enumerate(SHAPES):
         for rows in ("even", "uneven"):
-            MB = M // 32
-            cnt = np.full(MB, max(1, int(0.3 * K)), dtype=np.int64)
+            MB, KB = M // R, K // C
+            cnt = np.full(MB, max(1, int(0.3 * KB)), dtype=np.int64)
             if rows == "uneven":   # short, empty and dense rows (split into pieces: partial tiles in the workspace)
-                cnt[::2] = 3
+                cnt[::2] = min(3, KB)
                 cnt[1::5] = 0
-                cnt[MB // 2] = K
+                cnt[MB // 2] = KB
             seed = 9000 + 10 * k
-            w = synth.make_weight("xc", seed, M, K, 32, 1, "f32", 0, mask=synth.mask_from_row_counts(seed, cnt, K))
-            h = bsr.bsr_create(*build_on_gpu(w.W, 32, 1), 32, 1, M, K)
-            ref = oracle.bsr_from_dense(w.W, 32, 1)
+            w = synth.make_weight("xc", seed, M, K, R, C, "f32", 0, mask=synth.mask_from_row_counts(seed, cnt, KB))
+            h = bsr.bsr_create(*build_on_gpu(w.W, R, C), R, C, M, K)
+            ref = oracle.bsr_from_dense(w.W, R, C)
             X = synth.activations(seed + 1, N, K, "f32")
             tokens = np.unique(np.concatenate([np.arange(0, N, 7), np.arange(max(0, N - 130), N)]))
-            name = f"{rows} M={M} K={K} N={N}"
+            name = f"{R}x{C} {rows} M={M} K={K} N={N}"
             try:
                 for bias in (w.bias, None):
                     Y = to_host(h.spmm(to_dev(X), None if bias is None else to_dev(bias)))
@@ -53,12 +56,13 @@ def main() -> int:
             print(f"{name}: ok", flush=True)
             h.destroy()
     # three products of one grid (not by length) are bit for bit the single calls
-    ws = [synth.make_weight("xb", 9200 + i, 416, 512, 32, 1, "f32", s) for i, s in enumerate((50, 90, 70))]
-    hs = [bsr.bsr_create(*build_on_gpu(w.W, 32, 1), 32, 1, w.M, w.K) for w in ws]
     X = to_dev(synth.activations(9201, 700, 512, "f32"))
-    Ys = [torch.empty((700, w.M), device="cuda") for w in ws]
-    bsr.bsr_spmm_batch(hs[::-1], X, None, Ys[::-1], 700)
-    fails += sum(not torch.equal(h.spmm(X), Y) for h, Y in zip(hs, Ys))
+    for R in (16, 32):
+        ws = [synth.make_weight("xb", 9200 + i, 416, 512, R, 1, "f32", s) for i, s in enumerate((50, 90, 70))]
+        hs = [bsr.bsr_create(*build_on_gpu(w.W, R, 1), R, 1, w.M, w.K) for w in ws]
+        Ys = [torch.empty((700, w.M), device="cuda") for w in ws]
+        bsr.bsr_spmm_batch(hs[::-1], X, None, Ys[::-1], 700)
+        fails += sum(not torch.equal(h.spmm(X), Y) for h, Y in zip(hs, Ys))
     # a chunk that is never loaded: bounded waits, BSR_ERR_TIMEOUT, usable context
     os.environ.update(BSR_WAIT_LIMIT_NS="2000000", BSR_TEST_STALL_CHUNK="3")
     gpu = build_on_gpu(ws[0].W, 32, 1)
