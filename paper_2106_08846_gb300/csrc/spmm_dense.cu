@@ -183,6 +183,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
     float *bias_s = reinterpret_cast<float *>(base + (size_t)ns * stage_bytes);
     __shared__ uint64_t full[kDnStagesMax], empty[kDnStagesMax], acc_full[2], acc_empty[2], done;
     __shared__ int stop, loads[2][2];   // loads[producer][CTA of the pair]: loads issued
+    __shared__ int freed, handed;       // commits issued to `empty` and to `acc_full`
     __shared__ uint32_t tmem_s;
 
     // (a shuffle, so that the warp index and what follows from it is uniform)
@@ -199,7 +200,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
             ptx::mbar_init(&acc_empty[i], PAIR ? 2 * kEpiWarps : kEpiWarps);
         }
         ptx::mbar_init(&done, 1);
-        stop = 0;
+        stop = freed = handed = 0;
         ptx::fence_barrier_init();
     }
     if (warp == kMmaWarp) {
@@ -303,7 +304,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
         }
     } else if (warp == kMmaWarp) {
         if (rank == 0) {
-            int ab = 0;
+            int ab = 0, n_freed = 0, n_handed = 0;
             uint32_t fphase = 0, aphase = 1;
             bool ok = true;
             const uint64_t ad0 = tc5::desc_sw128(ptx::smem_addr(base)), step = stage_bytes >> 4;
@@ -333,6 +334,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
                         else tc5::commit(&empty[s]);
                     }
                     __syncwarp();
+                    n_freed++;
                     ad += step;
                     if (++s == ns) {
                         s = 0;
@@ -349,6 +351,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
                     else tc5::commit(&acc_full[ab]);
                 }
                 __syncwarp();
+                n_handed++;
                 ab ^= 1;
                 if (ab == 0) aphase ^= 1;
             }
@@ -356,6 +359,12 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
             if (elected) {
                 if constexpr (PAIR) tc5::commit_pair(&done);
                 else tc5::commit(&done);
+                freed = n_freed;
+                handed = n_handed;
+                if constexpr (PAIR) {
+                    ptx::store_cluster(ptx::map_to_cta(&freed, 1), (uint32_t)n_freed);
+                    ptx::store_cluster(ptx::map_to_cta(&handed, 1), (uint32_t)n_handed);
+                }
             }
             __syncwarp();
             ptx::mbar_wait_bounded(&done, 0, kDrainNs);
@@ -491,6 +500,22 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
         meet();
     }
     if (warp == kMmaWarp) {
+        // a commit arrives by itself, at both CTAs of a pair: each CTA waits for
+        // the last arrival at every barrier of its own before it gives up its
+        // tensor memory and its shared memory (a barrier a lane)
+        uint64_t *bar = nullptr;
+        int last = 0;   // the phase of the last arrival
+        if (lane < ns && lane < freed) {
+            bar = &empty[lane];
+            last = (freed - 1 - lane) / ns;
+        } else if (lane >= 29 && lane - 29 < min(2, handed)) {
+            bar = &acc_full[lane - 29];
+            last = (handed - 1 - (lane - 29)) / 2;
+        } else if (lane == 31) {
+            bar = &done;
+        }
+        if (bar) ptx::mbar_wait_bounded(bar, (uint32_t)last & 1, kDrainNs);
+        __syncwarp();
         tc5::fence_after();
         if constexpr (PAIR) tc5::dealloc_pair(tmem, 2 * kAccCols);
         else tc5::dealloc(tmem, 2 * kAccCols);

@@ -91,3 +91,29 @@ def test_dense_takes_sparse_narrow_weights_of_the_simt_variant(R, C, N):
         single = to_host(h.spmm(Xd, b if i == 0 else None))
         assert np.array_equal(to_host(Y), single)
         check_product(single, oracle.bsr_from_dense(w.W, R, C), X, ws[0].bias if i == 0 else None, M, rows=rows)
+
+
+@pytest.mark.parametrize("g", [2, 34, 48])
+def test_dense_back_to_back_launches_of_few_chunks(g):
+    """One chunk or two per unit, so that a CTA's last arrivals (ring stages,
+    accumulators, the second CTA's of a pair) come just before it ends and the
+    next launch takes its shared memory: 400 launches, bit for bit the first."""
+    code = """
+import torch, oracle, synth
+import paper_2106_08846_gb300 as bsr
+from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
+for K, N in ((64, 300), (128, 5000)):
+    w = synth.make_weight("de", 7900 + K, 512, K, 16, 16, "bf16", 50)
+    h = bsr.bsr_create(*build_on_gpu(w.W, 16, 16), 16, 16, 512, K)
+    X = synth.activations(7902, N, K, "bf16")
+    Xd, b = to_dev(X), to_dev(w.bias)
+    Ys = torch.empty((200, N, 512), dtype=torch.bfloat16, device="cuda")
+    for Y in Ys:
+        bsr.bsr_spmm(h, Xd, b, Y)
+    assert h.check_device_status() == 0
+    check_product(to_host(Ys[0]), oracle.bsr_from_dense(w.W, 16, 16), X, w.bias, 512)
+    assert all(torch.equal(Y, Ys[0]) for Y in Ys)
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, BSR_DENSE_G=str(g)),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-3000:]
