@@ -406,6 +406,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
             __syncwarp();   // (the last unit's biases have been read)
 #pragma unroll
             for (int j = 0; j < 8; j++) bs[lane + 32 * j] = bv[j];
+            __syncwarp();   // (other lanes read them)
             const int64_t nt = nw + lane;                      // this thread's token
             uint16_t *const yrow = a.Y + nt * a.M;
             for (int gq = 0; gq < gn; gq += 4) {               // 64 columns: four row groups

@@ -117,3 +117,26 @@ for K, N in ((64, 300), (128, 5000)):
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, BSR_DENSE_G=str(g)),
                        capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-3000:]
+
+
+@pytest.mark.parametrize("g", [5, 16, 48])
+def test_dense_each_unit_adds_its_own_bias(g):
+    """Tasks of more than four row groups, with chunks and without, the biases
+    of one unit unlike the next one's: a warp's lanes read one another's."""
+    code = """
+import numpy as np, torch, oracle, synth
+import paper_2106_08846_gb300 as bsr
+from tests.gpu_util import build_on_gpu, to_dev, to_host
+M, K, N = 16 * 203, 128, 2000
+cnt = np.zeros(M // 16, dtype=np.int64)
+cnt[::3] = 2
+w = synth.make_weight("dg", 8100, M, K, 16, 16, "bf16", 0, mask=synth.mask_from_row_counts(8100, cnt, K // 16))
+h = bsr.bsr_create(*build_on_gpu(w.W, 16, 16), 16, 16, M, K)
+bias = torch.arange(1, M + 1, device="cuda").bfloat16().float()
+Y = h.spmm(torch.zeros((N, K), dtype=torch.bfloat16, device="cuda"), bias)
+assert h.check_device_status() == 0
+assert torch.equal(Y.float(), bias.expand(N, M))
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, BSR_DENSE_G=str(g)),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-3000:]
