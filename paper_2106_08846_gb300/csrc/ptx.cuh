@@ -24,6 +24,10 @@ __device__ __forceinline__ unsigned char *align_smem(unsigned char *p) {
 // the stream be scheduled; wait until the kernels this one depends on have
 // completed and their writes are visible. Both are no-ops for a kernel
 // launched without programmatic serialisation.
+// A kernel that allocates tensor memory lets the next one be scheduled only
+// after it: a CTA of the next one on the same SM could otherwise take the
+// columns first and hold them while it waits for this kernel, which waits for
+// them without a limit.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -175,7 +175,6 @@ struct DnBatch {
 template <int MAXB, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
 k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatch<MAXB> b) {
-    ptx::pdl_launch_dependents();
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = ptx::align_smem(smem_raw);
     const int ns = b.ns;
@@ -211,6 +210,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
     __syncthreads();
     if constexpr (PAIR) ptx::cluster_barrier();   // the other CTA's barriers exist
     tc5::fence_after();
+    ptx::pdl_launch_dependents();   // (after the allocation: ptx.cuh)
     const uint32_t tmem = tmem_s;
     const unsigned units = b.start[b.n];
     const bool elected = ptx::elect_one();

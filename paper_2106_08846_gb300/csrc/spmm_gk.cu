@@ -234,7 +234,6 @@ __device__ __forceinline__ void gather_entry(uint32_t row, uint32_t sw, const in
 template <typename T, int R>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_gk(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ GkArgs a) {
-    ptx::pdl_launch_dependents();
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int KS = F32 ? 8 : 16;
     extern __shared__ unsigned char smem_raw[];
@@ -284,6 +283,7 @@ k_gk(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ GkArgs a)
     tc5::fence_before();
     __syncthreads();
     tc5::fence_after();
+    ptx::pdl_launch_dependents();   // (after the allocation: ptx.cuh)
     const uint32_t tmem = (uint32_t)misc[1];
     const uint32_t abase = tmem + (uint32_t)(a.G * R);   // A buffers after the accumulators
 

@@ -115,7 +115,6 @@ __device__ __forceinline__ int pad4(int n) { return (n + 3) & ~3; }
 // read X from DRAM twice on 1024-wide fp32 16x16 weights, 107.6 -> 102.2 us).
 template <typename T, int R>
 __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a, unsigned cta) {
-    ptx::pdl_launch_dependents();
     constexpr bool F32 = sizeof(T) == 4;
     const int NS = F32 ? a.ns : TcCfg<T>::NSMAX;
     const int nslot = F32 ? a.nslot : 1;
@@ -170,6 +169,7 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
     tc5::fence_before();
     __syncthreads();
     tc5::fence_after();
+    ptx::pdl_launch_dependents();   // (after the allocation: ptx.cuh)
     const uint32_t tmem = (uint32_t)misc[1];
     const uint32_t a_col = (uint32_t)max(32, a.G * R);           // fp32: the A slots' first column
     const uint32_t wblock = (uint32_t)R * C * (F32 ? 8 : 2);   // bytes of one block's B operand(s)

@@ -134,7 +134,6 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, uint64
 template <typename T, int R>
 __global__ void __launch_bounds__(TcpCfg<T>::NTHREADS, 1)
 k_tcp(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcpArgs a) {
-    ptx::pdl_launch_dependents();
     using Cfg = TcpCfg<T>;
     constexpr bool F32 = Cfg::F32;
     constexpr int SC = Cfg::SC;
@@ -197,6 +196,7 @@ k_tcp(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcpArgs 
     tc5::fence_before();
     __syncthreads();
     tc5::fence_after();
+    ptx::pdl_launch_dependents();   // (after the allocation: ptx.cuh)
     const uint32_t tmem = (uint32_t)misc[1];
     const uint32_t abase = tmem + (uint32_t)nacc * acc_cols;   // the A slots, after the accumulators
 

@@ -178,7 +178,6 @@ __device__ __forceinline__ void column(f2_t (&acc)[TT / 2][NR], const unsigned c
 template <int MAXB, int TT, int NR>
 __global__ void __launch_bounds__(kThreads, 1)
 k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch<MAXB> b) {
-    ptx::pdl_launch_dependents();
     constexpr uint32_t kX = 2 * kXcBox;
     constexpr int R = 4 * NR;
     extern __shared__ unsigned char smem_raw[];
@@ -202,6 +201,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
     tc5::fence_before();
     __syncthreads();
     tc5::fence_after();
+    ptx::pdl_launch_dependents();   // (after the allocation: ptx.cuh)
     const unsigned units = b.start[b.n];
     const bool elected = ptx::elect_one();
     auto halt = [&](int *status) {

@@ -140,3 +140,36 @@ assert torch.equal(Y.float(), bias.expand(N, M))
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, BSR_DENSE_G=str(g)),
                        capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-3000:]
+
+
+def test_kernels_that_allocate_tensor_memory_follow_one_another():
+    """Launches of the kernels that allocate tensor memory, one behind another
+    without a synchronisation, small enough to share an SM: each allocates
+    before the next may start, and every output is that of the call alone."""
+    import paper_2106_08846_gb300 as bsr
+    runs = []
+    for i, (R, C, M, K, dt, sp, N) in enumerate([
+            (16, 16, 4096, 4096, "bf16", 98, 200),   # block by block, two CTAs an SM
+            (16, 16, 512, 64, "bf16", 50, 200),      # dense tiles
+            (32, 32, 256, 64, "f32", 0, 200),        # block by block, fp32
+            (64, 1, 512, 768, "f32", 85, 1000),      # gathered K
+            (32, 1, 1024, 768, "f32", 50, 2000),     # column lists
+            (64, 64, 512, 192, "bf16", 0, 700)]):
+        w = synth.make_weight("tm", 8200 + i, M, K, R, C, dt, sp)
+        h = bsr.bsr_create(*build_on_gpu(w.W, R, C), R, C, M, K)
+        X = to_dev(synth.activations(8300 + i, N, K, dt))
+        h.reserve(N)
+        Y = h.spmm(X, to_dev(w.bias))
+        torch.cuda.synchronize()
+        runs.append((h, X, to_dev(w.bias), Y, torch.empty((8, *Y.shape), dtype=Y.dtype, device="cuda")))
+    pairs = [(a, b) for a in range(len(runs)) for b in range(len(runs))]
+    for rep in range(60):
+        for h, X, b, _, Ys in (runs[k] for k in pairs[rep % len(pairs)]):
+            for k in range(4):
+                bsr.bsr_spmm(h, X, b, Ys[k + 4 * (rep & 1)])
+    for rep in range(8):
+        for h, X, b, _, Ys in runs:
+            bsr.bsr_spmm(h, X, b, Ys[rep])
+    for h, X, b, Y, Ys in runs:
+        assert h.check_device_status() == 0
+        assert all(torch.equal(Y, Yk) for Yk in Ys)
