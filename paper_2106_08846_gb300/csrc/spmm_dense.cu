@@ -289,7 +289,12 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
     if (warp < 2) {
         if (elected) ptx::prefetch_tensormap(&xmap);
         more = seek();
-        if (prod == 0) ptx::pdl_wait();   // X may be an earlier kernel's output (the packed weight is not)
+        // X may be an earlier kernel's output; the packed weight is not, and the
+        // first ns stages are free. The next ones are when the MMAs have read X:
+        // their limit does not run while an earlier kernel does
+        if (prod)
+            while (more && issued < ns) more = load_chunk();
+        ptx::pdl_wait();
         while (more) {
             const bool got = wait_or_abort(&empty[s], phase, wait_ns, &stop);
             if (!__all_sync(0xffffffffu, got && !aborted(&stop))) {

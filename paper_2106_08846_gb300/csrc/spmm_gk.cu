@@ -356,6 +356,7 @@ k_gk(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ GkArgs a)
         // its part of every batch's program (its items' MMAs), one word per MMA
         if (lane == 0) {
             const int q = warp - 1;
+            ptx::pdl_wait();   // X comes after the earlier kernel: the waits are bounded from here on
             bool ok = true;
             int j = -1;
             int64_t task = -1, k = 0, kb = 0, ui = 0;
@@ -428,6 +429,7 @@ k_gk(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ GkArgs a)
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
         int lc = 0;
         while ((1 << lc) < a.C) lc++;
+        ptx::pdl_wait();
         bool ok = true;
         int j = -1;
         int64_t task = -1, k = 0, kb = 0;

@@ -246,6 +246,7 @@ __device__ __forceinline__ void tc_cta(const CUtensorMap &xmap, const TcArgs &a,
                 if (i1 == 0) i0 = 0;
             }
             const uint32_t ufirst = (uint32_t)i0, ucnt = (uint32_t)(i1 - i0);
+            ptx::pdl_wait();   // X comes after the earlier kernel: the waits are bounded from here on
             bool ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(rbar, 0, a.wait_ns) && !aborted(misc));
             const int32_t *ent = I_s + items_at + 4 * g_count;
             int s = 0, sl_ = 0;             // stage; fp32: A slot

@@ -282,6 +282,7 @@ k_tcp(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcpArgs 
         // every stage's program, one word per MMA
         if (lane == 0) {
             const int q = warp - 1;
+            ptx::pdl_wait();   // X comes after the earlier kernel: the waits are bounded from here on
             bool ok = true;
             int j = -1;
             int64_t task = -1, k = 0, ui = 0;
@@ -368,6 +369,7 @@ k_tcp(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcpArgs 
         const int t = 32 * q + lane;
         const uint32_t swz = (uint32_t)(t & 7);   // 128-byte swizzle: 16-byte group g of row t sits at g ^ (t % 8)
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
+        ptx::pdl_wait();
         bool ok = true;
         int j = -1;
         int64_t task = -1, k = 0;

@@ -285,6 +285,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
         // ---------------- consumers
         const int tg = lane & 7, rg = lane >> 3;
         const uint32_t tgx = (uint32_t)tg << 4;
+        ptx::pdl_wait();   // X, the bias, Y and the workspace may be an earlier kernel's; the waits are bounded from here on
         uint32_t phase = 0;
         bool ok = true;
         for (unsigned k = 0, u; ok && k * gridDim.x < units; k++) {
@@ -407,7 +408,6 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
             } else if (nch > a.seg) {
                 add_sums();
             }
-            ptx::pdl_wait();   // the bias, Y and the workspace may be an earlier kernel's
             if (!has) continue;
             // (the unit once more: the registers are the columns' until here)
             const Unit un = unit_at<TT>(a, u - b.start[h]);
