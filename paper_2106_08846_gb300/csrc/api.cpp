@@ -525,7 +525,7 @@ bsr_status_t bsr_spmm(bsr_handle_t h, const void *X, const float *bias, void *Y,
         Yd = h->stage_y;
     }
     LaunchArgs a{&sc, h->data_packed ? h->data_packed : h->data, Xd, bias, Yd, h->ws, h->d_status, N, s,
-                 h->wait_ns, h->stall_chunk, h->data};
+                 h->wait_ns, h->stall_chunk};
     if (launch_spmm(a) != cudaSuccess) {
         cudaGetLastError();
         return BSR_ERR_CUDA;
@@ -594,7 +594,7 @@ bsr_status_t bsr_spmm_batch(const bsr_handle_t *handles, int n, const void *X, c
         Handle *h = handles[i];
         as.push_back(LaunchArgs{h->sched.get(), h->data_packed ? h->data_packed : h->data, X,
                                 biases ? biases[i] : nullptr, Ys[i], h->ws, h->d_status, N, s, h->wait_ns,
-                                h->stall_chunk, h->data});
+                                h->stall_chunk});
     }
     if (launch_spmm_batch(as.data(), n) != cudaSuccess) {
         cudaGetLastError();
@@ -674,7 +674,7 @@ bsr_status_t bsr_plan_create(const bsr_handle_t *handles, const void *const *X, 
             const Handle *h = handles[i];
             as.push_back(LaunchArgs{h->sched.get(), h->data_packed ? h->data_packed : h->data, X[i],
                                     biases ? biases[i] : nullptr, Y[i], ws_of[(size_t)i], h->d_status, N[i], cs,
-                                    h->wait_ns, h->stall_chunk, h->data});
+                                    h->wait_ns, h->stall_chunk});
             plan->order.push_back(i);
             plan->call.push_back((int)c);
         }

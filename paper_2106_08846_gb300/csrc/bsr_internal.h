@@ -142,7 +142,6 @@ struct LaunchArgs {
     cudaStream_t stream;
     uint64_t wait_ns;      // bound on every device-side wait
     int stall_chunk;       // test hook, -1 in normal use
-    const void *raw;       // the caller's block values
 };
 cudaError_t launch_generic(const LaunchArgs &a);
 cudaError_t launch_xstage(const LaunchArgs &a, int G);

@@ -25,7 +25,7 @@ constexpr int kDnMaxSmem = 232448;   // 227 KB
 
 // The weight's rows in groups of 16; the groups that hold a kept block come
 // first and are the rows of the packed dense weight [16 n_full, K] (columns
-// without a kept block are zero), groups without one follow (their outputs
+// without a kept block are -0), groups without one follow (their outputs
 // are the bias). A task of size g is g consecutive groups; its table entry
 // lists the 64-column chunks in which any of its groups has a block.
 struct DensePlan {

@@ -91,7 +91,7 @@ extern "C" bsr_status_t bsr_spmm_noalloc(bsr_handle_t h, const void *X, const fl
                           Y,     scratch,
                           h->d_status, N,
                           static_cast<cudaStream_t>(stream), h->wait_ns,
-                          h->stall_chunk, h->data};
+                          h->stall_chunk};
         if (bsr::launch_spmm(a) != cudaSuccess) {
             cudaGetLastError();
             st = BSR_ERR_CUDA;

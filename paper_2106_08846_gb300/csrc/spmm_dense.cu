@@ -38,11 +38,17 @@
 // come from two warps. Y staged through shared memory for TMA stores took 1000
 // to 1900 cycles per 64 columns, waiting behind the tiles.
 //
-// Zeros stand for absent blocks, so an infinity or NaN of X in a column that
-// an output's row does not keep would make that output NaN (0 x inf). Finite
-// X gives exactly the kept blocks' sum, and a zero product can only turn an
-// output into NaN, never into another finite value; so every output whose
-// accumulator is NaN is computed again from the kept blocks alone.
+// Zeros (-0, which no kept element is packed as) stand for absent blocks, so an
+// infinity or NaN of X in a column that an output's row does not keep would
+// make that output NaN (0 x inf). Finite X gives exactly the kept blocks' sum,
+// and a zero product can only turn an output into NaN, never into another
+// finite value; so every output whose accumulator is NaN is computed again,
+// without what is absent, by the epilogue warp that stored it, once the
+// accumulators are handed on. That takes far longer than the product: 1024 x
+// 1024 at 90%, 32x1, 16384 tokens 115 us with one such token, 295 us with every
+// 97th, 6.6 ms with a NaN in every token (27 us without; one lane walking each
+// output's blocks, with the accumulators held, had taken 5.1, 15 and 46 ms, and
+// at K = 8192 350 ms where it is now 20).
 //
 // Launched with programmatic stream serialisation: the barriers, tensor
 // memory and the first weight tiles come before the wait for the previous
@@ -74,20 +80,20 @@ constexpr int kMmaWarp = 2;                        // after the two producers
 constexpr int kThreads = 32 * (kMmaWarp + 1 + kEpiWarps);
 constexpr uint32_t kBiasBytes = kEpiWarps * 256 * 4;
 constexpr uint32_t kAccCols = 256;                 // tensor-memory columns per accumulator buffer
+constexpr uint16_t kAbsent = 0x8000;               // -0: what the packed weight holds where no block is
 constexpr uint64_t kDrainNs = 200000000ull;        // bound for copies and MMAs already issued
 
 struct DnArgs {
     CUtensorMap wmap;             // packed weight [16 n_full, K], boxes of 16 g (a pair's CTA: 8 g) rows x 64 columns
     const int32_t *table;         // task list offsets, then chunk lists
     const int32_t *group_row;
-    const int32_t *indptr, *indices;   // the caller's structure and block values, for outputs with a NaN sum
-    const uint16_t *data;
+    const uint16_t *w;            // the packed weight
     const float *bias;
     uint16_t *Y;
     int *status;
     int64_t M;
     uint64_t wait_ns;
-    int R, C, g, n_groups, n_tasks, n_work;   // n_work: tasks with chunks (they come first)
+    int g, n_groups, n_full, n_tasks, n_work;   // n_full: groups with packed rows; n_work: tasks with chunks (they come first)
     unsigned tiles;
     int task_major;               // units task by task (unequal tasks), else tile by tile
     int stall_chunk;
@@ -124,13 +130,23 @@ __device__ __forceinline__ Unit unit_at(const DnArgs &a, unsigned v) {
 __device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
 __device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
 
-// Bounded wait that also gives up when another role of the CTA stopped.
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, uint64_t limit_ns, const int *flag) {
+// Bounded wait that also gives up when another role of the CTA stopped. The
+// limit begins anew while an epilogue warp of the CTA or its pair, for which
+// every role waits in the end, reports that it computes outputs again.
+__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, uint64_t limit_ns, const int *flag,
+                                              const int *beat) {
     if (ptx::mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = ptx::globaltimer();
+    uint64_t t0 = ptx::globaltimer();
+    int seen = 0;
     while (true) {
         if (ptx::mbar_try_wait(bar, parity)) return true;
-        if (aborted(flag) || ptx::globaltimer() - t0 > limit_ns) return false;
+        if (aborted(flag)) return false;
+        const uint64_t t = ptx::globaltimer();
+        if (t - t0 <= limit_ns) continue;
+        const int now = *reinterpret_cast<const volatile int *>(beat);
+        if (now == seen) return false;
+        seen = now;
+        t0 = t;
     }
 }
 
@@ -141,19 +157,121 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return r;
 }
 
-// gr[i] without a register array indexed at run time.
-__device__ __forceinline__ int gr_at(const int (&gr)[4], int i) { return i < 2 ? (i ? gr[1] : gr[0]) : (i == 2 ? gr[2] : gr[3]); }
-
-// Output m of the token with activations x, from its row's kept blocks alone.
-__device__ __noinline__ float kept_blocks_dot(const DnArgs &a, const uint16_t *x, int64_t m) {
-    const int64_t i = m / a.R, r = m - i * a.R;
-    float acc = 0.f;
-    for (int p = __ldg(a.indptr + i); p < __ldg(a.indptr + i + 1); p++) {
-        const uint16_t *xb = x + (int64_t)__ldg(a.indices + p) * a.C;
-        const uint16_t *wb = a.data + ((int64_t)p * a.R + r) * a.C;
-        for (int c = 0; c < a.C; c++) acc = fmaf(to_f32(xb[c]), to_f32(wb[c]), acc);
+// acc[r] = the sum over a unit's n chunks (eights of columns first, first +
+// step, ...) of activation times packed row r, leaving out what is absent.
+template <typename Beat>
+__device__ __forceinline__ void kept_sums(float (&acc)[kDnGroup], const uint16_t *x, const uint16_t *w, int64_t K,
+                                          const int32_t *list, int n, int first, int step, Beat beat) {
+#pragma unroll
+    for (int r = 0; r < kDnGroup; r++) acc[r] = 0.f;
+    int64_t col_next = K;   // the next eight columns and their activations, on their way (K: none; a multiple of 8)
+    uint4 x_next = {};
+    auto fetch = [&](int v) {
+        if (v < 8 * n) col_next = min(K, (int64_t)__ldg(list + (v >> 3)) * KC + 8 * (v & 7));
+        if (col_next < K) x_next = __ldg(reinterpret_cast<const uint4 *>(x + col_next));
+    };
+    fetch(first);
+    for (int v = first, k = 0; v < 8 * n; v += step, k++) {
+        if ((k & 31) == 0) beat();
+        const int64_t col = col_next;
+        const uint4 xq = x_next;
+        fetch(v + step);
+        if (col >= K) continue;
+        const uint32_t xw[4] = {xq.x, xq.y, xq.z, xq.w};
+        float xf[8];   // finite activations, zero for the others
+        bool all = true;
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            const uint32_t b = e & 1 ? xw[e / 2] & 0xffff0000u : xw[e / 2] << 16;
+            const bool fin = (b & 0x7f800000u) != 0x7f800000u;
+            all = all && fin;
+            xf[e] = fin ? __uint_as_float(b) : 0.f;
+        }
+#pragma unroll
+        for (int r = 0; r < kDnGroup; r++) {
+            const uint4 wq = __ldg(reinterpret_cast<const uint4 *>(w + r * K + col));
+            const uint32_t ww[4] = {wq.x, wq.y, wq.z, wq.w};
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                acc[r] = fmaf(xf[e], __uint_as_float(e & 1 ? ww[e / 2] & 0xffff0000u : ww[e / 2] << 16), acc[r]);
+        }
+        if (!all) {
+#pragma unroll 1
+            for (int e = 0; e < 8; e++) {
+                const float xv = to_f32(__ldg(x + col + e));
+                if (fabsf(xv) <= 3.4e38f) continue;
+#pragma unroll
+                for (int r = 0; r < kDnGroup; r++) {
+                    const uint16_t wv = __ldg(w + r * K + col + e);
+                    if (wv != kAbsent) acc[r] = fmaf(xv, to_f32(wv), acc[r]);
+                }
+            }
+            bool nan = true;   // more terms leave NaN sums so
+#pragma unroll
+            for (int r = 0; r < kDnGroup; r++) nan = nan && acc[r] != acc[r];
+            if (nan) break;
+        }
     }
-    return acc;
+}
+
+// Computes the NaN outputs of a unit's part again, for one warp's 32 tokens
+// from n0 on: row groups g0 .. g0 + gn - 1 (lane j knows the output rows 16 gl
+// of group j) over the unit's chunks. Bit j / 4 of this lane's `bad`: its token
+// may have such an output in group j. A few tokens of a group share the warp, a
+// lane taking every 32nd eight of columns; more take a lane each. `beat` is set
+// time and again, here and in the other CTA of a pair (remote: 0 without one).
+__device__ __noinline__ void compute_again(const DnArgs &a, const uint16_t *X, int64_t K, int64_t n0, int g0, int gn, int gl,
+                                           const int32_t *list, int chunks, uint32_t bad, int *beat_s, uint32_t remote) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();   // (other lanes' outputs are stored)
+    for (int j = 0; j < gn; j++) {
+        const int64_t row0 = (int64_t)__shfl_sync(0xffffffffu, gl, j) * kDnGroup;
+        bool any = false;   // this lane's token has a NaN output in the group
+        if ((bad >> (j >> 2)) & 1)
+            for (int e = 0; e < kDnGroup; e++) any |= (a.Y[(n0 + lane) * a.M + row0 + e] & 0x7fffu) > 0x7f80u;
+        const uint32_t tokens = __ballot_sync(0xffffffffu, any);
+        if (!tokens) continue;
+        const bool lane_each = __popc(tokens) > 4;
+        const int speaker = lane_each ? __ffs(tokens) - 1 : 0;
+        auto beat = [&]() {
+            if (lane == speaker) {
+                const uint32_t t = (uint32_t)ptx::globaltimer() | 1u;
+                *reinterpret_cast<volatile int *>(beat_s) = (int)t;
+                if (remote) ptx::store_cluster(remote, t);
+            }
+        };
+        const uint16_t *w = a.w + (int64_t)(g0 + j) * kDnGroup * K;
+        const int n = g0 + j < a.n_full ? chunks : 0;   // (groups without blocks have no packed rows)
+        float acc[kDnGroup];
+        if (lane_each) {
+            if (any) {
+                const int64_t t = n0 + lane;
+                kept_sums(acc, X + t * K, w, K, list, n, 0, 1, beat);
+                uint16_t *y = a.Y + t * a.M + row0;
+#pragma unroll
+                for (int r = 0; r < kDnGroup; r++)
+                    if ((y[r] & 0x7fffu) > 0x7f80u)
+                        y[r] = from_f32<uint16_t>(acc[r] + (a.bias ? __ldg(a.bias + row0 + r) : 0.f));
+            }
+        } else {
+            for (uint32_t left = tokens; left; left &= left - 1) {
+                const int64_t t = n0 + __ffs(left) - 1;
+                kept_sums(acc, X + t * K, w, K, list, n, lane, 32, beat);
+                __syncwarp();
+                float mine = 0.f;   // row `lane`'s sum
+#pragma unroll
+                for (int r = 0; r < kDnGroup; r++) {
+#pragma unroll
+                    for (int d = 16; d > 0; d >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], d);
+                    if (r == lane) mine = acc[r];
+                }
+                uint16_t *y = a.Y + t * a.M + row0 + lane;
+                if (lane < kDnGroup && (*y & 0x7fffu) > 0x7f80u)
+                    *y = from_f32<uint16_t>(mine + (a.bias ? __ldg(a.bias + row0 + lane) : 0.f));
+            }
+        }
+        __syncwarp();
+    }
 }
 
 // Several products that share X in one grid: product h owns units start[h] ..
@@ -183,6 +301,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
     __shared__ uint64_t full[kDnStagesMax], empty[kDnStagesMax], acc_full[2], acc_empty[2], done;
     __shared__ int stop, loads[2][2];   // loads[producer][CTA of the pair]: loads issued
     __shared__ int freed, handed;       // commits issued to `empty` and to `acc_full`
+    __shared__ int beat;                // changes while an epilogue warp computes outputs again
     __shared__ uint32_t tmem_s;
 
     // (a shuffle, so that the warp index and what follows from it is uniform)
@@ -199,7 +318,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
             ptx::mbar_init(&acc_empty[i], PAIR ? 2 * kEpiWarps : kEpiWarps);
         }
         ptx::mbar_init(&done, 1);
-        stop = freed = handed = 0;
+        stop = freed = handed = beat = 0;
         ptx::fence_barrier_init();
     }
     if (warp == kMmaWarp) {
@@ -296,7 +415,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
             while (more && issued < ns) more = load_chunk();
         ptx::pdl_wait();
         while (more) {
-            const bool got = wait_or_abort(&empty[s], phase, wait_ns, &stop);
+            const bool got = wait_or_abort(&empty[s], phase, wait_ns, &stop, &beat);
             if (!__all_sync(0xffffffffu, got && !aborted(&stop))) {
                 halt(status);
                 break;
@@ -322,10 +441,10 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
                 if (un.n == 0) continue;
                 const uint32_t id = tc5::idesc(false, PAIR ? 2 * TN : TN, a.g * kDnGroup);
                 const uint32_t d = tmem + (uint32_t)ab * kAccCols;
-                ok = __all_sync(0xffffffffu, wait_or_abort(&acc_empty[ab], aphase, a.wait_ns, &stop));
+                ok = __all_sync(0xffffffffu, wait_or_abort(&acc_empty[ab], aphase, a.wait_ns, &stop, &beat));
                 tc5::fence_after();
                 for (int i = 0; ok && i < un.n; i++) {
-                    ok = __all_sync(0xffffffffu, wait_or_abort(&full[s], fphase, a.wait_ns, &stop));
+                    ok = __all_sync(0xffffffffu, wait_or_abort(&full[s], fphase, a.wait_ns, &stop, &beat));
                     if (!ok) break;
                     tc5::fence_after();
                     if (elected) {
@@ -399,7 +518,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
                 bv[j] = a.bias && gj >= 0 ? __ldg(a.bias + gj * 16 + (lane & 15)) : 0.f;
             }
             if (un.n > 0) {
-                const bool got = wait_or_abort(&acc_full[ab], fphase, a.wait_ns * (uint64_t)(un.n + 2), &stop);
+                const bool got = wait_or_abort(&acc_full[ab], fphase, a.wait_ns * (uint64_t)(un.n + 2), &stop, &beat);
                 ok = __all_sync(0xffffffffu, got);
                 if (!ok) {
                     halt(a.status);
@@ -414,6 +533,7 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
             __syncwarp();   // (other lanes read them)
             const int64_t nt = nw + lane;                      // this thread's token
             uint16_t *const yrow = a.Y + nt * a.M;
+            uint32_t bad = 0;                                  // fours of groups with a NaN or infinite sum of this token
             for (int gq = 0; gq < gn; gq += 4) {               // 64 columns: four row groups
                 const int cnt = min(4, gn - gq);
                 uint32_t r[64] = {};
@@ -465,15 +585,12 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
                         }
                     }
                 }
-                if (probe != 0.f && nt < b.N) {   // true for NaN only
-                    for (int e = 0; e < 16 * cnt; e++) {
-                        const int64_t m = (int64_t)gr_at(gr, e >> 4) * kDnGroup + (e & 15);
-                        if ((yrow[m] & 0x7fffu) <= 0x7f80u) continue;
-                        yrow[m] = from_f32<uint16_t>(kept_blocks_dot(a, b.X + nt * b.K, m) +
-                                                     (a.bias ? __ldg(a.bias + m) : 0.f));
-                    }
-                }
+                if (probe != 0.f && nt < b.N) bad |= 1u << (gq >> 2);   // true for NaN only
             }
+            // (the accumulators are free: the next units' MMAs run on)
+            if (__any_sync(0xffffffffu, bad != 0))
+                compute_again(a, b.X, b.K, nw, g0, gn, gl, un.list, un.n, bad, &beat,
+                              PAIR ? ptx::map_to_cta(&beat, rank ^ 1) : 0u);
             if (un.n > 0) {
                 ab ^= 1;
                 if (ab == 0) fphase ^= 1;
@@ -528,8 +645,15 @@ k_dense(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ DnBatc
     }
 }
 
-// Kept blocks into the zero-filled dense rows: element (r, c) of stored block
-// p of block row i goes to packed row 16 pos(group) + row % 16.
+__global__ void k_fill_absent(uint4 *__restrict__ out, int64_t n) {
+    constexpr uint32_t two = (uint32_t)kAbsent << 16 | kAbsent;
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+        out[k] = make_uint4(two, two, two, two);
+}
+
+// Kept blocks into the dense rows: element (r, c) of stored block p of block
+// row i goes to packed row 16 pos(group) + row % 16 (a kept -0 as 0, which
+// gives the same sums).
 __global__ void k_pack_dense(const uint16_t *__restrict__ data, const int32_t *__restrict__ indptr,
                              const int32_t *__restrict__ indices, const int32_t *__restrict__ group_pos, int64_t MB,
                              int R, int C, int64_t K, uint16_t *__restrict__ out) {
@@ -539,8 +663,9 @@ __global__ void k_pack_dense(const uint16_t *__restrict__ data, const int32_t *_
             const int64_t b = e / (R * C);
             const int rc = (int)(e - b * R * C), r = rc / C, c = rc - r * C;
             const int64_t row = i * R + r;
+            const uint16_t v = data[(p0 + b) * R * C + rc];
             out[((int64_t)group_pos[row / kDnGroup] * kDnGroup + row % kDnGroup) * K +
-                (int64_t)indices[p0 + b] * C + c] = data[(p0 + b) * R * C + rc];
+                (int64_t)indices[p0 + b] * C + c] = v == kAbsent ? 0 : v;
         }
     }
 }
@@ -606,18 +731,15 @@ cudaError_t launch(const LaunchArgs *las, const int *gs, int n) {
         const int g = gs[i];
         a.table = pl.d_table + pl.table_at[g];
         a.group_row = pl.d_group_row;
-        a.indptr = sc.d_indptr;
-        a.indices = sc.d_indices;
-        a.data = static_cast<const uint16_t *>(la.raw);
+        a.w = reinterpret_cast<const uint16_t *>(static_cast<const unsigned char *>(la.data) + pl.w_off);
         a.bias = la.bias;
         a.Y = static_cast<uint16_t *>(la.Y);
         a.status = la.status;
         a.M = sc.M;
         a.wait_ns = la.wait_ns;
-        a.R = sc.R;
-        a.C = sc.C;
         a.g = g;
         a.n_groups = pl.n_groups;
+        a.n_full = pl.n_full;
         a.n_tasks = pl.n_tasks[g];
         a.n_work = (pl.n_full + g - 1) / g;
         a.tiles = (unsigned)((la.N + kUnitTokens - 1) / kUnitTokens);
@@ -628,8 +750,7 @@ cudaError_t launch(const LaunchArgs *las, const int *gs, int n) {
         a.task_major = pl.max_chunks[g] * (int64_t)pl.n_tasks[g] > pl.chunks[g] + pl.chunks[g] / 4;
         a.stall_chunk = la.stall_chunk;
         a.y32 = reinterpret_cast<uintptr_t>(la.Y) % 32 == 0;   // (M is a multiple of 16)
-        cudaError_t e = encode(static_cast<const unsigned char *>(la.data) + pl.w_off,
-                               std::max<int64_t>(1, (int64_t)pl.n_full * kDnGroup), sc.K, g * kWRows, &a.wmap);
+        cudaError_t e = encode(a.w, std::max<int64_t>(1, (int64_t)pl.n_full * kDnGroup), sc.K, g * kWRows, &a.wmap);
         if (e != cudaSuccess) return e;
         b.start[b.n] = (unsigned)units;
         units += (int64_t)a.tiles * a.n_tasks;
@@ -658,7 +779,10 @@ cudaError_t launch(const LaunchArgs *las, const int *gs, int n) {
 cudaError_t pack_dense_data(const Schedule &sc, const void *data, void *packed, cudaStream_t s) {
     const DensePlan &pl = sc.dense;
     unsigned char *out = static_cast<unsigned char *>(packed) + pl.w_off;
-    cudaError_t e = cudaMemsetAsync(out, 0, (size_t)pl.w_bytes, s);
+    if (pl.w_bytes == 0) return cudaSuccess;
+    const int64_t eights = pl.w_bytes / 16;   // (K is a multiple of 8)
+    k_fill_absent<<<(int)std::min<int64_t>((eights + 255) / 256, 1 << 16), 256, 0, s>>>(reinterpret_cast<uint4 *>(out), eights);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || sc.nnzb == 0) return e;
     const int grid = (int)std::min<int64_t>(sc.MB, 1 << 16);
     k_pack_dense<<<grid, 256, 0, s>>>(static_cast<const uint16_t *>(data), sc.d_indptr, sc.d_indices, pl.d_group_pos,

@@ -11,7 +11,7 @@ import torch
 
 import oracle
 import synth
-from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
+from tests.gpu_util import as_f64, build_on_gpu, check_product, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -33,7 +33,7 @@ def test_dense_bounded_wait_times_out_and_reports(g):
 import os, numpy as np, oracle, synth, torch
 import paper_2106_08846_gb300 as bsr
 from paper_2106_08846_gb300 import bsrlib as b
-from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
+from tests.gpu_util import as_f64, build_on_gpu, check_product, to_dev, to_host
 w = synth.make_weight("ds", 7700, 512, 1536, 16, 16, "bf16", 80)
 gpu = build_on_gpu(w.W, 16, 16)
 os.environ.update(BSR_WAIT_LIMIT_NS="2000000", BSR_TEST_STALL_CHUNK="9")
@@ -101,7 +101,7 @@ def test_dense_back_to_back_launches_of_few_chunks(g):
     code = """
 import torch, oracle, synth
 import paper_2106_08846_gb300 as bsr
-from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
+from tests.gpu_util import as_f64, build_on_gpu, check_product, to_dev, to_host
 for K, N in ((64, 300), (128, 5000)):
     w = synth.make_weight("de", 7900 + K, 512, K, 16, 16, "bf16", 50)
     h = bsr.bsr_create(*build_on_gpu(w.W, 16, 16), 16, 16, 512, K)
@@ -173,3 +173,39 @@ def test_kernels_that_allocate_tensor_memory_follow_one_another():
     for h, X, b, Y, Ys in runs:
         assert h.check_device_status() == 0
         assert all(torch.equal(Y, Yk) for Yk in Ys)
+
+
+@pytest.mark.parametrize("R,C,share", [(32, 1, 1.0), (32, 1, 0.04), (1, 1, 1.0), (4, 4, 1.0), (16, 16, 1.0), (64, 16, 0.04)])
+def test_dense_non_finite_tokens_at_large_k(R, C, share, monkeypatch):
+    """A NaN or an infinity in every token (or a few of each 32): its outputs
+    that do not keep the column are computed again, which takes far longer than
+    a wait's limit (1 ms) and leaves no call unfinished; N is several units a
+    CTA. Other tokens keep the finite call's bits."""
+    import paper_2106_08846_gb300 as bsr
+    M, K, N = 1024, 8192, 20000
+    MB, KB = M // R, K // C
+    w = synth.make_weight("dnf", 8600 + R, M, K, R, C, "bf16", 0, mask=synth.uniform_block_mask(8600 + R, MB, KB, MB * KB // 5))
+    gpu = build_on_gpu(w.W, R, C)
+    monkeypatch.setenv("BSR_WAIT_LIMIT_NS", "1000000")
+    h = bsr.bsr_create(*gpu, R, C, M, K)
+    monkeypatch.delenv("BSR_WAIT_LIMIT_NS")
+    gen = torch.Generator(device="cuda").manual_seed(8601)
+    X = torch.randn(N, K, device="cuda", generator=gen).bfloat16()
+    b = to_dev(w.bias)
+    finite = h.spmm(X, b)
+    tokens = torch.rand(N, device="cuda", generator=gen) < share
+    at = torch.randint(K, (N,), device="cuda", generator=gen)
+    special = torch.tensor([float("nan"), float("inf"), float("-inf")], device="cuda").bfloat16()[torch.arange(N, device="cuda") % 3]
+    X[tokens, at[tokens]] = special[tokens]
+    Y = h.spmm(X, b)
+    assert h.check_device_status() == 0
+    assert torch.equal(Y[~tokens], finite[~tokens])
+    rows = tokens.nonzero()[:, 0][::max(1, int(tokens.sum()) // 40)]
+    Xs, ref = to_host(X[rows]), oracle.bsr_from_dense(w.W, R, C)
+    with np.errstate(invalid="ignore"):
+        want = oracle.bsr_spmm(*ref, Xs, w.bias, M)
+    got, fin = as_f64(to_host(Y[rows])), np.isfinite(want)
+    assert fin.mean() > 0.5 and np.array_equal(np.isfinite(got), fin)
+    assert np.array_equal(got[~fin], want[~fin], equal_nan=True)
+    E = oracle.err_bound(*ref, np.where(np.isfinite(as_f64(Xs)), Xs, 0).astype(np.uint16), w.bias, M)
+    assert np.all(np.abs(got - want)[fin] <= 1e-2 * E[fin])
