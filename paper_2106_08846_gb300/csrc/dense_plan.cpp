@@ -12,7 +12,8 @@ int64_t plan_dense(Schedule &sc, int64_t base) {
     DensePlan &pl = sc.dense;
     pl.ok = false;
     const bool shape_ok = kDnGroup % sc.R == 0 || sc.R % kDnGroup == 0;
-    if ((sc.variant != V_TC && sc.variant != V_XSTAGE) || sc.dt != BSR_BF16 || sc.M % kDnGroup || sc.K % 8 || !shape_ok)
+    if ((sc.variant != V_TC && sc.variant != V_XSTAGE) || sc.dt != BSR_BF16 || sc.M == 0 || sc.M % kDnGroup || sc.K % 8 ||
+        !shape_ok)
         return base;
     const int64_t n_groups = sc.M / kDnGroup, nch = (sc.K + kDnChunk - 1) / kDnChunk;
     if (n_groups > INT32_MAX / 32 || nch > 1 << 20) return base;

@@ -758,7 +758,7 @@ cudaError_t launch(const LaunchArgs *las, const int *gs, int n) {
         b.n++;
         if (units > INT32_MAX) return cudaErrorInvalidConfiguration;
     }
-    if (b.n == 0) return cudaSuccess;
+    if (units == 0) return cudaSuccess;
     b.start[b.n] = (unsigned)units;
     b.stage_bytes = kXBytes + (uint32_t)gmax * kWRows * 128;
     const uint32_t fixed = kBiasBytes + 1024;

@@ -1,6 +1,7 @@
 """The dense-tile tensor-core kernel for bf16 weights: task sizes at the edges
 of its range, ragged tokens, rows and columns, unequal and empty rows, X with
 infinities and NaN, and a fused batch of different shapes."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -209,3 +210,28 @@ def test_dense_non_finite_tokens_at_large_k(R, C, share, monkeypatch):
     assert np.array_equal(got[~fin], want[~fin], equal_nan=True)
     E = oracle.err_bound(*ref, np.where(np.isfinite(as_f64(Xs)), Xs, 0).astype(np.uint16), w.bias, M)
     assert np.all(np.abs(got - want)[fin] <= 1e-2 * E[fin])
+
+
+@pytest.mark.parametrize("M,K", [(0, 64), (64, 0), (0, 0)])
+@pytest.mark.parametrize("R,C", [(16, 16), (32, 1)])
+def test_dense_weights_without_elements(R, C, M, K):
+    """M = 0: nothing to write; K = 0: the bias; through every call form."""
+    import paper_2106_08846_gb300 as bsr
+    N = 200
+    lib = bsr.load()
+    stream = torch.cuda.current_stream().cuda_stream
+    hs = [bsr.bsr_create(torch.zeros(M // R + 1, dtype=torch.int32, device="cuda"), torch.zeros(0, dtype=torch.int32, device="cuda"),
+                         torch.zeros((0, R, C), dtype=torch.bfloat16, device="cuda"), R, C, M, K) for _ in range(2)]
+    X = torch.zeros(N * max(K, 8), dtype=torch.bfloat16, device="cuda")
+    bias = torch.arange(1, M + 2, device="cuda").float()
+    Ys = [torch.full((N * max(M, 8),), 7.0, dtype=torch.bfloat16, device="cuda") for _ in hs]
+    want = bias[:M].bfloat16().expand(N, M).flatten() if M else Ys[0].clone()
+    for call in (lib.bsr_spmm, lib.bsr_spmm_noalloc):
+        Ys[0].fill_(7.0)
+        assert call(hs[0].ptr, X.data_ptr(), bias.data_ptr(), Ys[0].data_ptr(), N, stream) == 0
+        assert torch.equal(Ys[0], want)
+    ptrs = (ctypes.c_void_p * 2)
+    assert lib.bsr_spmm_batch(ptrs(*(h.ptr for h in hs)), 2, X.data_ptr(), ptrs(bias.data_ptr(), bias.data_ptr()),
+                              ptrs(*(Y.data_ptr() for Y in Ys)), N, stream) == 0
+    assert all(torch.equal(Y, want) for Y in Ys)
+    assert all(h.check_device_status() == 0 for h in hs)
