@@ -92,84 +92,6 @@ bsr_status_t grow(void **buf, size_t *cap, size_t need) {
     return BSR_OK;
 }
 
-// Stream-ordered scratch of one call, from a memory pool of the library's own
-// on the current device. The default pool gives its memory back at every
-// synchronisation, so each conversion mapped its scratch anew; this one keeps
-// up to 16 MB (until the process ends), more is given back.
-cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
-    static std::mutex mu;
-    static std::unordered_map<int, cudaMemPool_t> pools;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    cudaMemPool_t pool = nullptr;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        auto it = pools.find(dev);
-        if (it != pools.end()) {
-            pool = it->second;
-        } else {
-            cudaMemPoolProps props = {};
-            props.allocType = cudaMemAllocationTypePinned;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = dev;
-            if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
-            uint64_t keep = 16ull << 20;
-            if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
-                cudaMemPoolDestroy(pool);
-                return e;
-            }
-            pools[dev] = pool;
-        }
-    }
-    return cudaMallocFromPoolAsync(p, bytes, pool, s);
-}
-
-// One page-locked word for a call, taken from and returned to a list of at
-// most 16 (more are freed), so that calls of several threads have their own.
-struct HostWord {
-    static constexpr size_t kKeep = 16;
-    volatile int32_t *p = nullptr;
-    HostWord() {
-        {
-            std::lock_guard<std::mutex> lk(mu());
-            if (!kept().empty()) {
-                p = kept().back();
-                kept().pop_back();
-                return;
-            }
-        }
-        void *q = nullptr;
-        if (cudaHostAlloc(&q, sizeof(int32_t), cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess)
-            p = static_cast<int32_t *>(q);
-        else
-            cudaGetLastError();
-    }
-    ~HostWord() {
-        if (!p) return;
-        {
-            std::lock_guard<std::mutex> lk(mu());
-            if (kept().size() < kKeep) {
-                kept().push_back(p);
-                return;
-            }
-        }
-        cudaFreeHost((void *)p);
-    }
-    HostWord(const HostWord &) = delete;
-    HostWord &operator=(const HostWord &) = delete;
-
-  private:
-    static std::mutex &mu() {
-        static std::mutex m;
-        return m;
-    }
-    static std::vector<volatile int32_t *> &kept() {
-        static std::vector<volatile int32_t *> v;
-        return v;
-    }
-};
-
 bsr_status_t check_shape(int64_t M, int64_t K, int R, int C, bsr_dtype_t dt) {
     if (dt != BSR_F32 && dt != BSR_BF16) return BSR_ERR_UNSUPPORTED;
     if (M < 0 || K < 0 || R <= 0 || C <= 0) return BSR_ERR_INVALID_ARG;
@@ -337,23 +259,27 @@ bsr_status_t bsr_from_dense(const void *W, int64_t M, int64_t K, int R, int C, f
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
     int32_t *counts = nullptr;   // kept blocks per segment, then each segment's first
-    if (scratch_alloc((void **)&counts, (size_t)std::max<int64_t>(builder_segments(M, K, R, C, dt), 1) * 4, s) !=
+    if (cudaMallocAsync((void **)&counts, (size_t)std::max<int64_t>(builder_segments(M, K, R, C, dt), 1) * 4, s) !=
         cudaSuccess) {
         cudaGetLastError();
         return BSR_ERR_ALLOC;
     }
-    // the scan writes the count into the mapped word: no copy before the synchronisation
-    HostWord word;
-    int32_t last = 0;
-    st = word.p ? BSR_OK : BSR_ERR_ALLOC;
-    if (st == BSR_OK) {
-        if (launch_builder_count(W, dt, M, K, R, C, threshold, counts, indptr, (int32_t *)word.p, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
-            cudaGetLastError();
-            st = BSR_ERR_CUDA;
-        } else {
-            last = *word.p;
-        }
+    // where the GPU reaches the host's memory as it is (GB300's CPU link), the
+    // scan itself writes the count here: 4096 x 4096 fp32, 32x1, query and fill
+    // 98 us, with a copy of one word per call 114
+    volatile int32_t last = 0;
+    int device = 0, reaches = 0;
+    if (cudaGetDevice(&device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&reaches, cudaDevAttrPageableMemoryAccess, device) != cudaSuccess) {
+        cudaGetLastError();
+        reaches = 0;
+    }
+    int32_t *const word = const_cast<int32_t *>(&last);
+    if (launch_builder_count(W, dt, M, K, R, C, threshold, counts, indptr, reaches ? word : nullptr, s) != cudaSuccess ||
+        (!reaches && cudaMemcpyAsync(word, indptr + MB, sizeof *word, cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
+        cudaStreamSynchronize(s) != cudaSuccess) {
+        cudaGetLastError();
+        st = BSR_ERR_CUDA;
     }
     const int64_t nnzb = last;
     if (st == BSR_OK && last < 0) st = BSR_ERR_SHAPE;   // more than 2^31-1 kept blocks

@@ -128,7 +128,7 @@ k_count(const B *__restrict__ W, const Seg s, float thr, int32_t *__restrict__ c
 }
 
 // counts [MB][nseg] -> indptr, in place the first kept block of every segment,
-// and indptr[MB] once more where the host reads it.
+// and indptr[MB] once more in *nnzb (if given).
 __global__ void k_scan(int32_t *__restrict__ counts, int64_t MB, int64_t nseg, int32_t *__restrict__ indptr,
                        int32_t *__restrict__ nnzb) {
     __shared__ int64_t warp_tot[32];
@@ -152,7 +152,7 @@ __global__ void k_scan(int32_t *__restrict__ counts, int64_t MB, int64_t nseg, i
         }
         carry += total;
     }
-    if (threadIdx.x == 0) *nnzb = carry > INT32_MAX ? -1 : (int32_t)carry;
+    if (threadIdx.x == 0 && nnzb) *nnzb = carry > INT32_MAX ? -1 : (int32_t)carry;
 }
 
 template <typename B>  // B: uint32_t (fp32 bits) or uint16_t (bf16 bits)

@@ -2,6 +2,8 @@
 either direction, rows that are not 16-byte aligned, a misaligned W, one and
 many segments per block row, a partly filled last one; bit for bit against the
 oracle, NaN and threshold rule included."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -35,3 +37,22 @@ def test_builder_segments_match_the_oracle(R, C, M, K, dtype, offset):
     for thr in (0.0, 0.03):
         assert_structure_equal(bsr.bsr_from_dense(at, R, C, thr), oracle.bsr_from_dense(W, R, C, thr))
     assert dtype_of(W) == dtype
+
+
+def test_a_conversion_keeps_no_device_memory():
+    """What a call allocates comes from the device's default pool, and all of
+    it is back there afterwards."""
+    import paper_2106_08846_gb300 as bsr
+    W = torch.randn(1024, 4096, device="cuda") * (torch.rand(1024, 4096, device="cuda") < 0.01)
+    torch.cuda.synchronize()
+    cuda = ctypes.CDLL("libcuda.so.1")
+    pool, n = ctypes.c_void_p(), ctypes.c_uint64(0)
+    assert cuda.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    used, used_high = 7, 8   # CU_MEMPOOL_ATTR_USED_MEM_CURRENT, _HIGH
+    assert cuda.cuMemPoolSetAttribute(pool, used_high, ctypes.byref(n)) == 0
+    for R, C in ((1, 1), (32, 1), (16, 16)):
+        indptr, indices, data = bsr.bsr_from_dense(W, R, C)
+        assert indices.numel() == int(indptr[-1]) > 0
+    torch.cuda.synchronize()
+    assert cuda.cuMemPoolGetAttribute(pool, used_high, ctypes.byref(n)) == 0 and n.value > 0
+    assert cuda.cuMemPoolGetAttribute(pool, used, ctypes.byref(n)) == 0 and n.value == 0
