@@ -396,7 +396,7 @@ class Product:
             self.handles.append(h)
             self.biases.append(torch.from_numpy(w.bias).to(dev))
         self.Y = torch.empty((N, weights[0].M), dtype=X.dtype, device=dev)   # every weight here is M x K
-        self.scheds = [h.schedule() for h in self.handles]
+        self.scheds = [dict(h.schedule(), **h.call_info(N)) for h in self.handles]
         self.flops = [2 * N * w.nnz for w in weights]
         self.nbytes = [call_bytes(w, N, self.es) for w in weights]
         self.bsr = bsr
@@ -406,7 +406,7 @@ class Product:
             self.bsr.bsr_spmm(h, self.X, b, self.Y, self.N, stream)
 
     def launches(self):
-        return sum(s["launches_per_call"] for s in self.scheds)
+        return sum(s["launches"] for s in self.scheds)
 
     def check(self):
         for h in self.handles:
@@ -418,13 +418,21 @@ class Product:
             h.destroy()
 
 
+def kernel_of(sc):
+    """The kernel that runs the calls: the schedule's variant where the call did not say."""
+    return sc.get("kernel", sc["variant"])
+
+
+TENSOR_KERNELS = ("tcgen05", "dense", "gk", "tcp")
+
+
 def kernel_key(sc, w):
-    return f"{sc['variant']}_{w.R}x{w.C}_{'bf16' if w.dtype == 'bf16' else 'f32'}"
+    return f"{kernel_of(sc)}_{w.R}x{w.C}_{'bf16' if w.dtype == 'bf16' else 'f32'}"
 
 
 def pipe_peak(sc, dtype, pk, fp32_tflops):
     """(peak FLOP/s, description) of the pipe that bounds this kernel's arithmetic."""
-    if sc["variant"] == "tcgen05":
+    if kernel_of(sc) in TENSOR_KERNELS:
         bf16 = float(pk.get("bf16_tflops_sustained", pk["bf16_tflops"])) * 1e12
         if dtype == "bf16":
             return bf16, f"bf16 tensor, sustained ({pk['source']})"
@@ -538,12 +546,13 @@ def kernel_roofline(d, hbm):
         r = {"bound": "hbm", "achieved": nbytes / t / 1e9, "peak": hbm / 1e9, "unit": "GB/s",
              "peak_source": "HBM copy bandwidth, MEASURED_PEAKS.json"}
     else:
-        r = {"bound": "alu" if sc["variant"] != "tcgen05" else "tensor", "achieved": flops / t / 1e12,
+        r = {"bound": "tensor" if kernel_of(sc) in TENSOR_KERNELS else "alu", "achieved": flops / t / 1e12,
              "peak": d["peak"] / 1e12, "unit": "TFLOP/s", "peak_source": d["peak_desc"]}
     r["frac"] = r["achieved"] / r["peak"]
     r["traffic"] = profiled_traffic(kernel_key(sc, w) + f"_{w.M}x{w.K}")
-    r["kernel"] = (f"{sc['variant']} {w.R}x{w.C} {w.dtype}" +
-                   (f" (exec {sc['exec_R']}x{sc['exec_C']})" if (sc['exec_R'], sc['exec_C']) != (w.R, w.C) else ""))
+    r["kernel"] = f"{kernel_of(sc)} {w.R}x{w.C} {w.dtype}"
+    if kernel_of(sc) == "tcgen05" and (sc["exec_R"], sc["exec_C"]) != (w.R, w.C):
+        r["kernel"] += f" (exec {sc['exec_R']}x{sc['exec_C']})"
     r["us_per_launch"] = t * 1e6
     r["flops_per_launch"] = flops
     r["bytes_per_launch"] = nbytes

@@ -141,14 +141,26 @@ bsr_status_t bsr_spmm(bsr_handle_t h, const void *X, const float *bias, void *Y,
  * error a kernel of this handle recorded (BSR_ERR_TIMEOUT when a bounded
  * wait gave up), then clear it. BSR_OK if none. Structure errors are not
  * reported here: bsr_create validates indptr/indices on the host and the
- * kernels read only the handle's own repacked copy, built from the
- * validated structure.
+ * kernels take the structure from the handle's own copy of what it validated.
  */
 bsr_status_t bsr_check_device_status(bsr_handle_t h);
 
 /*
+ * bsr_get_call_info -- which kernel a bsr_spmm call of N tokens runs, and how
+ * many launches it makes, as "key=value" lines:
+ *   kernel    "xstage" (SIMT, per task), "xcol" (SIMT, column lists), "tcgen05"
+ *             (tensor cores, block by block), "dense" (tensor cores, bf16 weight
+ *             as zero-filled tiles), "gk" (tensor cores, gathered columns),
+ *             "tcp" (opt-in), "generic", or "none" (N = 0)
+ *   launches  kernel launches of the call (with the reduce pass, if any)
+ * Arguments as for bsr_get_schedule; BSR_ERR_INVALID_ARG for N < 0 too.
+ */
+bsr_status_t bsr_get_call_info(bsr_handle_t h, int64_t N, char *buf, size_t len);
+
+/*
  * bsr_get_schedule -- a text description of the handle's schedule: kernel
- * variant, execution block height and width (exec_R x exec_C: max(R, 16) x 64
+ * variant, the kernels that it holds operands for (a call's is chosen from its
+ * token count: bsr_get_call_info), execution block height and width (exec_R x exec_C: max(R, 16) x 64
  * where small or narrow bf16 blocks run on the tensor cores as zero-filled
  * tiles), tile sizes, work items, split
  * rows, launches per call, the schedule-cache statistics and the task sizes
@@ -199,9 +211,10 @@ bsr_status_t bsr_spmm_noalloc(bsr_handle_t h, const void *X, const float *bias, 
  * The paper prunes BERT (Section 2.3), whose self-attention applies several
  * weights (query, key, value) to the same activations; this entry point takes
  * such products together. Products whose weights run on the same kernel
- * configuration -- the SIMT kernel with the same dtype, block shape and task
- * layout for the call's N, or the tensor-core kernel with the same dtype and
- * block height -- are fused into one grid, up to 64 per launch, so one
+ * configuration -- the per-task SIMT kernel with the same dtype, block shape and
+ * task layout for the call's N, the column-list SIMT kernel with the same block
+ * height, the block-by-block tensor-core kernel with the same dtype and block
+ * height, or the dense-tile kernel with any block shapes -- are fused into one grid, up to 64 per launch, so one
  * product's last, partly filled wave overlaps the others' work; products on
  * the generic kernel run one after another on the same stream. Each output
  * is bit-identical to what bsr_spmm gives for the same arguments.

@@ -80,6 +80,8 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
         lib.bsr_check_device_status.restype = U
         lib.bsr_get_schedule.argtypes = [P, ctypes.c_char_p, ctypes.c_size_t]
         lib.bsr_get_schedule.restype = U
+        lib.bsr_get_call_info.argtypes = [P, I64, ctypes.c_char_p, ctypes.c_size_t]
+        lib.bsr_get_call_info.restype = U
         lib.bsr_destroy.argtypes = [P]
         lib.bsr_destroy.restype = None
         lib.bsr_status_str.argtypes = [U]
@@ -176,6 +178,10 @@ class Handle:
 
     def schedule(self) -> dict:
         return parse_schedule(bsr_get_schedule(self))
+
+    def call_info(self, N: int) -> dict:
+        """The kernel that a call of N tokens runs and its launches."""
+        return parse_schedule(bsr_get_call_info(self, N))
 
     def check_device_status(self) -> int:
         return bsr_check_device_status(self)
@@ -347,6 +353,12 @@ def bsr_check_device_status(h: Handle) -> int:
 def bsr_get_schedule(h: Handle) -> str:
     buf = ctypes.create_string_buffer(4096)
     _check(load().bsr_get_schedule(h.ptr, buf, len(buf)), "bsr_get_schedule")
+    return buf.value.decode()
+
+
+def bsr_get_call_info(h: Handle, N: int) -> str:
+    buf = ctypes.create_string_buffer(256)
+    _check(load().bsr_get_call_info(h.ptr, N, buf, len(buf)), "bsr_get_call_info")
     return buf.value.decode()
 
 

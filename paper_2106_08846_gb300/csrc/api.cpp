@@ -696,19 +696,29 @@ bsr_status_t bsr_get_schedule(bsr_handle_t h, char *buf, size_t len) {
         snprintf(xss + at, sizeof xss - at, at ? ",%d" : "%d", kXsG[gi]);
     }
     if (!xss[0]) snprintf(xss, sizeof xss, "none");
+    char kernels[64];   // the variant's own first
+    snprintf(kernels, sizeof kernels, "%s%s%s%s", variant_name(sc.variant), sc.dense.ok ? ",dense" : "",
+             sc.xc.ok ? ",xcol" : "", sc.gk.ok ? ",gk" : "");
     snprintf(buf, len,
-             "variant=%s\ndtype=%s\nR=%d\nC=%d\nexec_R=%d\nexec_C=%d\nM=%" PRId64 "\nK=%" PRId64 "\nMB=%" PRId64
+             "variant=%s\nkernels=%s\ndtype=%s\nR=%d\nC=%d\nexec_R=%d\nexec_C=%d\nM=%" PRId64 "\nK=%" PRId64 "\nMB=%" PRId64
              "\nKB=%" PRId64 "\nnnzb=%" PRId64 "\ntokens_per_cta=%d\nthreads=%d\nsmem_bytes=%zu\n"
              "item_groups=%d\nitems=%zu\nsplit_len=%d\nsplit_rows=%" PRId64 "\nslots=%d\n"
              "empty_rows=%" PRId64 "\nmax_row_blocks=%" PRId64 "\nlaunches_per_call=%d\n"
              "structure_hash=%016" PRIx64 "\ncache_hit=%d\nschedule_reuses=%" PRId64
              "\ncache_hits_total=%" PRId64 "\ncache_misses_total=%" PRId64 "\ntc_stacked_chunks=%s\n"
              "gk_task_sizes=%s\nxstage_task_sizes=%s\n",
-             variant_name(sc.variant), sc.dt == BSR_F32 ? "f32" : "bf16", sc.R, sc.C, sc.ex_R, sc.ex_C, sc.M, sc.K,
+             variant_name(sc.variant), kernels, sc.dt == BSR_F32 ? "f32" : "bf16", sc.R, sc.C, sc.ex_R, sc.ex_C, sc.M, sc.K,
              sc.MB, sc.KB, sc.nnzb, sc.tn, sc.threads, sc.smem, sc.groups, sc.items.size(),
              sc.split_len, split_rows, sc.n_slots, sc.empty_rows, sc.max_row, launches_per_call(sc),
              sc.hash, (int)h->cache_hit, (int64_t)sc.reuse_count, (int64_t)g_cache_hits,
              (int64_t)g_cache_misses, stacks, gks, xss);
+    return BSR_OK;
+}
+
+bsr_status_t bsr_get_call_info(bsr_handle_t h, int64_t N, char *buf, size_t len) {
+    if (!h || N < 0 || !buf || len == 0) return BSR_ERR_INVALID_ARG;
+    const Schedule &sc = *h->sched;
+    snprintf(buf, len, "kernel=%s\nlaunches=%d\n", kernel_name(sc, N), N ? launches_per_call(sc, N) : 0);
     return BSR_OK;
 }
 

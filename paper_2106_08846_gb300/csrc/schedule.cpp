@@ -821,6 +821,16 @@ cudaError_t launch_spmm_batch(const LaunchArgs *as, int n) {
     return cudaSuccess;
 }
 
+// (in the order of launch_spmm)
+const char *kernel_name(const Schedule &sc, int64_t N) {
+    if (N <= 0) return "none";
+    if (choose_gk(sc, N) >= 0) return "gk";
+    if (choose_tcp(sc, N) >= 0) return "tcp";
+    if (choose_xcol(sc, N)) return "xcol";
+    if (choose_dense(sc, N) > 0) return "dense";
+    return variant_name(sc.variant);
+}
+
 cudaError_t launch_spmm(const LaunchArgs &a) {
     const int gG = choose_gk(*a.sc, a.N);
     if (gG >= 0) return launch_gk(a, gG);   // every block row is an item: nothing to reduce

@@ -21,6 +21,9 @@ cudaError_t launch_spmm(const LaunchArgs &a);
 // runs alone. *G receives the task size chosen for N.
 int fusion_class(const Schedule &sc, int64_t N, int *G);
 
+// The kernel that runs a product of N tokens by itself.
+const char *kernel_name(const Schedule &sc, int64_t N);
+
 // Task size of the per-task SIMT kernel for N tokens; *cost: the model's cost of
 // it, in multiply-adds per token.
 int choose_tasks(const Schedule &sc, int64_t N, double *cost = nullptr);
@@ -30,8 +33,9 @@ int choose_tasks(const Schedule &sc, int64_t N, double *cost = nullptr);
 int choose_tc_tasks(const Schedule &sc, int64_t N, double *cost = nullptr);
 
 // Launches n products that share X, N and the stream: products whose kernels
-// share a template (xstage, or tensor-core of one dtype and R) run as one
-// grid, up to 64 at a time; generic-kernel products one after another.
+// share a template (xstage, or tensor-core of one dtype and R; dense of any
+// shapes; xcol of one R) run as one grid, up to 64 at a time; generic-kernel
+// products one after another.
 cudaError_t launch_spmm_batch(const LaunchArgs *as, int n);
 
 }  // namespace bsr

@@ -53,3 +53,19 @@ def test_kernel_roofline_fraction(variant, us, flops, nbytes, bound):
     assert r["frac"] == pytest.approx(r["achieved"] / r["peak"])
     assert r["roofline_frac"] == pytest.approx(max(flops / peak, nbytes / hbm) / t)
     assert r["us_per_launch"] == pytest.approx(us)
+
+
+@pytest.mark.parametrize("variant,kernel,dtype,peak", [
+    ("xstage", "xcol", "f32", 78.7e12),
+    ("xstage", "dense", "bf16", 1700e12),              # sparse narrow blocks on dense tiles
+    ("tcgen05", "dense", "bf16", 1700e12),
+    ("generic", "gk", "f32", 1700e12 * (1.1 / 2.25) / 3),
+])
+def test_the_kernel_of_the_call_names_the_line_and_its_pipe(variant, kernel, dtype, peak):
+    sc = {"variant": variant, "kernel": kernel, "exec_R": 32, "exec_C": 64}
+    w = W(0, 0, 1024, 1024, 32, 1, dtype)
+    assert bench.pipe_peak(sc, dtype, PK, 78.7)[0] == pytest.approx(peak)
+    assert bench.kernel_key(sc, w) == f"{kernel}_32x1_{dtype}"
+    d = {"ms": 1.0, "calls": 1, "flops": 3.44e9, "bytes": 1e6, "peak": peak, "peak_desc": "", "sc": sc, "w": w}
+    r = bench.kernel_roofline(d, 6813.8e9)
+    assert r["kernel"] == f"{kernel} 32x1 {dtype}" and r["bound"] == ("alu" if kernel == "xcol" else "tensor")

@@ -149,17 +149,18 @@ def test_kernels_that_allocate_tensor_memory_follow_one_another():
     before the next may start, and every output is that of the call alone."""
     import paper_2106_08846_gb300 as bsr
     runs = []
-    for i, (R, C, M, K, dt, sp, N) in enumerate([
-            (16, 16, 4096, 4096, "bf16", 98, 200),   # block by block, two CTAs an SM
-            (16, 16, 512, 64, "bf16", 50, 200),      # dense tiles
-            (32, 32, 256, 64, "f32", 0, 200),        # block by block, fp32
-            (64, 1, 512, 768, "f32", 85, 1000),      # gathered K
-            (32, 1, 1024, 768, "f32", 50, 2000),     # column lists
-            (64, 64, 512, 192, "bf16", 0, 700)]):
+    for i, (kernel, R, C, M, K, dt, sp, N) in enumerate([
+            ("tcgen05", 16, 16, 4096, 4096, "bf16", 97, 2048),   # two CTAs an SM
+            ("dense", 16, 16, 512, 64, "bf16", 50, 200),
+            ("tcgen05", 32, 32, 256, 64, "f32", 0, 200),
+            ("gk", 64, 1, 512, 768, "f32", 85, 1000),
+            ("xcol", 32, 1, 1024, 768, "f32", 50, 2000),
+            ("dense", 64, 64, 512, 192, "bf16", 0, 700)]):
         w = synth.make_weight("tm", 8200 + i, M, K, R, C, dt, sp)
         h = bsr.bsr_create(*build_on_gpu(w.W, R, C), R, C, M, K)
         X = to_dev(synth.activations(8300 + i, N, K, dt))
         h.reserve(N)
+        assert h.call_info(N)["kernel"] == kernel
         Y = h.spmm(X, to_dev(w.bias))
         torch.cuda.synchronize()
         runs.append((h, X, to_dev(w.bias), Y, torch.empty((8, *Y.shape), dtype=Y.dtype, device="cuda")))
@@ -209,7 +210,7 @@ def test_dense_non_finite_tokens_at_large_k(R, C, share, monkeypatch):
     assert fin.mean() > 0.5 and np.array_equal(np.isfinite(got), fin)
     assert np.array_equal(got[~fin], want[~fin], equal_nan=True)
     E = oracle.err_bound(*ref, np.where(np.isfinite(as_f64(Xs)), Xs, 0).astype(np.uint16), w.bias, M)
-    assert np.all(np.abs(got - want)[fin] <= 1e-2 * E[fin])
+    assert np.all(np.abs(got[fin] - want[fin]) <= 1e-2 * E[fin])
 
 
 @pytest.mark.parametrize("M,K", [(0, 64), (64, 0), (0, 0)])

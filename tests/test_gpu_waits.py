@@ -11,13 +11,13 @@ from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
 pytestmark = pytest.mark.gpu
 
 LIMIT_NS = 1_000_000
-SHAPES = {   # R, C, M, K, dtype, sparsity, N: more chunks than a ring has stages
-    "dense": (16, 16, 1024, 1536, "bf16", 80, 600),
-    "tc_bf16": (16, 16, 4096, 4096, "bf16", 98, 200),
-    "tc_f32": (32, 32, 512, 1536, "f32", 50, 300),
-    "xcol": (32, 1, 1024, 1536, "f32", 50, 3000),
-    "xstage": (8, 1, 512, 1536, "f32", 80, 300),
-    "gk": (64, 1, 512, 1536, "f32", 85, 1000),
+SHAPES = {   # the kernel; R, C, M, K, dtype, sparsity, N: more chunks than a ring has stages
+    "dense": ("dense", 16, 16, 1024, 1536, "bf16", 80, 600),
+    "tc_bf16": ("tcgen05", 16, 16, 4096, 4096, "bf16", 97, 2048),
+    "tc_f32": ("tcgen05", 32, 32, 512, 1536, "f32", 50, 300),
+    "xcol": ("xcol", 32, 1, 1024, 1536, "f32", 50, 3000),
+    "xstage": ("xstage", 8, 1, 512, 1536, "f32", 80, 300),
+    "gk": ("gk", 64, 1, 512, 1536, "f32", 85, 1000),
 }
 
 
@@ -45,7 +45,7 @@ def slow():
 @pytest.mark.parametrize("kind", list(SHAPES))
 def test_a_limit_does_not_run_while_the_previous_kernel_does(slow, kind, monkeypatch):
     import paper_2106_08846_gb300 as bsr
-    R, C, M, K, dt, sp, N = SHAPES[kind]
+    kernel, R, C, M, K, dt, sp, N = SHAPES[kind]
     w = synth.make_weight("wt", 8400 + R, M, K, R, C, dt, sp)
     gpu = build_on_gpu(w.W, R, C)
     monkeypatch.setenv("BSR_WAIT_LIMIT_NS", str(LIMIT_NS))
@@ -54,6 +54,7 @@ def test_a_limit_does_not_run_while_the_previous_kernel_does(slow, kind, monkeyp
     X = synth.activations(8500, N, K, dt)
     Xd, b = to_dev(X), to_dev(w.bias)
     h.reserve(N)
+    assert h.call_info(N)["kernel"] == kernel
     Y = h.spmm(Xd, b)
     torch.cuda.synchronize()
     for _ in range(3):
