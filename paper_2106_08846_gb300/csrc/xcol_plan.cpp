@@ -9,6 +9,28 @@
 
 namespace bsr {
 
+namespace {
+
+int xcol_mode() {
+    static const int mode = [] {
+        const char *v = getenv("BSR_XC"), *t = getenv("BSR_XC_TILE");
+        if (v && *v && atoi(v) == 0) return 0;
+        return (v && *v && atoi(v) == 1) || (t && *t) ? 1 : -1;   // 0: never, 1: always
+    }();
+    return mode;
+}
+
+bool model_takes(const Schedule &sc, int64_t N);
+
+// The blocks [p, p1) of an item that lie in chunk c, from its first not packed yet.
+int32_t chunk_end(const Schedule &sc, const Item &it, int32_t p, int64_t c) {
+    while (p < it.p1 && (int64_t)sc.indices[(size_t)p] * sc.C < (c + 1) * kXcChunk) p++;
+    return p;
+}
+
+}  // namespace
+
+// Nothing is kept (or packed) of a plan that no call would use.
 int64_t plan_xcol(Schedule &sc, int64_t base) {
     XcPlan &pl = sc.xc;
     pl.ok = false;
@@ -16,15 +38,45 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     // (wider blocks: the per-task kernel loads four activations at a time; 16x16 of
     // 768 x 768 at 70%, 4000 tokens 53 us against 71 here, 32x8 at 80% 36 against 39)
     if (sc.dt != BSR_F32 || (sc.R != 16 && sc.R != 32) || sc.C > 4 || kXcChunk % sc.C || sc.K % 4 || n_items == 0 ||
-        sc.variant != V_XSTAGE || sc.nnzb > INT32_MAX / 256 / sc.C)
+        sc.variant != V_XSTAGE || sc.nnzb > INT32_MAX / 256 / sc.C || xcol_mode() == 0)
         return base;
     const int64_t nch = (sc.K + kXcChunk - 1) / kXcChunk;
+    // sizes first
+    double longest = 0.0, apart = 0.0;   // of the items' blocks; from their mean
+    const double mean = (double)sc.nnzb / (double)n_items;
+    for (const Item &it : sc.items) {
+        longest = std::max(longest, (double)(it.p1 - it.p0));
+        apart += std::abs((double)(it.p1 - it.p0) - mean);
+    }
+    pl.even = longest <= 1.5 * mean && apart <= 0.25 * (double)sc.nnzb;
+    if (!pl.even && xcol_mode() != 1) return base;
+    int64_t ints = 0, most_columns = 0;   // 4-byte places
+    for (const Item &it : sc.items) {
+        int32_t p = it.p0;
+        for (int64_t c = 0; c < nch; c++) {
+            const int32_t p1 = chunk_end(sc, it, p, c);
+            const int64_t n = (int64_t)(p1 - p) * sc.C;
+            ints += 4 + ((n + 3) & ~int64_t(3)) + sc.R * n;
+            most_columns = std::max(most_columns, n);
+            p = p1;
+        }
+        if (ints > INT32_MAX / 2) return base;
+    }
+    pl.item_bytes = (uint32_t)((4 + ((most_columns + 3) & ~int64_t(3)) + sc.R * most_columns) * 4);
+    if (2 * xcol_stage_bytes(pl.item_bytes, kXcWarps) > kXcRoom) return base;   // a ring of two stages
+    // equal segments of at most 40 columns, or one chunk: outputs are then no
+    // further from 64 bits than the per-task kernel's, which shares a row among
+    // warps (relative errors of ten sizes 0.98 to 1.37e-7, the per-task kernel's 1.16
+    // to 1.43e-7; at 52 columns 1.17 to 1.47e-7, in one chain of 102 1.8e-7)
+    const double per_chunk = (double)sc.nnzb * sc.C / (double)(n_items * nch);
+    const int64_t most = per_chunk * (double)nch <= 40.0 ? nch : std::max<int64_t>(1, (int64_t)(40.0 / per_chunk));
+    const int64_t segs = (nch + most - 1) / most;
+    pl.seg = (int)((nch + segs - 1) / segs);
+    bool used = xcol_mode() == 1;   // by a call of some size
+    for (int64_t N = 64; !used && N <= (int64_t)1 << 21; N += std::max<int64_t>(64, N / 640 * 64)) used = model_takes(sc, N);
+    if (!used) return base;
     pl.off = (base + 1023) & ~int64_t(1023);
-    pl.table.clear();
-    pl.ints.clear();
-    pl.src.clear();
-    pl.item_bytes = 0;
-    int64_t at = 0;   // 4-byte places
+    int64_t at = 0;
     auto put = [&](int64_t place, int64_t v) {
         pl.ints.push_back((int32_t)place);
         pl.ints.push_back((int32_t)v);
@@ -33,9 +85,8 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     for (size_t i = 0; i < sc.items.size(); i++) next[i] = sc.items[i].p0;
     for (int64_t c = 0; c < nch; c++) {
         for (size_t i = 0; i < sc.items.size(); i++) {
-            const Item &it = sc.items[i];
-            int32_t &p = next[i], p1 = p;
-            while (p1 < it.p1 && (int64_t)sc.indices[(size_t)p1] * sc.C < (c + 1) * kXcChunk) p1++;
+            int32_t &p = next[i];
+            const int32_t p1 = chunk_end(sc, sc.items[i], p, c);
             const int64_t n = (int64_t)(p1 - p) * sc.C, vals = at + 4 + ((n + 3) & ~int64_t(3));
             pl.table.push_back((int32_t)(at / 4));
             put(at, n);
@@ -47,30 +98,11 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
                 pl.src.push_back((int32_t)(block * sc.C + in));
             }
             p = p1;
-            const int64_t end = vals + sc.R * n;
-            pl.item_bytes = std::max(pl.item_bytes, (uint32_t)((end - at) * 4));
-            at = end;
-            if (at > (int64_t)INT32_MAX / 2) return base;
+            at = vals + sc.R * n;
         }
     }
     pl.table.push_back((int32_t)(at / 4));
     pl.bytes = at * 4;
-    // equal segments of at most 40 columns, or one chunk: outputs are then no
-    // further from 64 bits than the per-task kernel's, which shares a row among
-    // warps (relative errors of ten sizes 0.98 to 1.37e-7, the per-task kernel's 1.16
-    // to 1.43e-7; at 52 columns 1.17 to 1.47e-7, in one chain of 102 1.8e-7)
-    const double per_chunk = (double)sc.nnzb * sc.C / (double)(n_items * nch);
-    const int64_t most = per_chunk * (double)nch <= 40.0 ? nch : std::max<int64_t>(1, (int64_t)(40.0 / per_chunk));
-    const int64_t segs = (nch + most - 1) / most;
-    pl.seg = (int)((nch + segs - 1) / segs);
-    double longest = 0.0, apart = 0.0;   // of the items' blocks; from their mean
-    const double mean = (double)sc.nnzb / (double)n_items;
-    for (const Item &it : sc.items) {
-        longest = std::max(longest, (double)(it.p1 - it.p0));
-        apart += std::abs((double)(it.p1 - it.p0) - mean);
-    }
-    pl.even = longest <= 1.5 * mean && apart <= 0.25 * (double)sc.nnzb;
-    if (2 * xcol_stage_bytes(pl.item_bytes, kXcWarps) > kXcRoom) return base;   // a ring of two stages
     pl.ok = true;
     return pl.off + pl.bytes;
 }
@@ -129,6 +161,8 @@ XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N) {
     return best;
 }
 
+namespace {
+
 // Against the per-task kernel, which takes its tasks' work and about 8500 + 4000 / G
 // cycles for each (G items a task; partly filled waves overlap). Measured (us, this
 // kernel and the per-task one): 1024 x 1024 at 90%, 16384 tokens 101 and 123, 4096
@@ -140,33 +174,31 @@ XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N) {
 // 1024 x 1024 at 90%, 16384 tokens 115 and 134; of 768 x 768 at 70%, 3000 tokens 32
 // and 41; 16x4 of 1024 x 1024 at 80%, 3000 tokens 43 and 60; 32x2 at 90%, 8000 tokens
 // 59 and 72.
-bool choose_xcol(const Schedule &sc, int64_t N) {
-    static const int mode = [] {
-        const char *v = getenv("BSR_XC");
-        return v && *v ? atoi(v) : -1;   // 0: never, 1: always
-    }();
-    static const bool forced = [] {
-        const char *v = getenv("BSR_XC_TILE");
-        return v && *v;
-    }();
-    const XcPlan &pl = sc.xc;
-    if (!pl.ok || N <= 0 || mode == 0) return false;
-    if (forced || mode == 1) return true;
-    // (the choice for the last N asked, which is what a steady stream of calls asks again)
-    const uint64_t memo = pl.last.load(std::memory_order_relaxed);
-    if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return memo & 1;
+bool model_takes(const Schedule &sc, int64_t N) {
     // rows of unequal length stay, because an item is one warp's here (pruned at
     // random, the longest row is below 1.5 means from about 40 columns on, and rows
     // are 0.15 means apart or less; 16x1 Zipf rows of 1024 x 1024 at 80%, 3000 tokens
     // 141 us, per-task 73)
-    if (!pl.even) return false;
+    if (!sc.xc.even) return false;
     const Schedule *one = &sc;
     double cost = 0.0;
     const int G = choose_tasks(sc, N, &cost);
     const int64_t items = (int64_t)sc.items.size(), tasks = (items + G - 1) / G;
     const double waves = (double)((N + kXsTokens - 1) / kXsTokens * tasks) / (double)sc.sm_count;
     const double work = (double)sc.nnzb * sc.R * sc.C / (double)tasks;
-    const bool yes = xcol_shape(&one, 1, N).cycles < std::max(1.0, waves) * (8500.0 + 4000.0 / G + work);
+    return xcol_shape(&one, 1, N).cycles < std::max(1.0, waves) * (8500.0 + 4000.0 / G + work);
+}
+
+}  // namespace
+
+bool choose_xcol(const Schedule &sc, int64_t N) {
+    const XcPlan &pl = sc.xc;
+    if (!pl.ok || N <= 0) return false;
+    if (xcol_mode() == 1) return true;
+    // (the choice for the last N asked, which is what a steady stream of calls asks again)
+    const uint64_t memo = pl.last.load(std::memory_order_relaxed);
+    if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return memo & 1;
+    const bool yes = model_takes(sc, N);
     if (N < (int64_t)1 << 48) pl.last.store((uint64_t)N << 16 | (uint64_t)yes, std::memory_order_relaxed);
     return yes;
 }

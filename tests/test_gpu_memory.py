@@ -27,23 +27,31 @@ torch.cuda.synchronize()
 before = torch.cuda.mem_get_info()[0]
 h = bsr.bsr_create(*arrays, R, C, M, K)
 torch.cuda.synchronize()
-print(before - torch.cuda.mem_get_info()[0])
+print(before - torch.cuda.mem_get_info()[0], h.schedule()["kernels"])
 """
 
 
 def held(weight, **env):
-    """Device bytes that creating the weight's handle takes."""
+    """Device bytes that creating the weight's handle takes, and the kernels it holds operands for."""
     r = subprocess.run([sys.executable, "-c", CODE, weight], cwd=ROOT, env=dict(os.environ, **env), capture_output=True,
                        text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-3000:]
-    return int(r.stdout)
+    n, kernels = r.stdout.split()
+    return int(n), kernels.split(",")
 
 
-@pytest.mark.parametrize("weight,off", [
-    # unequal rows, and a row that fills the ring's stages: never column lists
-    ("(32, 1, 4096, 4096, torch.float32, 0.1, 1)", "BSR_XC"),
-    ("(32, 1, 4096, 4096, torch.float32, 0.1, 2)", "BSR_XC"),
-    ("(16, 2, 4096, 4096, torch.float32, 0.002, 0)", "BSR_XC"),
+@pytest.mark.parametrize("weight,kernel,off", [
+    # column lists: not for unequal rows, a row that fills the ring's stages, few columns a chunk
+    ("(32, 1, 4096, 4096, torch.float32, 0.1, 1)", "xcol", "BSR_XC"),
+    ("(32, 1, 4096, 4096, torch.float32, 0.1, 2)", "xcol", "BSR_XC"),
+    ("(16, 2, 4096, 4096, torch.float32, 0.002, 0)", "xcol", "BSR_XC"),
 ])
-def test_no_memory_for_a_kernel_that_no_call_runs(weight, off):
-    assert held(weight) == held(weight, **{off: "0"})
+def test_no_memory_for_a_kernel_that_no_call_runs(weight, kernel, off):
+    n, kernels = held(weight)
+    assert kernel not in kernels
+    assert n == held(weight, **{off: "0"})[0]
+
+
+def test_operands_of_a_kernel_that_calls_run():
+    assert "xcol" in held("(32, 1, 1024, 1024, torch.float32, 0.1, 0)")[1]
+    assert "dense" in held("(16, 16, 1024, 1024, torch.bfloat16, 0.1, 0)")[1]
