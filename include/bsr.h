@@ -105,8 +105,10 @@ bsr_status_t bsr_from_dense(const void *W, int64_t M, int64_t K, int R, int C, f
  * indices, synchronous): indptr[0] == 0, non-decreasing, indices strictly
  * ascending per row and < K/C; otherwise BSR_ERR_STRUCTURE.
  * Owns: the schedule (shared with other handles of identical structure),
- * the work list, a repacked copy of data in the kernels' layout, a device
- * status word and workspaces. *out receives the handle.
+ * the work list, copies of data in the layouts of the kernels that calls may
+ * run (bf16 weights among them as zero-filled rows of K: up to 2 M K bytes,
+ * where that is at most 1 GB or 64 times the blocks), a device status word and
+ * workspaces. *out receives the handle.
  */
 bsr_status_t bsr_create(const int32_t *indptr, const int32_t *indices, const void *data, int R,
                         int C, int64_t M, int64_t K, bsr_dtype_t dt, bsr_handle_t *out);

@@ -8,60 +8,86 @@
 
 namespace bsr {
 
+namespace {
+
+int dense_mode() {
+    static const int mode = [] {
+        const char *v = getenv("BSR_DENSE");
+        return v && *v ? atoi(v) : -1;   // 0: never, 1: always, unset: by the model
+    }();
+    return mode;
+}
+
+int forced_groups() {
+    static const int forced = [] {
+        const char *v = getenv("BSR_DENSE_G");
+        const int f = v ? atoi(v) : 0, g = f & ~kDnPair;
+        return g >= 1 && g <= kDnMaxGroups && !((f & kDnPair) && g % 2) ? f : 0;
+    }();
+    return forced;
+}
+
+int model_takes(const Schedule &sc, int64_t N);
+
+}  // namespace
+
+// Nothing is kept (or packed) of a plan that no call would use.
 int64_t plan_dense(Schedule &sc, int64_t base) {
     DensePlan &pl = sc.dense;
     pl.ok = false;
     const bool shape_ok = kDnGroup % sc.R == 0 || sc.R % kDnGroup == 0;
     if ((sc.variant != V_TC && sc.variant != V_XSTAGE) || sc.dt != BSR_BF16 || sc.M == 0 || sc.M % kDnGroup || sc.K % 8 ||
-        !shape_ok)
+        !shape_ok || dense_mode() == 0)
         return base;
     const int64_t n_groups = sc.M / kDnGroup, nch = (sc.K + kDnChunk - 1) / kDnChunk;
     if (n_groups > INT32_MAX / 32 || nch > 1 << 20) return base;
-    // per row group, the chunks that hold a kept block (a byte each)
-    std::vector<uint8_t> used((size_t)(n_groups * nch), 0);
-    for (int64_t i = 0; i < sc.MB; i++) {
-        const int64_t gl = i * sc.R / kDnGroup, gh = (i * sc.R + sc.R - 1) / kDnGroup;
-        for (int32_t p = sc.indptr[(size_t)i]; p < sc.indptr[(size_t)i + 1]; p++) {
-            const int64_t col = (int64_t)sc.indices[(size_t)p] * sc.C;
-            for (int64_t c = col / kDnChunk; c <= (col + sc.C - 1) / kDnChunk; c++)
-                for (int64_t g = gl; g <= gh; g++) used[(size_t)(g * nch + c)] = 1;
-        }
+    // groups with blocks first, in row order (a task's outputs are then runs of Y)
+    std::vector<int32_t> rows, empty;
+    for (int64_t g = 0; g < n_groups; g++) {
+        const int64_t i0 = g * kDnGroup / sc.R, i1 = (g * kDnGroup + kDnGroup - 1) / sc.R;
+        (sc.indptr[(size_t)i1 + 1] > sc.indptr[(size_t)i0] ? rows : empty).push_back((int32_t)g);
     }
-    std::vector<int32_t> count((size_t)n_groups, 0);
-    for (int64_t g = 0; g < n_groups; g++)
-        for (int64_t c = 0; c < nch; c++) count[(size_t)g] += used[(size_t)(g * nch + c)];
-    // groups with blocks first, in row order (a task's outputs are then runs of
-    // Y, which the kernel stores in 64-column boxes); by their chunk counts
-    // where full-width tasks then visit a fifth fewer chunks (long groups share
-    // tasks and short ones leave chunks out)
-    pl.group_row.resize((size_t)n_groups);
-    for (int64_t g = 0; g < n_groups; g++) pl.group_row[(size_t)g] = (int32_t)g;
-    std::vector<int32_t> sorted = pl.group_row;
-    auto more = [&](int32_t x, int32_t y) { return count[(size_t)x] > count[(size_t)y]; };
-    auto some = [&](int32_t x, int32_t y) { return (count[(size_t)x] > 0) > (count[(size_t)y] > 0); };
-    std::stable_sort(pl.group_row.begin(), pl.group_row.end(), some);
-    std::stable_sort(sorted.begin(), sorted.end(), more);
+    const int64_t n_full = (int64_t)rows.size();
+    pl.w_bytes = std::max<int64_t>(n_full, 1) * kDnGroup * sc.K * 2;
+    if (pl.w_bytes > (int64_t)1 << 30 && pl.w_bytes > sc.nnzb * sc.R * sc.C * 128) return base;   // 64 times the blocks
+    // per group with blocks, the chunks that hold one (a byte each)
+    std::vector<uint8_t> used((size_t)(n_full * nch), 0);
+    std::vector<int32_t> count((size_t)n_full, 0);
+    for (int64_t k = 0; k < n_full; k++) {
+        uint8_t *u = &used[(size_t)(k * nch)];
+        const int64_t r0 = (int64_t)rows[(size_t)k] * kDnGroup;
+        for (int64_t i = r0 / sc.R; i <= (r0 + kDnGroup - 1) / sc.R; i++)
+            for (int32_t p = sc.indptr[(size_t)i]; p < sc.indptr[(size_t)i + 1]; p++) {
+                const int64_t col = (int64_t)sc.indices[(size_t)p] * sc.C;
+                for (int64_t c = col / kDnChunk; c <= (col + sc.C - 1) / kDnChunk; c++) u[c] = 1;
+            }
+        count[(size_t)k] = (int32_t)std::count(u, u + nch, 1);
+    }
+    // by their chunk counts where full-width tasks then visit a fifth fewer
+    // chunks (long groups share tasks and short ones leave chunks out)
+    std::vector<int32_t> order((size_t)n_full), sorted;
+    for (int64_t k = 0; k < n_full; k++) order[(size_t)k] = (int32_t)k;
+    sorted = order;
+    std::stable_sort(sorted.begin(), sorted.end(),
+                     [&](int32_t x, int32_t y) { return count[(size_t)x] > count[(size_t)y]; });
     std::vector<uint8_t> any((size_t)nch);
     // the chunks of the task of groups [k0, k1) in an order
-    auto unite = [&](const std::vector<int32_t> &order, int64_t k0, int64_t k1) {
+    auto unite = [&](const std::vector<int32_t> &o, int64_t k0, int64_t k1) {
         std::fill(any.begin(), any.end(), 0);
-        for (int64_t k = k0; k < k1; k++) {
-            const uint8_t *u = &used[(size_t)(order[(size_t)k] * nch)];
+        for (int64_t k = k0; k < std::min(n_full, k1); k++) {
+            const uint8_t *u = &used[(size_t)(o[(size_t)k] * nch)];
             for (int64_t c = 0; c < nch; c++) any[(size_t)c] |= u[c];
         }
         return std::count(any.begin(), any.end(), 1);
     };
     int64_t in_rows = 0, in_count = 0;
-    for (int64_t k = 0; k < n_groups; k += kDnMaxGroups) {
-        in_rows += unite(pl.group_row, k, std::min(n_groups, k + kDnMaxGroups));
-        in_count += unite(sorted, k, std::min(n_groups, k + kDnMaxGroups));
+    for (int64_t k = 0; k < n_full; k += kDnMaxGroups) {
+        in_rows += unite(order, k, k + kDnMaxGroups);
+        in_count += unite(sorted, k, k + kDnMaxGroups);
     }
-    if (in_count < in_rows - in_rows / 5) pl.group_row = sorted;
-    pl.group_pos.resize((size_t)n_groups);
-    for (int64_t k = 0; k < n_groups; k++) pl.group_pos[(size_t)pl.group_row[(size_t)k]] = (int32_t)k;
+    if (in_count < in_rows - in_rows / 5) order.swap(sorted);
     pl.n_groups = (int)n_groups;
-    pl.n_full = (int)std::count_if(count.begin(), count.end(), [](int32_t c) { return c > 0; });
-    pl.table.clear();
+    pl.n_full = (int)n_full;
     for (int g = 1; g <= kDnMaxGroups; g++) {
         const int64_t tasks = (n_groups + g - 1) / g;
         const size_t at = pl.table.size();
@@ -72,21 +98,34 @@ int64_t plan_dense(Schedule &sc, int64_t base) {
         pl.table.resize(at + (size_t)tasks + 1);
         for (int64_t t = 0; t < tasks; t++) {
             pl.table[at + (size_t)t] = (int32_t)(pl.table.size() - at);
-            const int32_t n = (int32_t)unite(pl.group_row, t * g, std::min(n_groups, t * g + g));
+            if (t * g >= n_full) continue;
+            const int32_t n = (int32_t)unite(order, t * g, t * g + g);
             for (int64_t c = 0; c < nch; c++)
                 if (any[(size_t)c]) pl.table.push_back((int32_t)c);
             pl.chunks[g] += n;
             pl.max_chunks[g] = std::max(pl.max_chunks[g], n);
         }
         pl.table[at + (size_t)tasks] = (int32_t)(pl.table.size() - at);
-        if (pl.table.size() > (size_t)INT32_MAX / 4) return base;
+        if (pl.table.size() > (size_t)INT32_MAX / 4) break;
     }
+    bool used_by_some = dense_mode() == 1 || forced_groups() > 0;   // token count
+    for (int64_t N = 16; !used_by_some && N <= (int64_t)1 << 21; N += std::max<int64_t>(64, N / 640 * 64))
+        used_by_some = model_takes(sc, N) > 0;
+    if (pl.table.size() > (size_t)INT32_MAX / 4 || !used_by_some) {
+        std::vector<int32_t>().swap(pl.table);
+        return base;
+    }
+    pl.group_row.reserve((size_t)n_groups);
+    for (int32_t k : order) pl.group_row.push_back(rows[(size_t)k]);
+    pl.group_row.insert(pl.group_row.end(), empty.begin(), empty.end());
+    pl.group_pos.resize((size_t)n_groups);
+    for (int64_t k = 0; k < n_groups; k++) pl.group_pos[(size_t)pl.group_row[(size_t)k]] = (int32_t)k;
     pl.w_off = (base + 1023) & ~int64_t(1023);
-    pl.w_bytes = (int64_t)std::max(pl.n_full, 1) * kDnGroup * sc.K * 2;
-    if (pl.w_bytes > (int64_t)1 << 30 && pl.w_bytes > sc.nnzb * sc.R * sc.C * 128) return base;   // 64 times the blocks
     pl.ok = true;
     return pl.w_off + pl.w_bytes;
 }
+
+namespace {
 
 // The busiest SM's cycles at each task size, and the least of them against the
 // block-by-block kernel's. A chunk costs about 250 + 34 g cycles (one CTA) or
@@ -104,22 +143,8 @@ int64_t plan_dense(Schedule &sc, int64_t base) {
 // block kernel have the per-task SIMT kernel beside this one, at about 0.85
 // cycles per unit of its model: 32x1 of 1024 x 1024 at 95%, 16384 tokens, 26.2
 // against 69 us.
-int choose_dense(const Schedule &sc, int64_t N) {
-    static const int mode = [] {
-        const char *v = getenv("BSR_DENSE");
-        return v && *v ? atoi(v) : -1;   // 0: never, 1: always, unset: by the model
-    }();
-    static const int forced = [] {
-        const char *v = getenv("BSR_DENSE_G");
-        return v ? atoi(v) : 0;
-    }();
+int model_takes(const Schedule &sc, int64_t N) {
     const DensePlan &pl = sc.dense;
-    if (!pl.ok || N <= 0 || mode == 0) return 0;
-    const int fg = forced & ~kDnPair;
-    if (fg >= 1 && fg <= kDnMaxGroups && !((forced & kDnPair) && fg % 2)) return forced;
-    // (the choice for the last N asked, which is what a steady stream of calls asks again)
-    const uint64_t memo = pl.last.load(std::memory_order_relaxed);
-    if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return (int)(memo & 0xffff);
     int best = 1;
     double best_cost = -1.0;
     for (int pair = 0; pair <= (N > kDnTokens && sc.sm_count >= 2 ? 1 : 0); pair++) {
@@ -158,7 +183,19 @@ int choose_dense(const Schedule &sc, int64_t N) {
         choose_tasks(sc, N, &other);
         other *= 0.85;
     }
-    if (mode != 1 && other > 0 && best_cost > other) best = 0;
+    return dense_mode() != 1 && other > 0 && best_cost > other ? 0 : best;
+}
+
+}  // namespace
+
+int choose_dense(const Schedule &sc, int64_t N) {
+    const DensePlan &pl = sc.dense;
+    if (!pl.ok || N <= 0) return 0;
+    if (forced_groups()) return forced_groups();
+    // (the choice for the last N asked, which is what a steady stream of calls asks again)
+    const uint64_t memo = pl.last.load(std::memory_order_relaxed);
+    if (N < (int64_t)1 << 48 && memo >> 16 == (uint64_t)N) return (int)(memo & 0xffff);
+    const int best = model_takes(sc, N);
     if (N < (int64_t)1 << 48) pl.last.store((uint64_t)N << 16 | (uint64_t)best, std::memory_order_relaxed);
     return best;
 }

@@ -45,6 +45,9 @@ def held(weight, **env):
     ("(32, 1, 4096, 4096, torch.float32, 0.1, 1)", "xcol", "BSR_XC"),
     ("(32, 1, 4096, 4096, torch.float32, 0.1, 2)", "xcol", "BSR_XC"),
     ("(16, 2, 4096, 4096, torch.float32, 0.002, 0)", "xcol", "BSR_XC"),
+    # dense tiles: not for wide weights too sparse for them at any token count
+    ("(32, 1, 8192, 8192, torch.bfloat16, 0.01, 0)", "dense", "BSR_DENSE"),
+    ("(1, 1, 8192, 8192, torch.bfloat16, 0.005, 0)", "dense", "BSR_DENSE"),
 ])
 def test_no_memory_for_a_kernel_that_no_call_runs(weight, kernel, off):
     n, kernels = held(weight)
