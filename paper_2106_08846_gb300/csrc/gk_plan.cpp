@@ -27,6 +27,14 @@ int32_t stage_offset(bsr_dtype_t dt, int64_t kk) {
     return (int32_t)((kk / box_cols) * (128 * 128) + (kk % box_cols) * es);
 }
 
+int gk_mode() {   // 0: never, 1: every shape it supports, else: the generic kernel's shapes
+    static const int mode = [] {
+        const char *v = getenv("BSR_GK");
+        return v ? atoi(v) : -1;
+    }();
+    return mode;
+}
+
 }  // namespace
 
 // Every block row is an item (empty rows too: their outputs are the bias).
@@ -52,6 +60,7 @@ void plan_gk(Schedule &sc, int64_t packed_end) {
         pl.pstage[gi] = 0;
     }
     if (packed_end < 0 || !gk_supports(sc.R, sc.C, sc.dt, sc.K) || sc.MB == 0 || sc.nnzb == 0) return;
+    if (gk_mode() != 1 && (gk_mode() == 0 || sc.variant != V_GENERIC)) return;   // no call would run it
     const bool f32 = sc.dt == BSR_F32;
     const int64_t KC = gk_chunk_cols(sc.dt), KS = gk_kslice(sc.dt);
     const int64_t nch = (sc.K + KC - 1) / KC;
@@ -279,10 +288,7 @@ void plan_gk(Schedule &sc, int64_t packed_end) {
 // kernels measured faster. BSR_GK=0 turns it off, BSR_GK=1 uses it whenever
 // it fits; BSR_GK_G forces a task size.
 int choose_gk(const Schedule &sc, int64_t N) {
-    static const int mode = [] {
-        const char *v = getenv("BSR_GK");
-        return v ? atoi(v) : -1;
-    }();
+    const int mode = gk_mode();
     static const int forced = [] {
         const char *v = getenv("BSR_GK_G");
         return v ? atoi(v) : 0;

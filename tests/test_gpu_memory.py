@@ -48,6 +48,9 @@ def held(weight, **env):
     # dense tiles: not for wide weights too sparse for them at any token count
     ("(32, 1, 8192, 8192, torch.bfloat16, 0.01, 0)", "dense", "BSR_DENSE"),
     ("(1, 1, 8192, 8192, torch.bfloat16, 0.005, 0)", "dense", "BSR_DENSE"),
+    # gathered columns: only for the shapes that are otherwise the generic kernel's
+    ("(16, 16, 4096, 4096, torch.bfloat16, 0.1, 0)", "gk", "BSR_GK"),
+    ("(32, 1, 4096, 4096, torch.float32, 0.1, 0)", "gk", "BSR_GK"),
 ])
 def test_no_memory_for_a_kernel_that_no_call_runs(weight, kernel, off):
     n, kernels = held(weight)
@@ -57,4 +60,5 @@ def test_no_memory_for_a_kernel_that_no_call_runs(weight, kernel, off):
 
 def test_operands_of_a_kernel_that_calls_run():
     assert "xcol" in held("(32, 1, 1024, 1024, torch.float32, 0.1, 0)")[1]
+    assert "gk" in held("(64, 1, 512, 768, torch.float32, 0.1, 0)")[1]
     assert "dense" in held("(16, 16, 1024, 1024, torch.bfloat16, 0.1, 0)")[1]
