@@ -27,18 +27,19 @@
 // launch chooses both for all of its products together: few items a task spread a
 // small call over the SMs (768 x 768 at 50%, 1024 tokens 43 -> 30 us), 48 products
 // of 1024 tokens fill the GPU with larger ones (plan of 48 weights at 50 to 95%, of
-// which those at 50% run here, 616 -> 486 us).
+// which those at 50% run here, 617 -> 499 us).
 // Items of a task are neighbours in length, so warps stay within the ring of one
 // another.
 //
 // So that an output is not one long chain of additions, a warp adds its tile to
 // a running sum after every segment of chunks (at most about 40 columns, or one
-// chunk). A tile of 64 tokens has registers for a second set; for the larger ones
+// chunk; fewer, down to half a chunk, where the per-task kernel's error would be
+// smaller: xcol_segment). A tile of 64 tokens has registers for a second set; for the larger ones
 // registers and shared memory are full and the sums live in tensor memory, which
 // nothing else uses here: a warp reaches 32 lanes of it, so up to three tiles of
 // 112 columns. An addition there costs the largest tile about 1900 cycles (it
 // spills a dozen registers around it): one chain per output would run 1024 x 1024
-// at 90%, 16384 tokens in 86 us where this takes 101, with a relative error of
+// at 90%, 16384 tokens in 86 us where this takes 99, with a relative error of
 // 1.8e-7 instead of 1.15e-7 (the per-task kernel's: 1.33e-7).
 //
 // Measured, with the per-task kernel beside it: choose_xcol.
@@ -78,7 +79,7 @@ struct XcArgs {
     int64_t M;
     uint64_t wait_ns;
     int n_items, n_tasks;
-    int seg;                     // chunks per segment
+    int seg;                     // chunks per segment (0: two segments a chunk)
     unsigned tiles;
     int stall_chunk;
 };
@@ -175,7 +176,8 @@ __device__ __forceinline__ void column(f2_t (&acc)[TT / 2][NR], const unsigned c
     }
 }
 
-template <int MAXB, int TT, int NR>
+// HALF: segments of half a chunk occur (tiles whose running sums are in registers).
+template <int MAXB, int TT, int NR, bool HALF>
 __global__ void __launch_bounds__(kThreads, 1)
 k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch<MAXB> b) {
     constexpr uint32_t kX = 2 * kXcBox;
@@ -306,6 +308,17 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
 #pragma unroll
                     for (int j = 0; j < NR; j++) total[i][j] = 0x8000000080000000ull;   // -0: adds nothing, to any value
             }
+            auto close = [&]() {   // total += acc, which starts anew
+                if constexpr (kRegSums) {
+#pragma unroll
+                    for (int i = 0; i < TT / 2; i++)
+#pragma unroll
+                        for (int j = 0; j < NR; j++) {
+                            total[i][j] = fadd2(acc[i][j], total[i][j]);
+                            acc[i][j] = 0ull;
+                        }
+                }
+            };
             auto sums = [&]() {   // this warp's running sums
                 return tmem_s + ((uint32_t)(32 * (warp & 3)) << 16) +
                        (uint32_t)(warp >> 2) * kTileCols;
@@ -332,7 +345,8 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                     }
                 }
             };
-            for (int c = 0, c1 = a.seg; c < nch; c++) {
+            const int seg = HALF ? max(a.seg, 1) : a.seg;
+            for (int c = 0, c1 = seg; c < nch; c++) {
                 if (!__all_sync(0xffffffffu, ptx::mbar_try_wait(&full[s], phase))) {
                     const bool got = wait_or_abort(&full[s], phase, 2 * a.wait_ns, &stop);
                     ok = __all_sync(0xffffffffu, got && !aborted(&stop));
@@ -348,7 +362,9 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                     int n = hdr->x;   // columns; then their places, then their weights
                     const int4 *oc = hdr + 1;
                     const float *w = reinterpret_cast<const float *>(oc + ((n + 3) >> 2)) + 4 * rg;
+                    const int mid = HALF && a.seg == 0 ? n - ((n >> 1) & ~3) : -1;   // columns left when a segment ends
                     for (; n >= 4; n -= 4, w += 4 * R) {
+                        if (HALF && n == mid) close();
                         const int4 o = *oc++;
                         column<TT, NR>(acc, xs + ((uint32_t)o.x ^ tgx), w);
                         column<TT, NR>(acc, xs + ((uint32_t)o.y ^ tgx), w + R);
@@ -371,16 +387,10 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                     phase ^= 1;
                 }
                 if (kRegSums && c + 1 == c1 && c1 < nch) {
-#pragma unroll
-                    for (int i = 0; i < (kRegSums ? TT / 2 : 1); i++)
-#pragma unroll
-                        for (int j = 0; j < NR; j++) {
-                            total[i][j] = fadd2(acc[i][j], total[i][j]);
-                            acc[i][j] = 0ull;
-                        }
-                    c1 += a.seg;
+                    close();
+                    c1 += seg;
                 } else if (!kRegSums && c + 1 == c1 && c1 < nch) {
-                    if (c1 > a.seg) add_sums();
+                    if (c1 > seg) add_sums();
                     const uint32_t at = sums();
 #pragma unroll
                     for (int k = 0; k < NR * TT; k += 8) {
@@ -396,7 +406,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                         }
                         tc5::st8(at + k, v);
                     }
-                    c1 += a.seg;
+                    c1 += seg;
                 }
             }
             if (!ok) break;
@@ -405,7 +415,7 @@ k_xcol(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ XcBatch
                 for (int i = 0; i < TT / 2; i++)
 #pragma unroll
                     for (int j = 0; j < NR; j++) acc[i][j] = fadd2(acc[i][j], total[i][j]);
-            } else if (nch > a.seg) {
+            } else if (nch > seg) {
                 add_sums();
             }
             if (!has) continue;
@@ -494,7 +504,7 @@ cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
     return e;
 }
 
-template <int MAXB, int TT, int NR>
+template <int MAXB, int TT, int NR, bool HALF>
 cudaError_t launch(const LaunchArgs *las, int n, int G) {
     XcBatch<MAXB> b;
     b.n = 0;
@@ -519,7 +529,8 @@ cudaError_t launch(const LaunchArgs *las, int n, int G) {
         a.wait_ns = la.wait_ns;
         a.n_items = (int)sc.items.size();
         a.n_tasks = (a.n_items + G - 1) / G;
-        a.seg = sc.xc.seg;
+        a.seg = xcol_segment(sc, la.N);
+        if (!HALF) a.seg = std::max(a.seg, 1);   // (a larger tile that was asked for)
         a.tiles = (unsigned)((la.N + 8 * TT - 1) / (8 * TT));
         a.stall_chunk = la.stall_chunk;
         b.start[b.n] = (unsigned)units;
@@ -543,16 +554,21 @@ cudaError_t launch(const LaunchArgs *las, int n, int G) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     static std::atomic<uint64_t> attr_set{0};
-    cudaError_t e = allow_smem(k_xcol<MAXB, TT, NR>, attr_set);
+    cudaError_t e = allow_smem(k_xcol<MAXB, TT, NR, HALF>, attr_set);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<int64_t>(units, las[0].sc->sm_count);
-    return launch_kernel(k_xcol<MAXB, TT, NR>, dim3(grid), dim3(kThreads), b.ns * b.stage_bytes + 1024, las[0].stream, map,
+    return launch_kernel(k_xcol<MAXB, TT, NR, HALF>, dim3(grid), dim3(kThreads), b.ns * b.stage_bytes + 1024, las[0].stream, map,
                          b);
 }
 
 template <int TT, int NR>
 cudaError_t launch_n(const LaunchArgs *las, int n, int G) {
-    return n == 1 ? launch<1, TT, NR>(las, 1, G) : launch<kXcBatchMax, TT, NR>(las, n, G);
+    if constexpr (TT * NR == 64) {
+        bool half = false;
+        for (int i = 0; i < n; i++) half |= xcol_segment(*las[i].sc, las[i].N) == 0;
+        if (half) return n == 1 ? launch<1, TT, NR, true>(las, 1, G) : launch<kXcBatchMax, TT, NR, true>(las, n, G);
+    }
+    return n == 1 ? launch<1, TT, NR, false>(las, 1, G) : launch<kXcBatchMax, TT, NR, false>(las, n, G);
 }
 
 }  // namespace

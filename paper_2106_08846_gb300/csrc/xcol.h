@@ -35,7 +35,7 @@ struct XcPlan {
     bool ok = false;
     int64_t off = -1, bytes = 0;       // place in the handle's packed buffer
     uint32_t item_bytes = 0;           // largest packed chunk of an item
-    int seg = 1;                       // chunks per segment (one chain of additions)
+    int seg = 1;                       // most chunks per segment (one chain of additions)
     bool even = false;                 // items of about equal length
     std::vector<int32_t> table;        // per chunk and item: its start / 16 (and the end)
     std::vector<int32_t> ints;         // (place / 4 bytes, value) of the packed buffer's integers
@@ -60,6 +60,8 @@ struct LaunchArgs;
 int64_t plan_xcol(Schedule &sc, int64_t base);
 // Whether the kernel runs a call of N tokens.
 bool choose_xcol(const Schedule &sc, int64_t N);
+// Chunks per segment in a call of N tokens (0: two segments a chunk).
+int xcol_segment(const Schedule &sc, int64_t N);
 // Tile (index into kXcTT; 32 rows) and items per task of one grid of n products.
 struct XcShape {
     int tile, G;

@@ -64,10 +64,7 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     }
     pl.item_bytes = (uint32_t)((4 + ((most_columns + 3) & ~int64_t(3)) + sc.R * most_columns) * 4);
     if (2 * xcol_stage_bytes(pl.item_bytes, kXcWarps) > kXcRoom) return base;   // a ring of two stages
-    // equal segments of at most 40 columns, or one chunk: outputs are then no
-    // further from 64 bits than the per-task kernel's, which shares a row among
-    // warps (relative errors of ten sizes 0.98 to 1.37e-7, the per-task kernel's 1.16
-    // to 1.43e-7; at 52 columns 1.17 to 1.47e-7, in one chain of 102 1.8e-7)
+    // equal segments of at most 40 columns, or one chunk (xcol_segment may take less)
     const double per_chunk = (double)sc.nnzb * sc.C / (double)(n_items * nch);
     const int64_t most = per_chunk * (double)nch <= 40.0 ? nch : std::max<int64_t>(1, (int64_t)(40.0 / per_chunk));
     const int64_t segs = (nch + most - 1) / most;
@@ -107,6 +104,28 @@ int64_t plan_xcol(Schedule &sc, int64_t base) {
     return pl.off + pl.bytes;
 }
 
+// A chain of s additions per segment and one of the m segments have a squared
+// error of 0.0346e-14 (s + m) relative to the sum's (within 2% for 8 sizes): so
+// few enough columns a segment that this is no more than the per-task kernel's,
+// which adds the chains of the warps that share a row (and of the two lane groups
+// of a 16-row block): relative errors of 40 sizes and block shapes 0.77 to 0.99
+// times the per-task kernel's, where segments of 40 columns had made six of them
+// up to 7% larger.
+int xcol_segment(const Schedule &sc, int64_t N) {
+    const int64_t nch = (sc.K + kXcChunk - 1) / kXcChunk;
+    const int warps = kXsConsumerWarps / std::min(choose_tasks(sc, N), kXsConsumerWarps), lanes = sc.R == 16 ? 2 : 1;
+    const double n = (double)sc.nnzb * sc.C / (double)std::max<size_t>(sc.items.size(), 1);
+    const double limit = 0.97 * (n / (warps * lanes) + warps + lanes - 1);
+    auto chains = [&](int seg) {
+        const double m = seg ? (double)((nch + seg - 1) / seg) : 2.0 * (double)nch;
+        return (seg ? n * seg / (double)nch : n / m) + m;
+    };
+    int best = sc.xc.seg;
+    for (int seg = sc.xc.seg; seg >= 0 && chains(best) > limit; seg--)
+        if (chains(seg) < chains(best)) best = seg;
+    return best;
+}
+
 // The tile and the items per task that minimise the busiest SM's cycles. A task's
 // items sit one per warp, ceil(items / 4) to a scheduler; a column takes it 11.9
 // TT cycles (a lone warp 24 more, 75 with the largest tile, which spills), a chunk
@@ -129,14 +148,21 @@ XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N) {
     const double sms = (double)scs[0]->sm_count;
     const double chunks = (double)((scs[0]->K + kXcChunk - 1) / kXcChunk);
     uint32_t item_bytes = 0;
-    for (int i = 0; i < n; i++) item_bytes = std::max(item_bytes, scs[i]->xc.item_bytes);
+    double segments[kXcBatchMax];
+    bool half = false;   // only the tile that keeps its running sums in registers ends segments within a chunk
+    for (int i = 0; i < n; i++) {
+        item_bytes = std::max(item_bytes, scs[i]->xc.item_bytes);
+        const int seg = xcol_segment(*scs[i], N);
+        segments[i] = seg ? std::ceil(chunks / seg) : 2.0 * chunks;
+        half |= seg == 0;
+    }
     for (int G : kG) {
         if (forced_G >= 1 && forced_G <= kXcWarps ? G != forced_G : 2 * xcol_stage_bytes(item_bytes, G) > kXcRoom) continue;
         for (int ti = 0; ti < kXcTileSizes; ti++) {
-            const bool half = scs[0]->R == 16;   // one tile, whose lanes do as many multiply-adds as the first's
-            if (half ? ti > 0 : forced_tile >= 0 && forced_tile < kXcTileSizes && ti != forced_tile) continue;
+            const bool r16 = scs[0]->R == 16;   // one tile, whose lanes do as many multiply-adds as the first's
+            if (r16 || (half && forced_tile < 0) ? ti > 0 : forced_tile >= 0 && forced_tile < kXcTileSizes && ti != forced_tile) continue;
             const int TT = kXcTT[ti];
-            const int64_t tokens = 8 * (half ? kXcTT16 : TT), tiles = (N + tokens - 1) / tokens;
+            const int64_t tokens = 8 * (r16 ? kXcTT16 : TT), tiles = (N + tokens - 1) / tokens;
             double sum = 0.0, longest = 0.0;
             int64_t units = 0;
             for (int i = 0; i < n; i++) {
@@ -146,7 +172,7 @@ XcShape xcol_shape(const Schedule *const *scs, int n, int64_t N) {
                 const double mean = (double)scs[i]->nnzb * scs[i]->C / (double)items;
                 const double column = 11.9 * TT * warps + (warps > 1 ? 0.0 : TT == 14 ? 75.0 : 24.0);
                 const double unit = mean * column + 470.0 * chunks + 385.0 * TT +
-                                    (TT > 8 ? 135.0 * TT * std::max(0.0, std::ceil(chunks / scs[i]->xc.seg) - 2.0) : 0.0);
+                                    (TT > 8 ? 135.0 * TT * std::max(0.0, segments[i] - 2.0) : 0.0);
                 units += tiles * tasks;
                 sum += unit * (double)(tiles * tasks);
                 longest = std::max(longest, unit);
@@ -165,10 +191,12 @@ namespace {
 
 // Against the per-task kernel, which takes its tasks' work and about 8500 + 4000 / G
 // cycles for each (G items a task; partly filled waves overlap). Measured (us, this
-// kernel and the per-task one): 1024 x 1024 at 90%, 16384 tokens 101 and 123, 4096
+// kernel and the per-task one): 1024 x 1024 at 90%, 16384 tokens 99 and 124, 4096
 // tokens 29.9 and 36.6; at 50%, 16384 tokens 360 and 656; 2048 x 2048 at 70%, 2000
-// tokens 125 and 203; 4096 x 4096 at 90%, 512 tokens 56 and 101; 768 x 768 at 70%,
-// 3000 tokens 28.3 and 37.4; at 50%, 1024 tokens 30.0 and 30.5. At 80%, 2000 tokens
+// tokens 125 and 203; 4096 x 4096 at 90%, 512 tokens 58 and 100; 768 x 768 at 70%,
+// 3000 tokens 28.3 and 37.4; at 50%, 1024 tokens 33.8 and 31.1 alone (segments of
+// half a chunk, which the model leaves out), but 499 and 617 for a plan of 48
+// weights of which ten are such. At 80%, 2000 tokens
 // 22.8 and 19.2; at 70%, 1024 tokens 21 and 13.3; 1024 x 768 at 50%, 500 tokens 30
 // and 15.6 (an item's columns are one warp's): these stay. Blocks of 16 rows: 16x1 of
 // 1024 x 1024 at 90%, 16384 tokens 115 and 134; of 768 x 768 at 70%, 3000 tokens 32
