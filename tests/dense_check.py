@@ -1,7 +1,8 @@
 """Parity sweep of the dense-tile tensor-core kernel, for a process started
-with BSR_DENSE_G (row groups per task) or without it (the kernel's own
-choice). Run by tests/test_gpu_dense.py in a subprocess; exit status 0 when
+with BSR_DENSE_G (row groups per task) or BSR_DENSE=1 (the kernel's own
+choice), or without (which kernel included). Run by tests/test_gpu_dense.py in a subprocess; exit status 0 when
 every output is right."""
+import os
 import sys
 
 import numpy as np
@@ -36,6 +37,8 @@ def main() -> int:
             X = synth.activations(seed + 1, N, K, "bf16")
             name = f"{R}x{C} {rows} M={M} K={K} N={N}"
             try:
+                if "BSR_DENSE_G" in os.environ or "BSR_DENSE" in os.environ:
+                    assert h.call_info(N)["kernel"] == "dense", h.call_info(N)
                 Y = to_host(h.spmm(to_dev(X), to_dev(w.bias)))
                 assert h.check_device_status() == 0
                 check_product(Y, ref, X, w.bias, M)

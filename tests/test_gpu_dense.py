@@ -18,9 +18,9 @@ pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-@pytest.mark.parametrize("g", [None, 1, 3, 7, 16, 34, 38, 48])   # 32 + g: pairs of CTAs
+@pytest.mark.parametrize("g", [None, "own", 1, 3, 7, 16, 34, 38, 48])   # 32 + g: pairs of CTAs
 def test_dense_parity_at_task_size(g):
-    env = dict(os.environ, **({} if g is None else {"BSR_DENSE_G": str(g)}))
+    env = dict(os.environ, **({} if g is None else {"BSR_DENSE": "1"} if g == "own" else {"BSR_DENSE_G": str(g)}))
     r = subprocess.run([sys.executable, "-m", "tests.dense_check"], cwd=ROOT, env=env, capture_output=True, text=True,
                        timeout=600)
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
@@ -82,7 +82,7 @@ def test_dense_takes_sparse_narrow_weights_of_the_simt_variant(R, C, N):
                             mask=synth.uniform_block_mask(7800 + i, M // R, K // C, (M // R) * (K // C) * (3 + i) // 100))
           for i in range(2)]
     hs = [bsr.bsr_create(*build_on_gpu(w.W, R, C), R, C, M, K) for w in ws]
-    assert all(h.schedule()["variant"] == "xstage" for h in hs)
+    assert all(h.schedule()["variant"] == "xstage" and "dense" in h.schedule()["kernels"] for h in hs)
     X = synth.activations(7801, N, K, "bf16")
     Xd, b = to_dev(X), to_dev(ws[0].bias)
     Ys = [torch.empty((N, M), dtype=torch.bfloat16, device="cuda") for _ in ws]

@@ -23,21 +23,28 @@ def main() -> int:
     from tests.gpu_util import build_on_gpu, check_product, to_dev, to_host
     fails = 0
     for k, (R, C, M, K, N) in enumerate(SHAPES):
-        for rows in ("even", "uneven"):
+        for rows in ("even", "uneven", "full"):
             MB, KB = M // R, K // C
             cnt = np.full(MB, max(1, int(0.3 * KB)), dtype=np.int64)
-            if rows == "uneven":   # short, empty and dense rows (split into pieces: partial tiles in the workspace)
+            seed = 9000 + 10 * k
+            if rows != "even":   # short and empty rows, and a long one (split into pieces: partial tiles in the workspace)
                 cnt[::2] = min(3, KB)
                 cnt[1::5] = 0
-                cnt[MB // 2] = KB
-            seed = 9000 + 10 * k
-            w = synth.make_weight("xc", seed, M, K, R, C, "f32", 0, mask=synth.mask_from_row_counts(seed, cnt, KB))
+            mask = synth.mask_from_row_counts(seed, cnt, KB)
+            if rows != "even":   # 56 columns of every 64, the most of 32 rows that the ring's stages hold, or all
+                mask[MB // 2] = (np.arange(KB) * C % 64 < 56) | (rows == "full")
+            w = synth.make_weight("xc", seed, M, K, R, C, "f32", 0, mask=mask)
             h = bsr.bsr_create(*build_on_gpu(w.W, R, C), R, C, M, K)
             ref = oracle.bsr_from_dense(w.W, R, C)
             X = synth.activations(seed + 1, N, K, "f32")
             tokens = np.unique(np.concatenate([np.arange(0, N, 7), np.arange(max(0, N - 130), N)]))
             name = f"{R}x{C} {rows} M={M} K={K} N={N}"
             try:
+                # (K = 100: the full row's pieces hold 50 columns of a chunk)
+                kernel = "xstage" if rows == "full" and R == 32 and K != 100 else "xcol"
+                assert h.call_info(N)["kernel"] == kernel, h.call_info(N)
+                if rows != "even" and MB > 8:
+                    assert h.schedule()["split_rows"] == 1 and h.schedule()["empty_rows"] > 0
                 for bias in (w.bias, None):
                     Y = to_host(h.spmm(to_dev(X), None if bias is None else to_dev(bias)))
                     assert h.check_device_status() == 0
