@@ -10,13 +10,14 @@
 //            kept block columns (ascending), and writes their values in block
 //            order from there (consecutive threads, consecutive addresses).
 //
-// HBM bounds large weights: W is read once per call, by 16-byte loads where W
-// and its rows are 16-byte aligned. Small ones are bounded by the two calls'
-// launches and synchronisations (about 75 us). A conversion (query and fill,
-// fp32, 4096 x 4096 at 90%, us; before: one thread per block, a flag per block
-// in memory, one CTA per row compacting through 64-bit divisions, scratch
-// mapped anew per call): 32x1 102 (197), 16x16 100 (156), 1x1 192 (892), 64x64
-// of 2048 x 4096 91 (1110), 8x1 of 768 x 768 75 (103).
+// A query reads W once (k_count), a fill twice (k_count, k_fill; the second
+// time from L2 where W fits it), by 16-byte loads where W and its rows are
+// 16-byte aligned; what bounds a conversion beside that are the two calls'
+// launches and synchronisations (about 65 us for a small weight). A conversion
+// (query and fill, fp32, 4096 x 4096 at 90%, us; before: one thread per block, a
+// flag per block in memory, one CTA per row compacting through 64-bit
+// divisions): 32x1 98 (195), 16x16 97 (159), 1x1 191 (896), 64x64 of 2048 x 4096
+// 82 (1110), 8x1 of 768 x 768 66 (102).
 #include <cuda_bf16.h>
 
 #include "bsr_internal.h"

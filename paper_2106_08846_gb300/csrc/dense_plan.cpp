@@ -136,13 +136,14 @@ namespace {
 // ones at 1024 and 3000 tokens (g = 3 to 8). The block-by-block kernel pays
 // about 300 cycles per unit of its own model (250 to 410 where measured):
 // against it the dense tiles won on every 50 to 95% sparse weight tried and on
-// 16x16 blocks of 1024 x 1024 at 99% (24 against 40 us at 16384 tokens), and
-// lost on 16x16 blocks of 4096 x 4096 at 97% (60 against 40 us at 2048
-// tokens: every chunk has a block of some row, and the dense tiles do 33
-// times the kept multiply-adds). Narrow blocks too sparse for the block-by-
+// 16x16 blocks of 1024 x 1024 at 99% (21 against 33 us at 16384 tokens). On 16x16
+// blocks of 4096 x 4096 at 97%, where every chunk has a block of some row and the
+// dense tiles do 33 times the kept multiply-adds, the two are close (us, dense and
+// block by block: 1000 tokens 21 and 26, 2048 46 and 62, 4096 94 and 94), and
+// the model keeps calls from 2048 tokens on block by block. Narrow blocks too sparse for the block-by-
 // block kernel have the per-task SIMT kernel beside this one, at about 0.85
 // cycles per unit of its model: 32x1 of 1024 x 1024 at 95%, 16384 tokens, 26.2
-// against 69 us.
+// against 68 us.
 int model_takes(const Schedule &sc, int64_t N) {
     const DensePlan &pl = sc.dense;
     int best = 1;

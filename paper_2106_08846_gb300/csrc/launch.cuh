@@ -2,7 +2,8 @@
 //
 // Every product kernel is launched with programmatic stream serialisation:
 // the kernel lets the next kernel of its stream be scheduled as soon as all
-// of its own CTAs are running (griddepcontrol.launch_dependents at entry),
+// of its own CTAs are running (griddepcontrol.launch_dependents at entry, or
+// right after the allocation of tensor memory),
 // and the next kernel runs its prologue -- barrier set-up, fetching the
 // handle's own schedule and block values -- on the SMs that free up, then
 // waits (griddepcontrol.wait) before it touches anything an earlier kernel

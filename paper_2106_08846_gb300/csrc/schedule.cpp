@@ -518,10 +518,10 @@ bsr_status_t build_schedule(Schedule &sc) {
         plan_xstage(sc);
     }
     if (sc.variant == V_XSTAGE && (int64_t)sc.xs_blob.size() > INT32_MAX) sc.variant = V_GENERIC;   // blob offsets are int32
-    // the dense-tile kernel (bf16), the column-list kernel
-    // (fp32 32x1 blocks) and
-    // the gathered-K kernel, after the variant's own packed values (the
-    // generic kernel's: a copy of the caller's block values)
+    // the dense-tile kernel (bf16), the column-list kernel (fp32 blocks of 16 or
+    // 32 rows and up to four columns) and the gathered-K kernel, where calls run
+    // them, after the variant's own packed values (the generic kernel's: a copy
+    // of the caller's block values)
     if (sc.variant == V_TC)
         plan_gk(sc, plan_dense(sc, sc.tc_w_total));
     else if (sc.variant == V_XSTAGE)

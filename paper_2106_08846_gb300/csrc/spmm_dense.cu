@@ -29,9 +29,9 @@
 // from registers.
 //
 // Measured (us, back to back, the block-by-block kernel in brackets): 1024 x
-// 1024 at 90%, 16384 tokens, 16x16 blocks 26.6 (43.1), 32x1 26.6 (64.1); 4096 x
-// 4096 at 95% with Zipf rows, 8192 tokens, 16x16 33.8 (161.5); 768 x 768 at 80%,
-// 1024 tokens, 32x1 5.3 (9.4); 1024 x 1024, 16 tokens 4.4 (6.8). One thread
+// 1024 at 90%, 16384 tokens, 16x16 blocks 26.4 (34.5), 32x1 26.5 (55.5); 4096 x
+// 4096 at 95% with Zipf rows, 8192 tokens, 16x16 33.2 (123.6); 768 x 768 at 80%,
+// 1024 tokens, 32x1 6.4 (8.4); 1024 x 1024, 16 tokens 5.2 (6.4). One thread
 // per role, in a branch that the compiler cannot see to be uniform, had put 424
 // cycles into a producer's step and 340 into four MMAs and a commit; whole
 // warps with one elected lane take 200 and 59, and the two loads of a stage
