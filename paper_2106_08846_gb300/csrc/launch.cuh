@@ -13,9 +13,14 @@
 // intact. BSR_PDL=0 in the environment turns it off (plain stream order).
 #pragma once
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+#include <cstdint>
 #include <cstdlib>
+#include <mutex>
 #include <utility>
 
 namespace bsr {
@@ -26,6 +31,36 @@ inline bool pdl_enabled() {
         return !(v && v[0] == '0');
     }();
     return on;
+}
+
+// cuTensorMapEncodeTiled (nullptr where the driver has none).
+inline PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+        else
+            cudaGetLastError();
+    });
+    return fn;
+}
+
+// Lets `kernel` take `bytes` of dynamic shared memory on the current device;
+// `done` keeps a bit per device that has it.
+template <typename K>
+cudaError_t allow_smem(K kernel, int bytes, std::atomic<uint64_t> &done) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const uint64_t bit = 1ull << (dev & 63);
+    if (done.load() & bit) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit);
+    return e;
 }
 
 // Launch `kernel` on `s` in clusters of `cluster` CTAs (1: no clusters).

@@ -60,12 +60,12 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "bsr_internal.h"
 #include "elem.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "status.cuh"
 #include "tcgen05.cuh"
 
 namespace bsr {
@@ -127,28 +127,6 @@ __device__ __forceinline__ Unit unit_at(const DnArgs &a, unsigned v) {
     return u;
 }
 
-__device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
-__device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
-
-// Bounded wait that also gives up when another role of the CTA stopped. The
-// limit begins anew while an epilogue warp of the CTA or its pair, for which
-// every role waits in the end, reports that it computes outputs again.
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, uint64_t limit_ns, const int *flag,
-                                              const int *beat) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    uint64_t t0 = ptx::globaltimer();
-    int seen = 0;
-    while (true) {
-        if (ptx::mbar_try_wait(bar, parity)) return true;
-        if (aborted(flag)) return false;
-        const uint64_t t = ptx::globaltimer();
-        if (t - t0 <= limit_ns) continue;
-        const int now = *reinterpret_cast<const volatile int *>(beat);
-        if (now == seen) return false;
-        seen = now;
-        t0 = t;
-    }
-}
 
 // Two values rounded to nearest even, the first in the low half.
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -670,25 +648,9 @@ __global__ void k_pack_dense(const uint16_t *__restrict__ data, const int32_t *_
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
 // A row-major bf16 matrix in boxes of `rows` x 64 columns, 128-byte swizzle.
 cudaError_t encode(const void *p, int64_t n_rows, int64_t n_cols, int rows, CUtensorMap *map) {
-    auto enc = encode_fn();
+    auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
     const cuuint64_t dims[2] = {(cuuint64_t)n_cols, (cuuint64_t)n_rows};
     const cuuint64_t strides[1] = {(cuuint64_t)n_cols * 2};
@@ -699,17 +661,6 @@ cudaError_t encode(const void *p, int64_t n_rows, int64_t n_cols, int rows, CUte
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
                ? cudaSuccess
                : cudaErrorInvalidValue;
-}
-
-template <typename K>
-cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (done.load() & bit) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDnMaxSmem - 1024);
-    if (e == cudaSuccess) done.fetch_or(bit);
-    return e;
 }
 
 template <int MAXB, bool PAIR>
@@ -765,7 +716,7 @@ cudaError_t launch(const LaunchArgs *las, const int *gs, int n) {
     b.ns = (int)std::min<uint32_t>(kDnStagesMax, (kDnMaxSmem - 1024 - fixed) / b.stage_bytes);
     CUtensorMap xmap;
     static std::atomic<uint64_t> attr_set{0};
-    cudaError_t e = allow_smem(k_dense<MAXB, PAIR>, attr_set);
+    cudaError_t e = allow_smem(k_dense<MAXB, PAIR>, kDnMaxSmem - 1024, attr_set);
     if (e == cudaSuccess) e = encode(las[0].X, las[0].N, las[0].sc->K, TN, &xmap);
     if (e != cudaSuccess) return e;
     const int64_t most = PAIR ? las[0].sc->sm_count / 2 : las[0].sc->sm_count;

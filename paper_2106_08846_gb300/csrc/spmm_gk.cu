@@ -57,13 +57,13 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "bsr_internal.h"
 #include "elem.cuh"
 #include "gk.h"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "status.cuh"
 #include "tcgen05.cuh"
 
 namespace bsr {
@@ -100,8 +100,6 @@ struct GkArgs {
     int stall_chunk;              // test hook: this chunk of each CTA's first unit is never loaded (-1: none)
 };
 
-__device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
-__device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
 __device__ __forceinline__ int pad4(int n) { return (n + 3) & ~3; }
 
 __device__ __forceinline__ float lds_f32(uint32_t a) {
@@ -628,25 +626,9 @@ __global__ void k_pack_gk(const T *__restrict__ data, const int32_t *__restrict_
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
 template <typename T>
 cudaError_t encode_x(const void *X, int64_t N, int64_t K, CUtensorMap *map) {
-    auto enc = encode_fn();
+    auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)N};
     const cuuint64_t strides[1] = {(cuuint64_t)K * sizeof(T)};
@@ -658,17 +640,6 @@ cudaError_t encode_x(const void *X, int64_t N, int64_t K, CUtensorMap *map) {
         CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     return cudaSuccess;
-}
-
-template <typename K>
-cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (done.load() & bit) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGkMaxSmem);
-    if (e == cudaSuccess) done.fetch_or(bit);
-    return e;
 }
 
 constexpr uint32_t kBarBytes = (2 * NS_MAX + 2 * NA_MAX + 2 + 4 + 1) * 8;
@@ -732,7 +703,7 @@ cudaError_t launch_r(const LaunchArgs &la, int G) {
     if (!smem || a.na < 2 || (uint32_t)(G * R) + (uint32_t)a.na * a.acols > (uint32_t)kGkTmemCols)
         return cudaErrorInvalidConfiguration;
     static std::atomic<uint64_t> attr_set{0};
-    cudaError_t e = allow_smem(k_gk<T, R>, attr_set);
+    cudaError_t e = allow_smem(k_gk<T, R>, kGkMaxSmem, attr_set);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     if ((e = encode_x<T>(la.X, la.N, sc.K, &map)) != cudaSuccess) return e;

@@ -50,12 +50,12 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdlib>
-#include <mutex>
 
 #include "bsr_internal.h"
 #include "elem.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "status.cuh"
 #include "tc.h"
 #include "tcgen05.cuh"
 
@@ -104,8 +104,6 @@ __device__ __forceinline__ float4 tf32_high(float4 v) {
                        __uint_as_float(__float_as_uint(v.z) & 0xffffe000u), __uint_as_float(__float_as_uint(v.w) & 0xffffe000u));
 }
 
-__device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
-__device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
 
 __device__ __forceinline__ int pad4(int n) { return (n + 3) & ~3; }
 
@@ -598,28 +596,12 @@ __global__ void k_reblock(const uint16_t *__restrict__ data, const int32_t *__re
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
 // Y [N, M] for the epilogue's TMA stores: boxes of 16 columns x 128 token rows,
 // with the swizzle of the row size (64 bytes fp32, 32 bytes bf16) in which
 // the epilogue stages them.
 template <typename T>
 cudaError_t encode_y(void *Y, int64_t N, int64_t M, CUtensorMap *map) {
-    auto enc = encode_fn();
+    auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
     const cuuint64_t dims[2] = {(cuuint64_t)M, (cuuint64_t)N};
     const cuuint64_t strides[1] = {(cuuint64_t)M * sizeof(T)};
@@ -689,20 +671,9 @@ cudaError_t make_tc_args(const LaunchArgs &la, int G, TcArgs &a, uint32_t &smem)
     return encode_y<T>(la.Y, la.N, sc.M, &a.ymap);
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (done.load() & bit) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);
-    if (e == cudaSuccess) done.fetch_or(bit);
-    return e;
-}
-
 template <typename T>
 cudaError_t encode_x(const void *X, int64_t N, int64_t K, CUtensorMap *map) {
-    auto enc = encode_fn();
+    auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)N};
     const cuuint64_t strides[1] = {(cuuint64_t)K * sizeof(T)};
@@ -728,7 +699,7 @@ cudaError_t launch_r(const LaunchArgs *las, const int *Gs, int n) {
         cudaError_t e = make_tc_args<T, R>(las[0], Gs[0], a, smem);
         if (e != cudaSuccess || smem == 0) return e;
         static std::atomic<uint64_t> attr_set{0};
-        if ((e = allow_smem(k_tc<T, R>, attr_set)) != cudaSuccess) return e;
+        if ((e = allow_smem(k_tc<T, R>, kTcMaxSmem, attr_set)) != cudaSuccess) return e;
         if ((e = encode_x<T>(las[0].X, las[0].N, las[0].sc->K, &map)) != cudaSuccess) return e;
         const int64_t grid = n_tiles * a.n_tasks;   // task-fastest order
         if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
@@ -753,7 +724,7 @@ cudaError_t launch_r(const LaunchArgs *las, const int *Gs, int n) {
     if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
     b.start[b.n] = (unsigned)grid;
     static std::atomic<uint64_t> attr_set_b{0};
-    cudaError_t e = allow_smem(k_tc_batch<T, R>, attr_set_b);
+    cudaError_t e = allow_smem(k_tc_batch<T, R>, kTcMaxSmem, attr_set_b);
     if (e != cudaSuccess) return e;
     if ((e = encode_x<T>(las[0].X, las[0].N, las[0].sc->K, &map)) != cudaSuccess) return e;
     return launch_kernel(k_tc_batch<T, R>, dim3((unsigned)grid), dim3(TcCfg<T>::NTHREADS), smem_max, las[0].stream, map, b);

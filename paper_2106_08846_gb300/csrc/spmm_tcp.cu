@@ -55,6 +55,7 @@
 #include "elem.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "status.cuh"
 #include "tc.h"
 #include "tcgen05.cuh"
 
@@ -106,8 +107,6 @@ struct TcpArgs {
                                         // loaded (-1: none)
 };
 
-__device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
-__device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
 __device__ __forceinline__ int pad4(int n) { return (n + 3) & ~3; }
 // The abort flag as the whole warp sees it (one value for every lane)
 __device__ __forceinline__ bool warp_aborted(const int *flag) { return __any_sync(0xffffffffu, aborted(flag)); }
@@ -559,17 +558,6 @@ k_tcp(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcpArgs 
     }
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (done.load() & bit) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);
-    if (e == cudaSuccess) done.fetch_or(bit);
-    return e;
-}
-
 constexpr uint32_t kBarBytes = (2 * NXMAX + 2 * NWMAX + 2 * NAMAX + 4 * 2 + 1) * 8;
 constexpr uint32_t kMinSmem = 118 * 1024;   // at least this much: one CTA per SM (each takes all tensor memory)
 
@@ -656,7 +644,7 @@ cudaError_t launch_r(const LaunchArgs &la, int G) {
             smem = layout(nx, Cfg::XBYTES, nw, a.wslot, ibytes, (uint32_t)sc.tc.stab_ints * 4u, G, R, &a);
     if (!smem) return cudaErrorInvalidConfiguration;
     static std::atomic<uint64_t> attr_set{0};
-    cudaError_t e = allow_smem(k_tcp<T, R>, attr_set);
+    cudaError_t e = allow_smem(k_tcp<T, R>, kTcMaxSmem, attr_set);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     if ((e = tc_encode_x(sc.dt, la.X, la.N, sc.K, &map)) != cudaSuccess) return e;

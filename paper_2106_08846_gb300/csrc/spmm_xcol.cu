@@ -51,11 +51,11 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "bsr_internal.h"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "status.cuh"
 #include "tcgen05.cuh"
 
 namespace bsr {
@@ -114,17 +114,6 @@ __device__ __forceinline__ f2_t fadd2(f2_t a, f2_t b) {
     f2_t d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
-}
-
-__device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
-__device__ __forceinline__ bool aborted(const int *flag) { return *reinterpret_cast<const volatile int *>(flag) != 0; }
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, uint64_t limit_ns, const int *flag) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = ptx::globaltimer();
-    while (true) {
-        if (ptx::mbar_try_wait(bar, parity)) return true;
-        if (aborted(flag) || ptx::globaltimer() - t0 > limit_ns) return false;
-    }
 }
 
 // The unit a CTA takes in its k-th turn (>= `units`: none). Several products come
@@ -477,33 +466,6 @@ __global__ void k_pack_xcol_ints(const int32_t *__restrict__ pairs, int64_t n, i
         out[pairs[2 * k]] = pairs[2 * k + 1];
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
-template <typename K>
-cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (done.load() & bit) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kXcMaxSmem - 1024);
-    if (e == cudaSuccess) done.fetch_or(bit);
-    return e;
-}
-
 template <int MAXB, int TT, int NR, bool HALF>
 cudaError_t launch(const LaunchArgs *las, int n, int G) {
     XcBatch<MAXB> b;
@@ -544,7 +506,7 @@ cudaError_t launch(const LaunchArgs *las, int n, int G) {
     b.stage_bytes = xcol_stage_bytes(item_bytes, G);
     b.ns = (int)std::min<uint32_t>(kXcStagesMax, kXcRoom / b.stage_bytes);
     if (b.ns < 1) return cudaErrorInvalidConfiguration;
-    auto enc = encode_fn();
+    auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)b.N}, strides[1] = {(cuuint64_t)K * 4};
@@ -554,7 +516,7 @@ cudaError_t launch(const LaunchArgs *las, int n, int G) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     static std::atomic<uint64_t> attr_set{0};
-    cudaError_t e = allow_smem(k_xcol<MAXB, TT, NR, HALF>, attr_set);
+    cudaError_t e = allow_smem(k_xcol<MAXB, TT, NR, HALF>, kXcMaxSmem - 1024, attr_set);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<int64_t>(units, las[0].sc->sm_count);
     return launch_kernel(k_xcol<MAXB, TT, NR, HALF>, dim3(grid), dim3(kThreads), b.ns * b.stage_bytes + 1024, las[0].stream, map,

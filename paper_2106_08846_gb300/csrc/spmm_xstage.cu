@@ -42,13 +42,13 @@
 
 #include <atomic>
 #include <cstdlib>
-#include <mutex>
 #include <vector>
 
 #include "bsr_internal.h"
 #include "elem.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "status.cuh"
 #include "xstage.h"
 
 namespace bsr {
@@ -223,11 +223,6 @@ __device__ __forceinline__ void load_wd(const float *wr, f2_t (&wd)[TR]) {
     }
 }
 
-__device__ __forceinline__ void set_status(int *status, int code) { atomicCAS(status, DEV_OK, code); }
-
-__device__ __forceinline__ bool aborted(const int *flag) {
-    return *reinterpret_cast<const volatile int *>(flag) != 0;
-}
 
 struct Shared {
     unsigned char *base;
@@ -748,22 +743,6 @@ __global__ void k_pack(const T *__restrict__ data, const Item *__restrict__ item
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
 // The ring, reused after the main loop for the warps' tile slots (one per
 // consumer warp, or one per item for one-row blocks, up to four per warp).
 size_t region_bytes(bsr_dtype_t dt, int R) {
@@ -813,7 +792,7 @@ cudaError_t make_args(const LaunchArgs &la, const XsPlan &pl, int G, XsArgs &a, 
 // The 2-D tensor map of X [N, K] for the ring's boxes (TN token rows each).
 template <typename T>
 cudaError_t encode_x(const void *X, int64_t N, int64_t K, CUtensorMap *map) {
-    auto enc = encode_fn();
+    auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
     const size_t es = sizeof(T);
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)N};
@@ -827,17 +806,6 @@ cudaError_t encode_x(const void *X, int64_t N, int64_t K, CUtensorMap *map) {
 }
 
 // Opt a kernel into the large dynamic shared memory once per device.
-template <typename K>
-cudaError_t allow_smem(K kernel, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = 1ull << (dev & 63);
-    if (done.load() & bit) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kXsMaxSmem);
-    if (e == cudaSuccess) done.fetch_or(bit);
-    return e;
-}
-
 // n products sharing X (same dtype, K, N, block shape and template); n == 1
 // is the plain launch, n > 1 one fused grid.
 template <typename T, int TR, int NRG, int CT, int RW, int NW>
@@ -851,7 +819,7 @@ cudaError_t launch_t(const LaunchArgs *las, const int *Gs, int n, const XsPlan *
         cudaError_t e = make_args<NW>(la, *pls[0], Gs[0], a, smem);
         if (e != cudaSuccess || smem == 0) return e;
         static std::atomic<uint64_t> attr_set{0};   // per instantiation, one bit per device
-        if ((e = allow_smem(k_xstage<T, TR, NRG, CT, RW, NW>, attr_set)) != cudaSuccess) return e;
+        if ((e = allow_smem(k_xstage<T, TR, NRG, CT, RW, NW>, kXsMaxSmem, attr_set)) != cudaSuccess) return e;
         const int64_t grid = n_tiles * a.n_tasks;   // task-major, tile-fastest
         if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
         CUtensorMap map;
@@ -878,7 +846,7 @@ cudaError_t launch_t(const LaunchArgs *las, const int *Gs, int n, const XsPlan *
     if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
     b.start[b.n] = (unsigned)grid;
     static std::atomic<uint64_t> attr_set_b{0};
-    cudaError_t e = allow_smem(k_xstage_batch<T, TR, NRG, CT, RW, NW>, attr_set_b);
+    cudaError_t e = allow_smem(k_xstage_batch<T, TR, NRG, CT, RW, NW>, kXsMaxSmem, attr_set_b);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     if ((e = encode_x<T>(las[0].X, las[0].N, las[0].sc->K, &map)) != cudaSuccess) return e;
