@@ -265,21 +265,25 @@ bsr_status_t bsr_from_dense(const void *W, int64_t M, int64_t K, int R, int C, f
         return BSR_ERR_ALLOC;
     }
     // where the GPU reaches the host's memory as it is (GB300's CPU link), the
-    // scan itself writes the count here: 4096 x 4096 fp32, 32x1, query and fill
-    // 98 us, with a copy of one word per call 114
-    volatile int32_t last = 0;
+    // scan itself writes the count there: 4096 x 4096 fp32, 32x1, query and fill
+    // 98 us, with a copy of one word per call 114. The word is the call's own, and
+    // left behind where a wait fails before the scan may have run.
+    int32_t last = 0;
     int device = 0, reaches = 0;
     if (cudaGetDevice(&device) != cudaSuccess ||
         cudaDeviceGetAttribute(&reaches, cudaDevAttrPageableMemoryAccess, device) != cudaSuccess) {
         cudaGetLastError();
         reaches = 0;
     }
-    int32_t *const word = const_cast<int32_t *>(&last);
-    if (launch_builder_count(W, dt, M, K, R, C, threshold, counts, indptr, reaches ? word : nullptr, s) != cudaSuccess ||
-        (!reaches && cudaMemcpyAsync(word, indptr + MB, sizeof *word, cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
+    int32_t *const word = reaches ? new (std::nothrow) int32_t(0) : nullptr;
+    if (launch_builder_count(W, dt, M, K, R, C, threshold, counts, indptr, word, s) != cudaSuccess ||
+        (!word && cudaMemcpyAsync(&last, indptr + MB, sizeof last, cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         cudaGetLastError();
         st = BSR_ERR_CUDA;
+    } else if (word) {
+        last = *const_cast<volatile int32_t *>(word);
+        delete word;
     }
     const int64_t nnzb = last;
     if (st == BSR_OK && last < 0) st = BSR_ERR_SHAPE;   // more than 2^31-1 kept blocks

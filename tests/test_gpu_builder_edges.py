@@ -2,6 +2,7 @@
 either direction, rows that are not 16-byte aligned, a misaligned W, one and
 many segments per block row, a partly filled last one; bit for bit against the
 oracle, NaN and threshold rule included."""
+import concurrent.futures
 import ctypes
 
 import numpy as np
@@ -56,3 +57,40 @@ def test_a_conversion_keeps_no_device_memory():
     torch.cuda.synchronize()
     assert cuda.cuMemPoolGetAttribute(pool, used_high, ctypes.byref(n)) == 0 and n.value > 0
     assert cuda.cuMemPoolGetAttribute(pool, used, ctypes.byref(n)) == 0 and n.value == 0
+
+
+def test_conversions_of_several_threads_and_under_capture():
+    """Each call reads its own count: eight threads on streams of their own; and
+    a call in a stream capture, whose wait fails, leaves later ones right."""
+    import paper_2106_08846_gb300 as bsr
+    lib = bsr.load()
+    Ws, refs = [], []
+    for k in range(8):
+        w = synth.make_weight("bt", 8900 + k, 256, 512, 8, 4, "f32", 10 * k)
+        Ws.append(to_dev(w.W))
+        refs.append(oracle.bsr_from_dense(w.W, 8, 4))
+    torch.cuda.synchronize()
+
+    def convert(k):
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            for _ in range(50):
+                out = bsr.bsr_from_dense(Ws[k], 8, 4, stream=s)
+        s.synchronize()
+        return out
+
+    def check():
+        with concurrent.futures.ThreadPoolExecutor(8) as ex:
+            for out, ref in zip(ex.map(convert, range(8)), refs):
+                assert_structure_equal(out, ref)
+
+    check()
+    indptr, s, graph = torch.empty(33, dtype=torch.int32, device="cuda"), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        graph.capture_begin()
+        status = lib.bsr_from_dense(Ws[0].data_ptr(), 256, 512, 8, 4, 0.0, 0, indptr.data_ptr(), None, None, 0, None,
+                                    s.cuda_stream)
+        with pytest.raises(RuntimeError):
+            graph.capture_end()
+    assert status != 0
+    check()
