@@ -298,7 +298,7 @@ bsr_status_t bsr_from_dense(const void *W, int64_t M, int64_t K, int R, int C, f
             st = BSR_ERR_CUDA;
         }
     }
-    cudaFreeAsync(counts, s);
+    if (cudaFreeAsync(counts, s) != cudaSuccess) cudaGetLastError();   // (not for the next call to find)
     return st;
 }
 

@@ -93,4 +93,5 @@ def test_conversions_of_several_threads_and_under_capture():
         with pytest.raises(RuntimeError):
             graph.capture_end()
     assert status != 0
+    assert_structure_equal(bsr.bsr_from_dense(Ws[0], 8, 4), refs[0])   # (this thread finds no error of that call)
     check()
