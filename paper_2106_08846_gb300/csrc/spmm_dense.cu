@@ -45,10 +45,10 @@
 // finite value; so every output whose accumulator is NaN is computed again,
 // without what is absent, by the epilogue warp that stored it, once the
 // accumulators are handed on. That takes far longer than the product: 1024 x
-// 1024 at 90%, 32x1, 16384 tokens 115 us with one such token, 295 us with every
-// 97th, 6.6 ms with a NaN in every token (27 us without; one lane walking each
-// output's blocks, with the accumulators held, had taken 5.1, 15 and 46 ms, and
-// at K = 8192 350 ms where it is now 20).
+// 1024 at 90%, 32x1, 16384 tokens 130 us with one such token, 330 us with every
+// 97th, 8.4 ms with a NaN in every token (39 us without, each call by itself;
+// one lane walking each output's blocks, with the accumulators held, had taken
+// 5.1, 15 and 46 ms, and at K = 8192 350 ms where it is now 23).
 //
 // Launched with programmatic stream serialisation: the barriers, tensor
 // memory and the first weight tiles come before the wait for the previous
@@ -156,28 +156,26 @@ __device__ __forceinline__ void kept_sums(float (&acc)[kDnGroup], const uint16_t
         fetch(v + step);
         if (col >= K) continue;
         const uint32_t xw[4] = {xq.x, xq.y, xq.z, xq.w};
-        float xf[8];   // finite activations, zero for the others
-        bool all = true;
+        float xf[8];
+        bool finite = true;
 #pragma unroll
         for (int e = 0; e < 8; e++) {
-            const uint32_t b = e & 1 ? xw[e / 2] & 0xffff0000u : xw[e / 2] << 16;
-            const bool fin = (b & 0x7f800000u) != 0x7f800000u;
-            all = all && fin;
-            xf[e] = fin ? __uint_as_float(b) : 0.f;
+            xf[e] = __uint_as_float(e & 1 ? xw[e / 2] & 0xffff0000u : xw[e / 2] << 16);
+            finite = finite && (__float_as_uint(xf[e]) & 0x7f800000u) != 0x7f800000u;
         }
+        if (finite) {   // (times -0 adds nothing)
 #pragma unroll
-        for (int r = 0; r < kDnGroup; r++) {
-            const uint4 wq = __ldg(reinterpret_cast<const uint4 *>(w + r * K + col));
-            const uint32_t ww[4] = {wq.x, wq.y, wq.z, wq.w};
+            for (int r = 0; r < kDnGroup; r++) {
+                const uint4 wq = __ldg(reinterpret_cast<const uint4 *>(w + r * K + col));
+                const uint32_t ww[4] = {wq.x, wq.y, wq.z, wq.w};
 #pragma unroll
-            for (int e = 0; e < 8; e++)
-                acc[r] = fmaf(xf[e], __uint_as_float(e & 1 ? ww[e / 2] & 0xffff0000u : ww[e / 2] << 16), acc[r]);
-        }
-        if (!all) {
+                for (int e = 0; e < 8; e++)
+                    acc[r] = fmaf(xf[e], __uint_as_float(e & 1 ? ww[e / 2] & 0xffff0000u : ww[e / 2] << 16), acc[r]);
+            }
+        } else {
 #pragma unroll 1
             for (int e = 0; e < 8; e++) {
                 const float xv = to_f32(__ldg(x + col + e));
-                if (fabsf(xv) <= 3.4e38f) continue;
 #pragma unroll
                 for (int r = 0; r < kDnGroup; r++) {
                     const uint16_t wv = __ldg(w + r * K + col + e);

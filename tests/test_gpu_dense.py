@@ -236,3 +236,35 @@ def test_dense_weights_without_elements(R, C, M, K):
                               ptrs(*(Y.data_ptr() for Y in Ys)), N, stream) == 0
     assert all(torch.equal(Y, want) for Y in Ys)
     assert all(h.check_device_status() == 0 for h in hs)
+
+
+@pytest.mark.parametrize("R,C", [(32, 1), (4, 4), (16, 16)])
+@pytest.mark.parametrize("every", [1, 16])
+def test_dense_infinities_in_the_weight_too(R, C, every):
+    """Infinities, NaN and zeros of both signs in kept elements, against X with
+    infinities, NaN and zeros in the same columns and in others: NaN and
+    infinite outputs where the oracle has them (tokens: all, or two of 32)."""
+    import paper_2106_08846_gb300 as bsr
+    M, K, N = 256, 320, 200
+    w = synth.make_weight("dw", 9600 + R, M, K, R, C, "bf16", 60)
+    W, rng = w.W.copy(), np.random.RandomState(5)
+    rows, cols = np.nonzero(W)
+    pick = rng.permutation(rows.size)[:24]
+    for k, at in enumerate(pick):
+        W[rows[at], cols[at]] = (0x7f80, 0xff80, 0x7fc0, 0x8000, 0x0000)[k % 5]
+    gpu, ref = build_on_gpu(W, R, C), oracle.bsr_from_dense(W, R, C)
+    h = bsr.bsr_create(*gpu, R, C, M, K)
+    assert h.call_info(N)["kernel"] == "dense"
+    X = synth.activations(9601, N, K, "bf16")
+    for t in range(0, N, every):
+        for k, c in enumerate([cols[pick[t % 24]], rng.randint(K)]):
+            X[t, c] = (0x7f80, 0xff80, 0x7fc1, 0x0000, 0x8000)[(t // every + k) % 5]
+    got = as_f64(to_host(h.spmm(to_dev(X), to_dev(w.bias))))
+    assert h.check_device_status() == 0
+    with np.errstate(invalid="ignore"):
+        want = oracle.bsr_spmm(*ref, X, w.bias, M)
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    inf = np.isinf(want)
+    assert inf.any() and np.array_equal(np.isinf(got), inf) and np.array_equal(got[inf], want[inf])
+    fin = np.isfinite(want)
+    assert np.allclose(got[fin], want[fin], rtol=2e-2, atol=2e-2)
